@@ -171,6 +171,22 @@ __device__ __forceinline__ float splat_power(const SplatRow &r, float dy) {
     return __fmaf_rn(__fmaf_rn(r.c2, dy, r.c1), dy, r.c0);
 }
 
+// 2^x. Results below the normal range flush to zero; the composited alphas
+// are compared with 1/255, so nothing downstream sees the difference, and the
+// instruction needs none of the scaling that keeps subnormal results.
+__device__ __forceinline__ float ex2_ftz(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+constexpr float kLog2e = 1.44269504088896341f;  // exp(x) = 2^(x log2 e)
+
+template <int N>
+struct IntC {  // a compile-time integer passed as an argument
+    static constexpr int value = N;
+};
+
 constexpr float kAlphaMin = 1.0f / 255.0f;
 constexpr float kAlphaMax = 0.99f;
 constexpr float kTMin = 1e-4f;

@@ -1,10 +1,10 @@
 // Tile rasteriser: front-to-back alpha compositing (Sec. 3.1, Eq. 2) and its
 // backward (Sec. 3.2.4), which skips the gradient work of frozen Gaussians.
 //
-// One CTA per screen tile, two pixels per thread. The tile's sorted splat
-// list is staged through shared memory in batches, so every thread reads
-// each splat as a shared-memory broadcast. No tensor
-// cores: the work is a per-pixel exponential and a handful of FMAs.
+// One CTA per screen tile; the tile's sorted splat list is staged through
+// shared memory, so every thread reads each splat as a shared-memory
+// broadcast. No tensor cores: the work is a per-pixel exponential and a
+// handful of FMAs.
 //
 // The backward walks each list back to front and recovers the transmittance
 // in front of every splat from the value the forward left over, so no
@@ -21,263 +21,489 @@ namespace gs {
 namespace {
 
 
-// A thread owns PPT pixels of its tile, (x, y + k TS/PPT) for k < PPT. Each
-// splat staged in shared memory is loaded once per PPT evaluations, and the
-// per-pixel update is written with selects instead of branches so the PPT
-// independent chains interleave.
+// ---- warps of a tile ----
+// A tile is cut into blocks of 8 x 4 PPT pixels, one per warp: lane l owns the
+// pixels (l % 8, l / 8 + 4 k), k < PPT, of its warp's block. Every warp walks
+// the tile's list by itself, 32 entries at a time, and keeps of them only the
+// splats that can reach its own block (block_hit); where the block is the
+// tile (8-pixel tiles, two pixels per thread) the list is already that
+// selection. So a tile of 16 or 32 pixels pays per 8-pixel block what 8-pixel
+// tiles pay, and no warp waits for another.
 //
-// With resume given, the walk also records where the backward may start:
-// resume_pos[tile] = 1 + the list position of the last unfrozen splat it
-// passed (0 if none), and per pixel resume = (T after that splat, the colour
-// blended behind it), so that the backward skips the frozen splats behind
-// every unfrozen one: they carry no gradient, and the state they would
-// rebuild is this one.
-template <int TS, int PPT, int B>
+// With an even number of pixels per thread the pixels go in pairs through the
+// packed FP32 instructions (f2_*); the code is written once over a value type
+// V (f32x2 or float) with the same rounded operations, so every shape gives
+// the same bits.
+__device__ __forceinline__ float v_sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ f32x2 v_sub(f32x2 a, f32x2 b) { return f2_sub(a, b); }
+__device__ __forceinline__ float v_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ f32x2 v_mul(f32x2 a, f32x2 b) { return f2_mul(a, b); }
+__device__ __forceinline__ float v_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ f32x2 v_fma(f32x2 a, f32x2 b, f32x2 c) { return f2_fma(a, b, c); }
+__device__ __forceinline__ void v_get(float v, float (&o)[1]) { o[0] = v; }
+__device__ __forceinline__ void v_get(f32x2 v, float (&o)[2]) { f2_unpack(v, o[0], o[1]); }
+__device__ __forceinline__ void v_set(float &v, const float (&o)[1]) { v = o[0]; }
+__device__ __forceinline__ void v_set(f32x2 &v, const float (&o)[2]) { v = f2_pack(o[0], o[1]); }
+template <class V>
+__device__ __forceinline__ V v_dup(float x);
+template <>
+__device__ __forceinline__ float v_dup<float>(float x) { return x; }
+template <>
+__device__ __forceinline__ f32x2 v_dup<f32x2>(float x) { return f2_pack(x, x); }
+
+template <int PPT>
+struct Lanes {
+    static constexpr int L = PPT % 2 == 0 ? 2 : 1;  // pixels per value
+    static constexpr int NP = PPT / L;              // values per thread
+};
+template <int L>
+struct ValueOf { typedef float T; };
+template <>
+struct ValueOf<2> { typedef f32x2 T; };
+
+template <class V>
+struct alignas(16) V4 {
+    V x, y, z, w;
+};
+
+constexpr int kStage = 32;  // list entries a warp stages at once, one per lane
+
+// The staged splats of one warp, every value duplicated into the halves of V:
+// a = (mean_x, mean_y, -conic_a / 2, -conic_b), b = (-conic_c / 2, opacity,
+// red, green) and blue -- the halves and signs formed once per splat instead
+// of once per thread (exact).
+template <class V>
+struct Stage {
+    V4<V> a[kStage], b[kStage];
+    V blue[kStage];
+    uint8_t pos[kStage];  // list position of each staged splat, from the first entry of the 32
+};
+
+struct SplatIn {  // what the rasteriser reads of a splat record
+    float4 xa, co;
+    float blue;
+};
+
+__device__ __forceinline__ SplatIn splat_in(const float *__restrict__ splats, uint32_t g) {
+    const float4 *r = reinterpret_cast<const float4 *>(splats + (int64_t)g * kSplat);
+    SplatIn s;
+    s.xa = __ldg(r);
+    s.co = __ldg(r + 1);
+    s.blue = __ldg(reinterpret_cast<const float *>(r + 2));
+    return s;
+}
+
+template <class V>
+__device__ __forceinline__ void stage_splat(Stage<V> &S, int q, const SplatIn &s) {
+    S.a[q] = V4<V>{v_dup<V>(s.xa.x), v_dup<V>(s.xa.y), v_dup<V>(__fmul_rn(-0.5f, s.xa.z)), v_dup<V>(-s.xa.w)};
+    S.b[q] = V4<V>{v_dup<V>(__fmul_rn(-0.5f, s.co.x)), v_dup<V>(s.co.y), v_dup<V>(s.co.z), v_dup<V>(s.co.w)};
+    S.blue[q] = v_dup<V>(s.blue);
+}
+
+// Whether the splat may blend at a pixel of the block [x0, x1] x [y0, y1]
+// (pixel centres). False only when alpha stays below 1/255 on the whole
+// block: q = d^T Q d exceeds tau + 2e-3 (1 + |tau|), tau = 2 ln(255 o),
+// everywhere on it. For a centre outside the block the least q lies on an
+// edge that faces the centre, at the clamped minimiser of that edge; both
+// facing edges are tried (any point of the block only lowers the least value
+// found). Rounding: with kappa = (a + |b| + c)(a + c) / det, this evaluation
+// and the compositing's own exponent are each off by at most 4 u kappa q
+// (u = 2^-24); up to kappa = 1e3 that is 5e-4 q together, inside the margin,
+// and conics beyond are never rejected. So the pixels' results do not depend
+// on this test.
+__device__ __forceinline__ bool block_hit(const SplatIn &s, float x0, float x1, float y0, float y1) {
+    const float mx = s.xa.x, my = s.xa.y, a = s.xa.z, b = s.xa.w, c = s.co.x;
+    const float det = a * c - b * b;
+    if (!(det > 0.f) || !(a > 0.f) || !(c > 0.f)) return true;
+    if (!((a + fabsf(b) + c) * (a + c) <= 1e3f * det)) return true;
+    const float tau = 2.f * __logf(255.f * s.co.y);
+    const float lim = tau + 2e-3f * (1.f + fabsf(tau));
+    const float dx = fminf(fmaxf(mx, x0), x1) - mx, dy = fminf(fmaxf(my, y0), y1) - my;
+    const float yy = fminf(fmaxf(my - __fdividef(b, c) * dx, y0), y1) - my;
+    const float xx = fminf(fmaxf(mx - __fdividef(b, a) * dy, x0), x1) - mx;
+    const float q1 = a * dx * dx + 2.f * b * dx * yy + c * yy * yy;
+    const float q2 = a * xx * xx + 2.f * b * xx * dy + c * dy * dy;
+    return !(fminf(q1, q2) > lim);
+}
+
+// Alpha of one splat at the L pixels of a value (0 where the splat is skipped:
+// positive exponent or alpha < 1/255), with splat_power's rounded operations.
+template <int L, class V>
+__device__ __forceinline__ void alphas(V px, V py, const V4<V> &a, const V4<V> &b, float (&al)[L], bool (&use)[L],
+                                       V &dy, float (&oG)[L]) {
+    const V dx = v_sub(a.x, px);
+    const V c0 = v_mul(a.z, v_mul(dx, dx)), c1 = v_mul(a.w, dx);
+    dy = v_sub(a.y, py);
+    const V pw = v_fma(v_fma(b.x, dy, c1), dy, c0);
+    float p[L], x[L], G[L];
+    v_get(pw, p);
+    v_get(v_mul(pw, v_dup<V>(kLog2e)), x);
+#pragma unroll
+    for (int l = 0; l < L; ++l) G[l] = ex2_ftz(x[l]);
+    V g;
+    v_set(g, G);
+    v_get(v_mul(b.y, g), oG);
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+        const float m = fminf(kAlphaMax, oG[l]);
+        use[l] = p[l] <= 0.f && m >= kAlphaMin;
+        al[l] = use[l] ? m : 0.f;
+    }
+}
+
+// The compositing forward of one tile. It is bound by instruction issue and by
+// the longest tile's chain of splats, not by memory.
+//
+// What a step does per pixel: two compares decide whether the splat blends,
+// a select zeroes alpha if not, and from there on nothing is conditional (an
+// alpha of 0 leaves T and the colour as they are, bit for bit). A pixel that
+// has stopped gets a NaN row coordinate, so that every later exponent is NaN
+// and fails its compare: no done flag is tested. G splats are evaluated
+// together -- their alphas do not depend on one another, only T runs through
+// them -- and the stop T < 1e-4 is tested once per G, on the last T (T never
+// grows): only a group that crosses it is gone through splat by splat.
+//
+// With RES, the walk also records where the backward may start: in every
+// batch of `batch` list entries, the state after its last unfrozen splat is
+// kept if some pixel of the tile is still alive when the walk gets there;
+// resume_pos[tile] = 1 + that splat's list position (0 if none), and per
+// pixel resume = (T after that splat, the colour blended behind it), so that
+// the backward skips the frozen splats behind it: they carry no gradient,
+// and the state they would rebuild is this one.
+//
+// Measured against the kernel before it (a barrier-separated batch per CTA,
+// done flags and a stop test per splat, every warp through the whole tile's
+// list): 1M Gaussians, 1237x822, 8-pixel tiles, two pixels per thread with the
+// record 202 -> 140 us; 3M at 1920x1080, 16-pixel tiles 633 -> 327 us; 400K
+// at 800x800, 16-pixel tiles with the record 240 -> 103 us; 2K at 128x128
+// 31 -> 15 us; the same bits in every output.
+template <int TS, int PPT, bool RES>
 __device__ __forceinline__ void render_tile(const float *__restrict__ splats, const uint32_t *__restrict__ vals,
                                             const uint32_t *__restrict__ ranges, const DevCam &cam,
                                             float *__restrict__ image, float *__restrict__ t_final,
-                                            int32_t *__restrict__ n_last, int tile,
+                                            int32_t *__restrict__ n_last, int tile, int batch = 0,
                                             const uint8_t *__restrict__ frozen = nullptr,
                                             float4 *__restrict__ resume = nullptr,
                                             int32_t *__restrict__ resume_pos = nullptr) {
-    constexpr int NT = TS * TS / PPT;  // threads; B = splats per staged batch
-    // With an even number of pixels per thread, the pixels go in pairs through
-    // the packed FP32 instructions (f2_*), and each splat is staged with every
-    // value duplicated into both halves of a 64-bit pair.
-    constexpr bool kPair = PPT % 2 == 0;
-    constexpr int NP = kPair ? PPT / 2 : 1;
-    __shared__ float4 s_xyab[kPair ? 1 : B];
-    __shared__ float4 s_cocg[kPair ? 1 : B];
-    __shared__ float s_blue[kPair ? 1 : B];
-    __shared__ ulonglong2 s_pk[kPair ? 4 * B : 1];  // (mx, my), (-a/2, -b), (-c/2, o), (r, g), each duplicated
-    __shared__ f32x2 s_pb[kPair ? B : 1];           // (blue, blue)
-    __shared__ int s_lu;  // the batch's last unfrozen splat (-1: none)
+    constexpr int L = Lanes<PPT>::L, NP = Lanes<PPT>::NP;
+    typedef typename ValueOf<L>::T V;
+    constexpr int kWarps = TS * TS / PPT / 32, kH = 4 * PPT;
+    constexpr bool kWholeTile = TS == 8 && kH == 8;  // the warp's block is the tile
+    constexpr int kG = 4;
+    // RES: the snapshot (T, colour) of every pixel waits in shared memory (in
+    // registers for 32-pixel tiles, whose staging takes most of it)
+    constexpr bool kSnapShared = RES && TS <= 16;
+    __shared__ Stage<V> s_stage[kWarps];
+    __shared__ float4 s_snap[kSnapShared ? TS * TS : 1];
     __shared__ int s_upos;
-    const int tx = tile % cam.tiles_x, ty = tile / cam.tiles_x;
-    const int px = tx * TS + (int)(threadIdx.x % TS);
-    const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1];
-    const float fpx = (float)px;
-    float fpy[PPT], T[PPT], c0[PPT], c1[PPT], c2[PPT];
-    int last[PPT], py[PPT];
-    bool done[PPT];
-    float uT[PPT], u0[PPT], u1[PPT], u2[PPT];  // T and colour after the last unfrozen splat passed
-    int upos = 0;
-#pragma unroll
-    for (int k = 0; k < PPT; ++k) {
-        py[k] = ty * TS + (int)(threadIdx.x / TS) + k * (TS / PPT);
-        fpy[k] = (float)py[k];
-        T[k] = 1.f;
-        c0[k] = c1[k] = c2[k] = 0.f;
-        last[k] = 0;
-        done[k] = !(px < cam.W && py[k] < cam.H);
-        uT[k] = 1.f;
-        u0[k] = u1[k] = u2[k] = 0.f;
-    }
-    // packed state of pixel pairs (2h, 2h + 1); the scalar arrays are brought up
-    // to date from it where they are read (the resume record and the end)
-    f32x2 T2[NP], r2[NP], g2[NP], b2[NP], fpy2[NP];
-    const f32x2 fpx2 = f2_pack(fpx, fpx), one2 = f2_pack(1.f, 1.f);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    Stage<V> &S = s_stage[warp];
+    const int bx = (tile % cam.tiles_x) * TS + (warp % (TS / 8)) * 8;
+    const int by = (tile / cam.tiles_x) * TS + (warp / (TS / 8)) * kH;
+    const int px = bx + (lane & 7), py0 = by + (lane >> 3);
+    const uint32_t start = ranges[2 * tile];
+    const int n = (int)(ranges[2 * tile + 1] - start);
+    const uint32_t *list = vals + start;
+    const float nan = __int_as_float(0x7fffffff);
+
+    const V fx = v_dup<V>((float)px), one = v_dup<V>(1.f);
+    V T[NP], r[NP], g[NP], b[NP];
+    float fy[PPT];  // row coordinate; NaN once the pixel is done (or outside the image)
+    int last[PPT], hit_last[PPT];
 #pragma unroll
     for (int h = 0; h < NP; ++h) {
-        T2[h] = one2;
-        r2[h] = g2[h] = b2[h] = f2_pack(0.f, 0.f);
-        fpy2[h] = kPair ? f2_pack(fpy[2 * h], fpy[(2 * h + 1) % PPT]) : 0ull;
+        T[h] = one;
+        r[h] = g[h] = b[h] = v_dup<V>(0.f);
     }
-    auto to_scalar = [&]() {
-        if constexpr (kPair) {
 #pragma unroll
-            for (int h = 0; h < NP; ++h) {
-                f2_unpack(T2[h], T[2 * h], T[2 * h + 1]);
-                f2_unpack(r2[h], c0[2 * h], c0[2 * h + 1]);
-                f2_unpack(g2[h], c1[2 * h], c1[2 * h + 1]);
-                f2_unpack(b2[h], c2[2 * h], c2[2 * h + 1]);
-            }
+    for (int k = 0; k < PPT; ++k) {
+        const int y = py0 + 4 * k;
+        fy[k] = px < cam.W && y < cam.H ? (float)y : nan;
+        last[k] = 0;
+        hit_last[k] = -1;
+    }
+    float4 u[PPT];  // RES: T and colour after the last unfrozen splat passed
+    int upos = 0, stop_at = -1, snap_at = -1;  // snap_at: the staged splat the snapshot is taken after
+    auto state = [&](float4 (&o)[PPT]) {
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+            float t_[L], r_[L], g_[L], b_[L];
+            v_get(T[h], t_); v_get(r[h], r_); v_get(g[h], g_); v_get(b[h], b_);
+#pragma unroll
+            for (int l = 0; l < L; ++l) o[L * h + l] = make_float4(t_[l], r_[l], g_[l], b_[l]);
         }
     };
-    if (resume) {  // a uniform branch
-        if (threadIdx.x == 0) s_upos = 0;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) s_lu = -1;  // ordered before the staging's atomics by the loop's first barrier
-    for (uint32_t base = start; base < end; base += B) {
-        bool all = true;
+    auto snapshot = [&]() {
+        state(u);
+        if (kSnapShared) {
 #pragma unroll
-        for (int k = 0; k < PPT; ++k) all = all && done[k];
-        if (__syncthreads_count(all) == NT) break;
-        for (int q = threadIdx.x; q < B; q += NT) {
-            if (base + q < end) {
-                // staged with -a/2 and -c/2 in place of a and c: the row coefficients of
-                // splat_row, rounded once here instead of once per thread
-                const uint32_t g = vals[base + q];
-                const float4 *r = reinterpret_cast<const float4 *>(splats + (int64_t)g * kSplat);
-                float4 xa = __ldg(r), co = __ldg(r + 1);
-                const float blue = __ldg(reinterpret_cast<const float *>(r + 2));
-                xa.z = __fmul_rn(-0.5f, xa.z);
-                co.x = __fmul_rn(-0.5f, co.x);
-                if constexpr (kPair) {
-                    s_pk[4 * q] = make_ulonglong2(f2_pack(xa.x, xa.x), f2_pack(xa.y, xa.y));
-                    s_pk[4 * q + 1] = make_ulonglong2(f2_pack(xa.z, xa.z), f2_pack(-xa.w, -xa.w));
-                    s_pk[4 * q + 2] = make_ulonglong2(f2_pack(co.x, co.x), f2_pack(co.y, co.y));
-                    s_pk[4 * q + 3] = make_ulonglong2(f2_pack(co.z, co.z), f2_pack(co.w, co.w));
-                    s_pb[q] = f2_pack(blue, blue);
-                } else {
-                    s_xyab[q] = xa;
-                    s_cocg[q] = co;
-                    s_blue[q] = blue;
-                }
-                if (resume && !(frozen && frozen[g])) atomicMax(&s_lu, q);
-            }
+            for (int k = 0; k < PPT; ++k) s_snap[k * (TS * TS / PPT) + threadIdx.x] = u[k];
         }
-        __syncthreads();
-        const int cnt = (int)min((uint32_t)B, end - base);
-        // One splat of the batch for this thread's pixels; false once they are all done.
-        auto blend = [&](int j) -> bool {
-            const float4 xa = s_xyab[j], co = s_cocg[j];
-            const float blue = s_blue[j];
-            const float dx = __fsub_rn(xa.x, fpx);
-            SplatRow row;  // splat_row's coefficients from the staged halves
-            row.c0 = __fmul_rn(xa.z, __fmul_rn(dx, dx));
-            row.c1 = __fmul_rn(-xa.w, dx);
-            row.c2 = co.x;
-            bool alive = false;
+    };
+    auto snapped = [&](int k) -> float4 { return kSnapShared ? s_snap[k * (TS * TS / PPT) + threadIdx.x] : u[k]; };
+    if (RES) snapshot();
+    auto all_done = [&]() {
+        bool d = true;
 #pragma unroll
-            for (int k = 0; k < PPT; ++k) {
-                const float dy = __fsub_rn(xa.y, fpy[k]);
-                const float power = splat_power(row, dy);
-                const float alpha = fminf(kAlphaMax, __fmul_rn(co.y, __expf(power)));
-                const float tn = __fmul_rn(T[k], __fsub_rn(1.f, alpha));
-                const bool use = !done[k] && power <= 0.f && alpha >= kAlphaMin;
-                const bool stop = use && tn < kTMin;
-                const bool add = use && !stop;
-                const float w = add ? alpha * T[k] : 0.f;
-                c0[k] += co.z * w;
-                c1[k] += co.w * w;
-                c2[k] += blue * w;
-                T[k] = add ? tn : T[k];
-                last[k] = add ? (int)(base - start) + j + 1 : last[k];
-                done[k] = done[k] || stop;
-                alive = alive || !done[k];
-            }
-            return alive;
-        };
-        // The same for a pair of pixels per packed instruction: every rounded
-        // operation is the scalar one's, so the results are bit for bit those of
-        // blend (the exponential stays scalar).
-        auto blend2 = [&](int j) -> bool {
-            const ulonglong2 q0 = s_pk[4 * j], q1 = s_pk[4 * j + 1], q2 = s_pk[4 * j + 2], q3 = s_pk[4 * j + 3];
-            const f32x2 qb = s_pb[j];
-            const f32x2 dx2 = f2_sub(q0.x, fpx2);
-            const f32x2 rc0 = f2_mul(q1.x, f2_mul(dx2, dx2)), rc1 = f2_mul(q1.y, dx2);
-            bool alive = false;
+        for (int k = 0; k < PPT; ++k) d = d && !(fy[k] == fy[k]);
+        return __all_sync(kFull, d) != 0;
+    };
+
+    // Staged splats j .. j + G - 1 for this thread's pixels; true once all
+    // pixels of the warp are done (stop_at: the staged splat that ended the last).
+    auto blend = [&](auto Gc, int j) -> bool {
+        constexpr int G = decltype(Gc)::value;
+        float al[G][NP][L];
+        int before[PPT];  // hit_last in front of this group
+#pragma unroll
+        for (int k = 0; k < PPT; ++k) before[k] = hit_last[k];
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            const V4<V> sa = S.a[j + i], sb = S.b[j + i];
 #pragma unroll
             for (int h = 0; h < NP; ++h) {
-                const int ka = 2 * h, kb = (2 * h + 1) % PPT;
-                const f32x2 dy2 = f2_sub(q0.y, fpy2[h]);
-                const f32x2 pw2 = f2_fma(f2_fma(q2.x, dy2, rc1), dy2, rc0);
-                float pa, pb;
-                f2_unpack(pw2, pa, pb);
-                float oa, ob;
-                f2_unpack(f2_mul(q2.y, f2_pack(__expf(pa), __expf(pb))), oa, ob);
-                const float aa = fminf(kAlphaMax, oa), ab = fminf(kAlphaMax, ob);
-                const f32x2 al2 = f2_pack(aa, ab);
-                float tna, tnb, ata, atb, Ta, Tb;
-                f2_unpack(f2_mul(T2[h], f2_sub(one2, al2)), tna, tnb);
-                f2_unpack(f2_mul(al2, T2[h]), ata, atb);
-                f2_unpack(T2[h], Ta, Tb);
-                const bool usea = !done[ka] && pa <= 0.f && aa >= kAlphaMin;
-                const bool useb = !done[kb] && pb <= 0.f && ab >= kAlphaMin;
-                const bool stopa = usea && tna < kTMin, stopb = useb && tnb < kTMin;
-                const bool adda = usea && !stopa, addb = useb && !stopb;
-                const f32x2 w2 = f2_pack(adda ? ata : 0.f, addb ? atb : 0.f);
-                r2[h] = f2_fma(q3.x, w2, r2[h]);
-                g2[h] = f2_fma(q3.y, w2, g2[h]);
-                b2[h] = f2_fma(qb, w2, b2[h]);
-                T2[h] = f2_pack(adda ? tna : Ta, addb ? tnb : Tb);
-                const int idx = (int)(base - start) + j + 1;
-                last[ka] = adda ? idx : last[ka];
-                last[kb] = addb ? idx : last[kb];
-                done[ka] = done[ka] || stopa;
-                done[kb] = done[kb] || stopb;
-                alive = alive || !done[ka] || !done[kb];
+                float y[L], oG[L];
+                bool use[L];
+                V py, dy;
+#pragma unroll
+                for (int l = 0; l < L; ++l) y[l] = fy[L * h + l];
+                v_set(py, y);
+                alphas<L, V>(fx, py, sa, sb, al[i][h], use, dy, oG);
+#pragma unroll
+                for (int l = 0; l < L; ++l) hit_last[L * h + l] = use[l] ? j + i : hit_last[L * h + l];
             }
-            return alive;
+        }
+        V t[G + 1][NP];
+        bool stop = false;
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+            t[0][h] = T[h];
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+                V a;
+                v_set(a, al[i][h]);
+                t[i + 1][h] = v_mul(t[i][h], v_sub(one, a));
+            }
+            float e[L];
+            v_get(t[G][h], e);
+#pragma unroll
+            for (int l = 0; l < L; ++l) stop = stop || e[l] < kTMin;
+        }
+        const bool any_stop = __any_sync(kFull, stop);
+        if (any_stop) {  // some ray ends in this group, before the splat that would take T below the floor
+            if (RES) stop_at = -1;
+#pragma unroll
+            for (int h = 0; h < NP; ++h) {
+                int at[L];
+#pragma unroll
+                for (int l = 0; l < L; ++l) at[l] = -1;
+#pragma unroll
+                for (int i = G - 1; i >= 0; --i) {
+                    float e[L];
+                    v_get(t[i + 1][h], e);
+#pragma unroll
+                    for (int l = 0; l < L; ++l) {
+                        at[l] = e[l] < kTMin ? j + i : at[l];
+                        al[i][h][l] = e[l] < kTMin ? 0.f : al[i][h][l];
+                    }
+                }
+#pragma unroll
+                for (int l = 0; l < L; ++l) {
+                    const int k = L * h + l;
+                    if (RES) stop_at = max(stop_at, at[l]);
+                    fy[k] = at[l] >= 0 ? nan : fy[k];
+                    hit_last[k] = before[k];
+                }
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+                    V a;
+                    v_set(a, al[i][h]);
+                    t[i + 1][h] = v_mul(t[i][h], v_sub(one, a));
+#pragma unroll
+                    for (int l = 0; l < L; ++l)
+                        hit_last[L * h + l] = al[i][h][l] > 0.f ? j + i : hit_last[L * h + l];
+                }
+            }
+        }
+        auto add = [&](int i) {
+            const V4<V> sb = S.b[j + i];
+            const V sblue = S.blue[j + i];
+#pragma unroll
+            for (int h = 0; h < NP; ++h) {
+                V a;
+                v_set(a, al[i][h]);
+                const V w = v_mul(a, t[i][h]);
+                r[h] = v_fma(sb.z, w, r[h]);
+                g[h] = v_fma(sb.w, w, g[h]);
+                b[h] = v_fma(sblue, w, b[h]);
+                T[h] = t[i + 1][h];
+            }
         };
-        auto step = [&](int jj) -> bool {
-            if constexpr (kPair) return blend2(jj);
-            else return blend(jj);
-        };
-        // with resume, the loop runs in two parts around the batch's last unfrozen
-        // splat, recording the state after it; no test per splat
-        const int lu = resume ? s_lu : -1;
+        if (RES && (unsigned)(snap_at - j) < (unsigned)G) {  // uniform
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+                add(i);
+                if (snap_at == j + i) snapshot();
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < G; ++i) add(i);
+        }
+        return any_stop && all_done();
+    };
+    auto walk = [&](int &j, int to) -> bool {
+        for (; j + kG <= to; j += kG)
+            if (blend(IntC<kG>(), j)) return true;
+        for (; j < to; ++j)
+            if (blend(IntC<1>(), j)) return true;
+        return false;
+    };
+
+    // The records (and freeze flags) of the next 32 entries are loaded while the
+    // current ones are blended, their indices one round earlier.
+    bool dead = all_done();
+    uint32_t g1 = 0;
+    SplatIn rec;
+    rec.xa = rec.co = make_float4(0.f, 0.f, 0.f, 0.f);
+    rec.blue = 0.f;
+    unsigned asleep = 0;  // the entry's freeze flag, as loaded (compared only when it is staged)
+    if (!dead) {
+        if (lane < n) {
+            const uint32_t g0 = list[lane];
+            rec = splat_in(splats, g0);
+            if (RES && frozen) asleep = frozen[g0];
+        }
+        if (lane + kStage < n) g1 = list[lane + kStage];
+    }
+    // RES: a snapshot is taken at the last unfrozen entry of every 32; when its
+    // batch has been walked to the end it is kept (written to the record), and
+    // when the walk ends inside a batch it counts only if it is the batch's
+    // last unfrozen entry, else the state kept before is the one.
+    int kept = 0, batch_end = batch;
+    auto keep = [&]() {
+        kept = upos;
+#pragma unroll
+        for (int k = 0; k < PPT; ++k) {
+            const int y = py0 + 4 * k;
+            if (px < cam.W && y < cam.H) resume[(int64_t)y * cam.W + px] = snapped(k);
+        }
+    };
+    for (int base = 0; base < n && !dead; base += kStage) {
+        if (RES && base == batch_end) {
+            if (upos != kept) keep();
+            batch_end += batch;
+        }
+        const bool valid = base + lane < n;
+        bool hit = valid;
+        if (!kWholeTile && valid)
+            hit = block_hit(rec, (float)bx, (float)(bx + 7), (float)by, (float)(by + kH - 1));
+        const unsigned hits = __ballot_sync(kFull, hit);
+        const unsigned wake = RES ? __ballot_sync(kFull, valid && asleep == 0) : 0u;
+        const int cnt = __popc(hits);
+        if (hit) {
+            const int q = kWholeTile ? lane : __popc(hits & ((1u << lane) - 1u));
+            stage_splat(S, q, rec);
+            if (!kWholeTile) S.pos[q] = (uint8_t)lane;
+        }
+        if (base + kStage + lane < n) {
+            rec = splat_in(splats, g1);
+            if (RES && frozen) asleep = frozen[g1];
+        }
+        if (base + 2 * kStage + lane < n) g1 = list[base + 2 * kStage + lane];
+        __syncwarp();
+        const int lu = 31 - __clz(wake);  // the last unfrozen of the 32
+        if (RES && wake) {
+            snap_at = __popc(hits & (kFull >> (31 - lu))) - 1;
+            if (snap_at < 0) snapshot();  // in front of the first staged splat
+        }
         int j = 0;
-        bool alive = true;
-        if (lu >= 0) {
-            for (; j <= lu && alive; ++j) alive = step(j);
-            if (alive || j == lu + 1) {  // reached the state after splat lu
-                to_scalar();
+        dead = walk(j, cnt);
+        bool cut = false;  // the walk ended in front of an unfrozen entry of its batch
+        if (RES && wake) {
+            snap_at = -1;
+            upos = base + lu + 1;
+            if (dead) {
+                const int e = __reduce_max_sync(kFull, stop_at);
+                cut = (kWholeTile ? e : (int)S.pos[e]) < lu;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < PPT; ++k) {
+            if (hit_last[k] >= 0) last[k] = base + 1 + (kWholeTile ? hit_last[k] : (int)S.pos[hit_last[k]]);
+            hit_last[k] = -1;
+        }
+        if (RES && dead && upos != kept) {
+            for (int q = base + kStage; q < min(n, batch_end) && !cut; q += kStage)
+                cut = __any_sync(kFull, q + lane < min(n, batch_end) && !(frozen && frozen[list[q + lane]]));
+            if (cut) {  // back to the state kept before
+                upos = kept;
 #pragma unroll
                 for (int k = 0; k < PPT; ++k) {
-                    uT[k] = T[k];
-                    u0[k] = c0[k];
-                    u1[k] = c1[k];
-                    u2[k] = c2[k];
+                    const int y = py0 + 4 * k;
+                    const bool in = kept > 0 && px < cam.W && y < cam.H;
+                    u[k] = in ? resume[(int64_t)y * cam.W + px] : make_float4(1.f, 0.f, 0.f, 0.f);
+                    if (kSnapShared) s_snap[k * (TS * TS / PPT) + threadIdx.x] = u[k];
                 }
-                upos = (int)(base - start) + lu + 1;
             }
         }
-        for (; j < cnt && alive; ++j) alive = step(j);
-        __syncthreads();
-        if (threadIdx.x == 0) s_lu = -1;  // read by every thread before the barrier above
+        __syncwarp();  // the staged splats are no longer read
     }
-    to_scalar();
-    if (resume) {
-        // A thread leaves the splat loop once its own pixels are done, so it may
-        // have stopped before the tile's last unfrozen splat: its pixels are then
-        // done at that position too, with their final T and nothing blended behind.
-        if (upos > 0) atomicMax(&s_upos, upos);
-        __syncthreads();
-        const int umax = s_upos;
-        if (upos < umax) {
-#pragma unroll
-            for (int k = 0; k < PPT; ++k) {
-                uT[k] = T[k];
-                u0[k] = c0[k];
-                u1[k] = c1[k];
-                u2[k] = c2[k];
-            }
+    if (RES) {
+        // A warp whose pixels were done before the splat the tile resumes behind
+        // has its final state there.
+        int umax = upos;
+        if (kWarps > 1) {
+            if (threadIdx.x == 0) s_upos = 0;
+            __syncthreads();
+            if (lane == 0 && upos > 0) atomicMax(&s_upos, upos);
+            __syncthreads();
+            umax = s_upos;
+            if (upos < umax) snapshot();
         }
-        upos = umax;
+        if (threadIdx.x == 0) resume_pos[tile] = umax;
     }
+    float4 f[PPT];
+    state(f);
     const int64_t HW = (int64_t)cam.W * cam.H;
 #pragma unroll
     for (int k = 0; k < PPT; ++k) {
-        if (px < cam.W && py[k] < cam.H) {
-            const int64_t pix = (int64_t)py[k] * cam.W + px;
-            image[pix] = c0[k] + T[k] * cam.bg[0];
-            image[HW + pix] = c1[k] + T[k] * cam.bg[1];
-            image[2 * HW + pix] = c2[k] + T[k] * cam.bg[2];
-            t_final[pix] = T[k];
+        const int y = py0 + 4 * k;
+        if (px < cam.W && y < cam.H) {
+            const int64_t pix = (int64_t)y * cam.W + px;
+            image[pix] = f[k].y + f[k].x * cam.bg[0];
+            image[HW + pix] = f[k].z + f[k].x * cam.bg[1];
+            image[2 * HW + pix] = f[k].w + f[k].x * cam.bg[2];
+            t_final[pix] = f[k].x;
             n_last[pix] = last[k];
-            if (resume)
-                resume[pix] = make_float4(uT[k], __fsub_rn(c0[k], u0[k]), __fsub_rn(c1[k], u1[k]),
-                                          __fsub_rn(c2[k], u2[k]));
+            if (RES) {
+                const float4 v = snapped(k);
+                resume[pix] = make_float4(v.x, __fsub_rn(f[k].y, v.y), __fsub_rn(f[k].z, v.z), __fsub_rn(f[k].w, v.w));
+            }
         }
     }
-    if (resume && threadIdx.x == 0) resume_pos[tile] = upos;
 }
 
-template <int TS, int PPT, int B>
-__global__ void __launch_bounds__(TS * TS / PPT) k_render_fwd(const float *__restrict__ splats,
-                                                              const uint32_t *__restrict__ vals,
-                                                              const uint32_t *__restrict__ ranges, DevCam cam,
-                                                              float *__restrict__ image, float *__restrict__ t_final,
-                                                              int32_t *__restrict__ n_last,
-                                                              const uint8_t *__restrict__ frozen,
-                                                              float4 *__restrict__ resume,
-                                                              int32_t *__restrict__ resume_pos) {
+// Blocks to keep resident per SM: with one pixel per thread 32 warps (24 when
+// the resume record is kept, whose state would spill), which cost registers
+// the step can spare (3M Gaussians at 1920x1080, 16-pixel tiles: 327 us
+// against 355 without; 400K at 800x800 with the record 103 against 119); with
+// two or four the G splats in flight need them (140 us against 144 at 1M,
+// 1237x822).
+template <int TS, int PPT, bool RES>
+constexpr int fwd_blocks() {
+    constexpr int warps = PPT == 1 ? (RES ? 24 : 32) : 1, per = TS * TS / PPT / 32;
+    return warps / per > 1 ? warps / per : 1;
+}
+
+template <int TS, int PPT, bool RES>
+__global__ void __launch_bounds__(TS * TS / PPT, fwd_blocks<TS, PPT, RES>())
+    k_render_fwd(const float *__restrict__ splats, const uint32_t *__restrict__ vals, const uint32_t *__restrict__ ranges,
+                 DevCam cam, float *__restrict__ image, float *__restrict__ t_final, int32_t *__restrict__ n_last,
+                 int batch, const uint8_t *__restrict__ frozen, float4 *__restrict__ resume,
+                 int32_t *__restrict__ resume_pos) {
     wait_prior_grid();
-    render_tile<TS, PPT, B>(splats, vals, ranges, cam, image, t_final, n_last, blockIdx.x, frozen, resume,
-                            resume_pos);
+    render_tile<TS, PPT, RES>(splats, vals, ranges, cam, image, t_final, n_last, blockIdx.x, batch, frozen, resume,
+                              resume_pos);
 }
 
 // Sum of nine per-lane values over a warp by recursive halving: at each of
@@ -634,7 +860,7 @@ __device__ __forceinline__ bool job_ok(const DevCam &cam, int W, int H, int TS) 
     return false;
 }
 
-template <int TS, int PPT, int B>
+template <int TS, int PPT>
 __global__ void __launch_bounds__(TS * TS / PPT) k_render_fwd_batch(const gs_raster_job *__restrict__ jobs,
                                                                     int W, int H, int tiles_per_job, int total,
                                                                     uint32_t *__restrict__ queue) {
@@ -643,7 +869,8 @@ __global__ void __launch_bounds__(TS * TS / PPT) k_render_fwd_batch(const gs_ras
         const gs_raster_job &j = jobs[item / tiles_per_job];
         const DevCam cam = make_cam(&j.cam);
         if (!job_ok(cam, W, H, TS)) continue;
-        render_tile<TS, PPT, B>(j.splats, j.vals, j.ranges, cam, j.image, j.t_final, j.n_last, item % tiles_per_job);
+        render_tile<TS, PPT, false>(j.splats, j.vals, j.ranges, cam, j.image, j.t_final, j.n_last,
+                                    item % tiles_per_job);
     }
 }
 
@@ -695,10 +922,16 @@ struct BwdArgs {
     const int32_t *resume_pos;
 };
 
-template <int TS, int PPT, int B>
-void launch(const FwdArgs &a, cudaStream_t s) {
-    launch_chained(k_render_fwd<TS, PPT, B>, a.cam.tiles_x * a.cam.tiles_y, TS * TS / PPT, s, a.splats, a.vals,
-                   a.ranges, a.cam, a.image, a.t_final, a.n_last, a.frozen, a.resume, a.resume_pos);
+template <int TS, int PPT, bool RES>
+void launch_fwd(int batch, const FwdArgs &a, cudaStream_t s) {
+    launch_chained(k_render_fwd<TS, PPT, RES>, a.cam.tiles_x * a.cam.tiles_y, TS * TS / PPT, s, a.splats, a.vals,
+                   a.ranges, a.cam, a.image, a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos);
+}
+
+template <int TS, int PPT>
+void by_batch(int batch, const FwdArgs &a, cudaStream_t s) {
+    if (a.resume) launch_fwd<TS, PPT, true>(batch, a, s);
+    else launch_fwd<TS, PPT, false>(batch, a, s);
 }
 
 template <int TS, int PPT, int B>
@@ -731,13 +964,13 @@ void launch(const BatchArgs &a, cudaStream_t s) {
         const int grid = resident_ctas(k_raster_bwd_batch<TS, PPT, B>, NT);
         k_raster_bwd_batch<TS, PPT, B><<<grid, NT, 0, s>>>(a.jobs, a.W, a.H, a.tiles_per_job, a.total, a.queue);
     } else {
-        const int grid = resident_ctas(k_render_fwd_batch<TS, PPT, B>, NT);
-        k_render_fwd_batch<TS, PPT, B><<<grid, NT, 0, s>>>(a.jobs, a.W, a.H, a.tiles_per_job, a.total, a.queue);
+        const int grid = resident_ctas(k_render_fwd_batch<TS, PPT>, NT);
+        k_render_fwd_batch<TS, PPT><<<grid, NT, 0, s>>>(a.jobs, a.W, a.H, a.tiles_per_job, a.total, a.queue);
     }
 }
 
 template <int TS, int PPT, class A>
-void by_batch(int batch, const A &a, cudaStream_t s) {
+void by_batch(int batch, const A &a, cudaStream_t s) {  // backward and batched launches
     switch (batch) {
         case 32: launch<TS, PPT, 32>(a, s); break;
         case 64: launch<TS, PPT, 64>(a, s); break;
