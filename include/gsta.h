@@ -167,7 +167,8 @@ int gs_render_fwd(const float *splats, const uint32_t *vals, const uint32_t *ran
  * camera's tile size. */
 typedef struct {
     int32_t pixels_per_thread; /* pixels each thread composites: 1, 2, or 4 (tiles of 16 and 32) */
-    int32_t batch;             /* splats staged per shared-memory batch: 32, 64, 128 or 256 */
+    int32_t batch;             /* list entries per batch: 32, 64, 128 or 256 (the resume record of
+                                * gs_render_fwd_resume keeps one state per batch) */
 } gs_raster_config;
 
 /* Sec. 3.1, Eq. 2: gs_render_fwd with an explicit launch shape (cfg may be

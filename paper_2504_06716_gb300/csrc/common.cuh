@@ -180,6 +180,14 @@ __device__ __forceinline__ float ex2_ftz(float x) {
     return r;
 }
 
+// 1 / x of an x in [0.01, 1] (within one unit in the last place, as the
+// division by it was; no scaling for extreme operands).
+__device__ __forceinline__ float rcp_ftz(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 constexpr float kLog2e = 1.44269504088896341f;  // exp(x) = 2^(x log2 e)
 
 template <int N>

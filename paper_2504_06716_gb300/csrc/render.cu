@@ -8,10 +8,9 @@
 //
 // The backward walks each list back to front and recovers the transmittance
 // in front of every splat from the value the forward left over, so no
-// per-pixel list is stored. A warp's 32 pixels see the same splat at the
-// same time; their nine gradient terms are summed with a recursive-halving
-// warp reduction, added once per warp into a shared accumulator, and the
-// accumulator goes to global memory with one atomic per value per tile.
+// per-pixel list is stored. A warp's pixels see the same splat at the same
+// time; its nine gradient terms are summed with a recursive-halving warp
+// reduction and added to the splat's row in global memory.
 #include "common.cuh"
 
 static_assert(sizeof(gs_camera) == 112, "gs_camera layout");
@@ -44,6 +43,12 @@ __device__ __forceinline__ void v_get(float v, float (&o)[1]) { o[0] = v; }
 __device__ __forceinline__ void v_get(f32x2 v, float (&o)[2]) { f2_unpack(v, o[0], o[1]); }
 __device__ __forceinline__ void v_set(float &v, const float (&o)[1]) { v = o[0]; }
 __device__ __forceinline__ void v_set(f32x2 &v, const float (&o)[2]) { v = f2_pack(o[0], o[1]); }
+__device__ __forceinline__ float v_lo(float v) { return v; }
+__device__ __forceinline__ float v_lo(f32x2 v) {
+    float a, b;
+    f2_unpack(v, a, b);
+    return a;
+}
 template <class V>
 __device__ __forceinline__ V v_dup(float x);
 template <>
@@ -130,7 +135,7 @@ __device__ __forceinline__ bool block_hit(const SplatIn &s, float x0, float x1, 
 // positive exponent or alpha < 1/255), with splat_power's rounded operations.
 template <int L, class V>
 __device__ __forceinline__ void alphas(V px, V py, const V4<V> &a, const V4<V> &b, float (&al)[L], bool (&use)[L],
-                                       V &dy, float (&oG)[L]) {
+                                       V &dy, float (&oG)[L]) {  // use: in, whether the pixel takes part
     const V dx = v_sub(a.x, px);
     const V c0 = v_mul(a.z, v_mul(dx, dx)), c1 = v_mul(a.w, dx);
     dy = v_sub(a.y, py);
@@ -146,7 +151,7 @@ __device__ __forceinline__ void alphas(V px, V py, const V4<V> &a, const V4<V> &
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         const float m = fminf(kAlphaMax, oG[l]);
-        use[l] = p[l] <= 0.f && m >= kAlphaMin;
+        use[l] = use[l] && p[l] <= 0.f && m >= kAlphaMin;
         al[l] = use[l] ? m : 0.f;
     }
 }
@@ -266,7 +271,10 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
                 bool use[L];
                 V py, dy;
 #pragma unroll
-                for (int l = 0; l < L; ++l) y[l] = fy[L * h + l];
+                for (int l = 0; l < L; ++l) {
+                    y[l] = fy[L * h + l];
+                    use[l] = true;
+                }
                 v_set(py, y);
                 alphas<L, V>(fx, py, sa, sb, al[i][h], use, dy, oG);
 #pragma unroll
@@ -506,71 +514,87 @@ __global__ void __launch_bounds__(TS * TS / PPT, fwd_blocks<TS, PPT, RES>())
                               resume_pos);
 }
 
-// Sum of nine per-lane values over a warp by recursive halving: at each of
-// the five xor levels a lane keeps half of its remaining slots and adds the
-// partner's copy of them (5 + 3 + 2 + 1 + 1 = 12 shuffles instead of 45).
-// On return, lane L holds the warp total of value kSlotOf[(L >> 1) & 15]
-// (-1: none); lanes L and L ^ 1 hold the same total.
-__device__ __constant__ int8_t kSlotOf[16] = {0, 1, 2, -1, 3, 4, -1, -1, 5, 6, 7, -1, 8, -1, -1, -1};
+// Sums over a warp by recursive halving: at each xor level a lane keeps half
+// of its remaining slots and adds the partner's copy of them.
+__device__ __forceinline__ float keep_half(bool upper, float lo, float hi, int mask) {
+    return (upper ? hi : lo) + __shfl_xor_sync(kFull, upper ? lo : hi, mask);
+}
 
-__device__ __forceinline__ float warp_sum9(const float (&g)[9], int lane) {
-    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4, h1 = lane & 2;
-    float r[5];
+// Which of the nine values lane l holds after sum9 (-1: none): the levels 8,
+// 4, 2 and 1 split them as {0-4 | 5-8}, {0-2 | 3-4} and {5-7 | 8}, ...
+__device__ __forceinline__ int slot_of(int lane) {
+    const int h3 = lane & 8, h2 = lane & 4, q = lane & 3;
+    if (q == 3) return -1;
+    if (!h2) return (h3 ? 5 : 0) + q;
+    if (h3) return q == 0 ? 8 : -1;
+    return q < 2 ? 3 + q : -1;
+}
+
+// What the totals of slot are multiplied by: rows of grad2d hold dL/d(mean,
+// conic, opacity, colour), and dpower/da = -dx^2 / 2 and so on.
+__device__ __forceinline__ float grad_scale(int slot) {
+    return slot == 2 || slot == 4 ? -0.5f : slot == 3 ? -1.f : 1.f;
+}
+
+// The nine values of each half-warp summed over its 16 lanes: lane l gets the
+// total of value slot_of(l).
+__device__ __forceinline__ float sum9_half(const float (&g)[9], int lane) {
+    const bool h3 = lane & 8, h2 = lane & 4, h1 = lane & 2, h0 = lane & 1;
+    float r[5], s[3];
 #pragma unroll
-    for (int j = 0; j < 5; ++j) {  // keep values 0-4 (lower half) or 5-8 (upper half)
-        const float lo = g[j], hi = j < 4 ? g[5 + j] : 0.f;
-        const float mine = h4 ? hi : lo, other = h4 ? lo : hi;
-        r[j] = mine + __shfl_xor_sync(kFull, other, 16);
-    }
-    float s[3];
+    for (int j = 0; j < 5; ++j) r[j] = keep_half(h3, g[j], j < 4 ? g[5 + j] : 0.f, 8);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {  // keep slots 0-2 or 3-4
-        const float lo = r[j], hi = j < 2 ? r[3 + j] : 0.f;
-        const float mine = h3 ? hi : lo, other = h3 ? lo : hi;
-        s[j] = mine + __shfl_xor_sync(kFull, other, 8);
-    }
-    float u[2];
+    for (int j = 0; j < 3; ++j) s[j] = keep_half(h2, r[j], j < 2 ? r[3 + j] : 0.f, 4);
+    const float u0 = keep_half(h1, s[0], s[2], 2), u1 = keep_half(h1, s[1], 0.f, 2);
+    return keep_half(h0, u0, u1, 1);
+}
+
+// Two splats' nine values at once: lanes 0-15 get the totals of a, lanes 16-31
+// those of b (20 shuffles for both; one splat alone takes 18).
+__device__ __forceinline__ float sum9_pair(const float (&a)[9], const float (&b)[9], int lane) {
+    const bool h4 = lane & 16;
+    float g[9];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {  // keep slots 0-1 or 2
-        const float lo = s[j], hi = j < 1 ? s[2 + j] : 0.f;
-        const float mine = h2 ? hi : lo, other = h2 ? lo : hi;
-        u[j] = mine + __shfl_xor_sync(kFull, other, 4);
-    }
-    float w = (h1 ? u[1] : u[0]) + __shfl_xor_sync(kFull, h1 ? u[0] : u[1], 2);
-    return w + __shfl_xor_sync(kFull, w, 1);
+    for (int j = 0; j < 9; ++j) g[j] = keep_half(h4, a[j], b[j], 16);
+    return sum9_half(g, lane);
+}
+
+// One splat's nine values: both half-warps get its totals.
+__device__ __forceinline__ float sum9_one(const float (&a)[9], int lane) {
+    float g[9];
+#pragma unroll
+    for (int j = 0; j < 9; ++j) g[j] = a[j] + __shfl_xor_sync(kFull, a[j], 16);
+    return sum9_half(g, lane);
 }
 
 // Backward state of one pixel: recovered transmittance T, dL/dC, and the
-// colour blended behind the current splat, kept only as G = dL/dC . sum over
-// the splats k behind it of c_k alpha_k T_k (all dL/dalpha needs): a splat
-// with alpha and T in front of it has dL/dalpha = T dL/dC . c - (G + T_final
-// dL/dC . bg) / (1 - alpha), and adds dL/dC . c alpha T to G.
+// colour blended behind the current splat with the background, kept only as
+// G = dL/dC . (sum over the splats k behind it of c_k alpha_k T_k + T_final bg)
+// (all dL/dalpha needs): a splat with alpha and T in front of it has dL/dalpha
+// = T dL/dC . c - G / (1 - alpha), and adds dL/dC . c alpha T to G.
 struct PixBwd {
-    float T, Tf, dC0, dC1, dC2, bgdot;
+    float T, dC0, dC1, dC2;
     float G;
     int nl;
 };
 
-// One (pixel, splat) step of the backward blend. The exponent's derivatives
-// with respect to the 2-D mean and conic are dx/dy polynomials; the thread's
-// pixels share dx, so only the dy moments of dL/dpower are summed here
-// (g[0] += dpow, g[1] += dy dpow, g[2] += dy^2 dpow) and geo_grads() turns
-// them into the five gradients once per splat. FRZ: the splat is frozen, so
-// only the pixel's state moves (a separate instantiation, so that a frozen
-// splat issues none of the gradient instructions).
-template <bool FRZ>
-__device__ __forceinline__ bool pix_bwd(PixBwd &p, int pos, const SplatRow &row, float dy, const float4 &co,
+// One (pixel, splat) step of the backward blend, skipped where the splat is not
+// blended. The exponent's derivatives with respect to the 2-D mean and conic
+// are dx/dy polynomials and the thread's pixels share dx, so the dy moments of
+// dL/dpower are summed (g[0] += dpow, g[1] += dy dpow, g[2] += dy^2 dpow), the
+// opacity's gradient in g[5], the colour's in g[6..8].
+__device__ __forceinline__ bool pix_bwd(PixBwd &p, bool frz, const SplatRow &row, float dy, const float4 &co,
                                         float blue, float (&g)[9]) {
     const float power = splat_power(row, dy);
-    const float G = __expf(power);
+    const float G = ex2_ftz(__fmul_rn(power, kLog2e));
     const float oG = __fmul_rn(co.y, G);
     const float alpha = fminf(kAlphaMax, oG);
-    if (!(pos < p.nl && power <= 0.f && alpha >= kAlphaMin)) return false;
-    const float om = 1.f - alpha;
-    p.T = __fdividef(p.T, om);  // transmittance in front of this splat
+    if (!(power <= 0.f && alpha >= kAlphaMin)) return false;
+    const float r = rcp_ftz(1.f - alpha);
+    p.T *= r;  // transmittance in front of this splat
     const float dcc = p.dC0 * co.z + p.dC1 * co.w + p.dC2 * blue;
-    if (!FRZ) {
-        const float dA = p.T * dcc - __fdividef(fmaf(p.Tf, p.bgdot, p.G), om);
+    if (!frz) {
+        const float dA = p.T * dcc - p.G * r;
         const float wT = alpha * p.T;
         g[6] += wT * p.dC0;
         g[7] += wT * p.dC1;
@@ -588,18 +612,6 @@ __device__ __forceinline__ bool pix_bwd(PixBwd &p, int pos, const SplatRow &row,
     return true;
 }
 
-// dy moments (s0, s1, s2) of dL/dpower -> gradients of the 2-D mean and
-// conic for power = -0.5 (a dx^2 + c dy^2) - b dx dy, dx = mean_x - px.
-__device__ __forceinline__ void geo_grads(float (&g)[9], float dx, float a, float b, float c) {
-    const float s0 = g[0], s1 = g[1], s2 = g[2];
-    const float xs0 = dx * s0;
-    g[0] = -(a * xs0 + b * s1);
-    g[1] = -(b * xs0 + c * s1);
-    g[2] = -0.5f * dx * xs0;
-    g[3] = -dx * s1;
-    g[4] = -0.5f * s2;
-}
-
 // The walk starts from the pixel's final state (T = T_final, nothing behind),
 // or, with resume, from the state the forward recorded after the tile's last
 // unfrozen splat (T there, and the colour blended behind it).
@@ -607,7 +619,6 @@ __device__ __forceinline__ void pix_load(PixBwd &p, bool inside, int64_t pix, in
                                          const int32_t *n_last, const float *dl, const float4 *resume,
                                          const DevCam &cam) {
     p.T = 1.f; p.dC0 = p.dC1 = p.dC2 = 0.f; p.nl = 0;
-    p.G = 0.f;
     if (inside) {
         p.T = t_final[pix];
         p.nl = n_last[pix];
@@ -615,16 +626,75 @@ __device__ __forceinline__ void pix_load(PixBwd &p, bool inside, int64_t pix, in
         p.dC1 = dl[HW + pix];
         p.dC2 = dl[2 * HW + pix];
     }
-    p.Tf = p.T;
-    p.bgdot = cam.bg[0] * p.dC0 + cam.bg[1] * p.dC1 + cam.bg[2] * p.dC2;
+    p.G = p.T * (cam.bg[0] * p.dC0 + cam.bg[1] * p.dC1 + cam.bg[2] * p.dC2);
     if (inside && resume) {
         const float4 r = resume[pix];
         p.T = r.x;
-        p.G = p.dC0 * r.y + p.dC1 * r.z + p.dC2 * r.w;
+        p.G += p.dC0 * r.y + p.dC1 * r.z + p.dC2 * r.w;
     }
 }
 
-template <int TS, int PPT, int B>
+// The staged splats of a warp, one (pixel, splat) step at a time: see
+// raster_bwd_tile. p[k].nl is the first staged splat of pixel k here. Not
+// inlined: it is rare, and its registers would be the packed path's too.
+template <int PPT, class V>
+__device__ __noinline__ void scalar_steps(PixBwd *p, const Stage<V> &S, const uint32_t *gid, int cnt, unsigned fz,
+                                          float fpx, float fpy0, float *grad2d) {
+    const int lane = threadIdx.x & 31, slot = slot_of(lane);
+    for (int j = 0; j < cnt; ++j) {
+        const float dx = __fsub_rn(v_lo(S.a[j].x), fpx), ha = v_lo(S.a[j].z), nb = v_lo(S.a[j].w), hc = v_lo(S.b[j].x);
+        SplatRow row;
+        row.c0 = __fmul_rn(ha, __fmul_rn(dx, dx));
+        row.c1 = __fmul_rn(nb, dx);
+        row.c2 = hc;
+        const float4 co = make_float4(hc, v_lo(S.b[j].y), v_lo(S.b[j].z), v_lo(S.b[j].w));
+        const bool frz = (fz >> j) & 1u;
+        float g[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        bool c = false;
+        for (int k = 0; k < PPT; ++k)
+            if (j >= p[k].nl)
+                c |= pix_bwd(p[k], frz, row, __fsub_rn(v_lo(S.a[j].y), fpy0 + (float)(4 * k)), co, v_lo(S.blue[j]), g);
+        if (!frz && __any_sync(kFull, c)) {
+            const float mx = dx * g[0];
+            const float e[9] = {fmaf(ha, mx + mx, nb * g[1]), fmaf(hc, g[1] + g[1], nb * mx), dx * mx, dx * g[1], g[2],
+                                g[5], g[6], g[7], g[8]};
+            const float tot = sum9_one(e, lane) * grad_scale(slot);
+            if (slot >= 0 && lane < 16 && tot != 0.f)
+                atomicAdd(grad2d + (int64_t)(gid[j] & 0x7fffffffu) * kG2d + slot, tot);
+        }
+    }
+}
+
+// The rasteriser backward of one tile: every warp walks its block's part of the
+// list back to front (32 entries at a time, those that can reach the block, as
+// in the forward), recovering T in front of each splat by a reciprocal of
+// 1 - alpha. It is bound by instruction issue and, where one tile's list is
+// much longer than the others', by that tile's chain of splats: two splats are
+// gone through together so that their latencies overlap.
+//
+// An unfrozen splat needs nine sums over the block: the moments s0 = sum of
+// dL/dpower, s1 and s2 (times dy and dy^2, formed per pixel), turned per lane
+// into the gradients of mean and conic; the opacity's, which is s0 / opacity
+// (dL/dpower = dL/dalpha alpha where alpha is not capped); the three of the
+// colour. Two unfrozen splats are summed over the warp together and added to
+// grad2d by the lanes that hold the totals, 18 adds to two rows in one
+// instruction: no shared accumulator, and per splat and block two sectors of
+// atomics instead of nine scattered words.
+//
+// A frozen splat only moves T and G, a uniform branch.
+//
+// In the packed steps a pixel that does not use a splat contributes terms
+// multiplied by alpha = 0, which is nothing only while they are finite: a
+// block whose pixel state is not finite, or 32 splats with a colour or
+// opacity that is not, go through the scalar steps (pix_bwd), which skip.
+//
+// Measured against the kernel before it (a barrier-separated batch per CTA,
+// scalar steps with divisions, one splat's sums at a time into a shared
+// accumulator by atomics): 1M Gaussians, 1237x822, 8-pixel tiles, two pixels
+// per thread, nothing frozen 492 -> 349 us, 95% frozen 220 -> 157 us (one
+// pixel per thread 208 -> 138 us); 400K at 800x800, 16-pixel tiles, half frozen
+// 445 -> 172 us; 2K at 128x128 114 -> 33 us.
+template <int TS, int PPT>
 __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats, const uint32_t *__restrict__ vals,
                                                 const uint32_t *__restrict__ ranges, const DevCam &cam,
                                                 const float *__restrict__ t_final, const int32_t *__restrict__ n_last,
@@ -632,117 +702,255 @@ __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats
                                                 float *__restrict__ grad2d, int tile,
                                                 const float4 *__restrict__ resume = nullptr,
                                                 const int32_t *__restrict__ resume_pos = nullptr) {
-    constexpr int NT = TS * TS / PPT;
-    __shared__ float4 s_xyab[B];
-    __shared__ float4 s_cocg[B];
-    __shared__ float s_blue[B];
-    __shared__ uint32_t s_gid[B];
-    __shared__ int s_frz[B];
-    __shared__ float s_acc[9][B];
-    __shared__ int s_maxlast;
-    const int tx = tile % cam.tiles_x, ty = tile / cam.tiles_x;
-    const int px = tx * TS + (int)(threadIdx.x % TS);
-    const uint32_t start = ranges[2 * tile];
-    const float fpx = (float)px;
+    constexpr int L = Lanes<PPT>::L, NP = Lanes<PPT>::NP;
+    typedef typename ValueOf<L>::T V;
+    constexpr int kWarps = TS * TS / PPT / 32, kH = 4 * PPT;
+    constexpr bool kWholeTile = TS == 8 && kH == 8;
+    __shared__ Stage<V> s_stage[kWarps];
+    __shared__ uint32_t s_gid[kWarps][kStage];  // Gaussian index, bit 31: frozen
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    Stage<V> &S = s_stage[warp];
+    uint32_t *gid = s_gid[warp];
+    const int bx = (tile % cam.tiles_x) * TS + (warp % (TS / 8)) * 8;
+    const int by = (tile / cam.tiles_x) * TS + (warp / (TS / 8)) * kH;
+    const int px = bx + (lane & 7), py0 = by + (lane >> 3);
+    const uint32_t *list = vals + ranges[2 * tile];
     const int64_t HW = (int64_t)cam.W * cam.H;
-    PixBwd p[PPT];
-    float fpy[PPT];
-    int nlmax = 0;
-#pragma unroll
-    for (int k = 0; k < PPT; ++k) {
-        const int py = ty * TS + (int)(threadIdx.x / TS) + k * (TS / PPT);
-        fpy[k] = (float)py;
-        pix_load(p[k], px < cam.W && py < cam.H, (int64_t)py * cam.W + px, HW, t_final, n_last, dl_dimage, resume,
-                 cam);
-        nlmax = max(nlmax, p[k].nl);
-    }
-    if (threadIdx.x == 0) s_maxlast = 0;
-    __syncthreads();
-    if (nlmax > 0) atomicMax(&s_maxlast, nlmax);
-    __syncthreads();
-    // with resume, the frozen splats behind the last unfrozen one are skipped
-    const uint32_t rend = start + (uint32_t)(resume ? min(s_maxlast, resume_pos[tile]) : s_maxlast);
-    const int lane = threadIdx.x & 31;
-    const int slot = kSlotOf[(lane >> 1) & 15];
-    const bool writer = slot >= 0 && !(lane & 1);
 
-    for (int64_t bend = rend; bend > (int64_t)start; bend -= B) {
-        const int64_t bstart = bend - B > (int64_t)start ? bend - B : (int64_t)start;
-        const int cnt = (int)(bend - bstart);
-        for (int q = threadIdx.x; q < B; q += NT) {
-            if (q < cnt) {
-                const uint32_t g = vals[bstart + q];
-                const float4 *r = reinterpret_cast<const float4 *>(splats + (int64_t)g * kSplat);
-                // -a/2 and -c/2 in place of a and c, as in the forward (exact halves;
-                // geo_grads gets a and c back by an exact doubling)
-                float4 xa = __ldg(r), co = __ldg(r + 1);
-                xa.z = __fmul_rn(-0.5f, xa.z);
-                co.x = __fmul_rn(-0.5f, co.x);
-                s_xyab[q] = xa;
-                s_cocg[q] = co;
-                s_blue[q] = __ldg(reinterpret_cast<const float *>(r + 2));
-                s_gid[q] = g;
-                s_frz[q] = frozen ? (int)frozen[g] : 0;
-            }
+    const float fpx = (float)px;
+    const V fx = v_dup<V>(fpx), one = v_dup<V>(1.f);
+    V T[NP], G[NP], d0[NP], d1[NP], d2[NP], fy[NP];  // G: dL/dC . (colour behind), background included
+    int nl[PPT], nlmax = 0;
+    bool finite = true;
 #pragma unroll
-            for (int k = 0; k < 9; ++k) s_acc[k][q] = 0.f;
+    for (int h = 0; h < NP; ++h) {
+        float T_[L], G_[L], a_[L], b_[L], c_[L], y_[L];
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            const int k = L * h + l, y = py0 + 4 * k;
+            PixBwd p;
+            pix_load(p, px < cam.W && y < cam.H, (int64_t)y * cam.W + px, HW, t_final, n_last, dl_dimage, resume, cam);
+            T_[l] = p.T; G_[l] = p.G; a_[l] = p.dC0; b_[l] = p.dC1; c_[l] = p.dC2;
+            y_[l] = (float)y;
+            nl[k] = p.nl;
+            nlmax = max(nlmax, p.nl);
+            finite = finite && isfinite(p.T) && isfinite(p.G) && isfinite(p.dC0) && isfinite(p.dC1) && isfinite(p.dC2);
         }
-        __syncthreads();
-        for (int j = cnt - 1; j >= 0; --j) {
-            const int pos = (int)(bstart - (int64_t)start) + j;  // position in the tile list
-            const float4 xa = s_xyab[j], co = s_cocg[j];
-            const float blue = s_blue[j];
-            const bool frz = s_frz[j] != 0;  // the same for every thread: a uniform branch
-            const float dx = __fsub_rn(xa.x, fpx);
-            SplatRow row;  // splat_row's coefficients from the staged halves
-            row.c0 = __fmul_rn(xa.z, __fmul_rn(dx, dx));
-            row.c1 = __fmul_rn(-xa.w, dx);
-            row.c2 = co.x;
-            float g[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (frz) {
-#pragma unroll
-                for (int k = 0; k < PPT; ++k) pix_bwd<true>(p[k], pos, row, __fsub_rn(xa.y, fpy[k]), co, blue, g);
-            } else {
-                bool c = false;
-#pragma unroll
-                for (int k = 0; k < PPT; ++k)
-                    c |= pix_bwd<false>(p[k], pos, row, __fsub_rn(xa.y, fpy[k]), co, blue, g);
-                if (__any_sync(kFull, c)) {
-                    geo_grads(g, dx, -2.f * xa.z, xa.w, -2.f * co.x);
-                    const float tot = warp_sum9(g, lane);
-                    if (writer) atomicAdd(&s_acc[slot][j], tot);
-                }
-            }
-        }
-        __syncthreads();
-        for (int q = threadIdx.x; q < cnt; q += NT) {
-            if (!s_frz[q]) {
-                float *dst = grad2d + (int64_t)s_gid[q] * kG2d;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const float v = s_acc[k][q];
-                    if (v != 0.f) atomicAdd(dst + k, v);
-                }
-            }
-        }
-        __syncthreads();
+        v_set(T[h], T_); v_set(G[h], G_); v_set(d0[h], a_); v_set(d1[h], b_); v_set(d2[h], c_); v_set(fy[h], y_);
     }
+    finite = __all_sync(kFull, finite);
+    int end = __reduce_max_sync(kFull, nlmax);
+    if (resume) end = min(end, resume_pos[tile]);  // the frozen splats behind the last unfrozen one are left out
+
+    const int slot = slot_of(lane);
+    const float scale = grad_scale(slot);
+    float pend[9];  // the sums of an unfrozen splat that waits for a second one
+    uint32_t pend_g = 0;
+    float pend_o = 1.f;
+    bool waiting = false;
+    auto give = [&](float tot, uint32_t g, float o, bool holds) {
+        const float v = slot == 5 ? __fdividef(tot, o) : tot * scale;
+        if (holds && v != 0.f) atomicAdd(grad2d + (int64_t)g * kG2d + slot, v);
+    };
+
+    // entries in reverse: lane l takes entry bend - 1 - l, so that staged splats
+    // 0, 1, ... go back to front
+    uint32_t g0 = 0, g1 = 0;
+    SplatIn rec;
+    rec.xa = rec.co = make_float4(0.f, 0.f, 0.f, 0.f);
+    rec.blue = 0.f;
+    unsigned asleep = 0;
+    if (lane < end) {
+        g0 = list[end - 1 - lane];
+        rec = splat_in(splats, g0);
+        if (frozen) asleep = frozen[g0];
+    }
+    if (lane + kStage < end) g1 = list[end - kStage - 1 - lane];
+    for (int bend = end; bend > 0; bend -= kStage) {
+        const bool valid = lane < bend;
+        bool hit = valid;
+        if (!kWholeTile && valid)
+            hit = block_hit(rec, (float)bx, (float)(bx + 7), (float)by, (float)(by + kH - 1));
+        const unsigned hits = __ballot_sync(kFull, hit);
+        const bool odd = hit && !(isfinite(rec.co.y) && isfinite(rec.co.z) && isfinite(rec.co.w) && isfinite(rec.blue));
+        const bool packed = finite && !__any_sync(kFull, odd);
+        const int cnt = __popc(hits);
+        if (hit) {
+            const int q = kWholeTile ? lane : __popc(hits & ((1u << lane) - 1u));
+            stage_splat(S, q, rec);
+            gid[q] = g0 | (asleep ? 0x80000000u : 0u);
+        }
+        if (lane < bend - kStage) {
+            g0 = g1;
+            rec = splat_in(splats, g0);
+            if (frozen) asleep = frozen[g0];
+        }
+        if (lane < bend - 2 * kStage) g1 = list[bend - 2 * kStage - 1 - lane];
+        __syncwarp();
+        // the first staged splat in front of each pixel's last contributor
+        int from[PPT];
+#pragma unroll
+        for (int k = 0; k < PPT; ++k) {
+            const int l0 = bend - nl[k];  // entries of lanes below it lie behind
+            from[k] = l0 <= 0 ? 0 : l0 >= 32 ? 32 : kWholeTile ? l0 : __popc(hits & ((1u << l0) - 1u));
+        }
+        const unsigned fz = __ballot_sync(kFull, lane < cnt && (gid[lane] >> 31));
+
+        // K splats from staged j on, K = 2 where there are two: their alphas do not
+        // depend on one another, T and G run through them; then the gradients of
+        // the unfrozen ones, a uniform branch.
+        auto steps = [&](auto Kc, int j) {
+            constexpr int K = decltype(Kc)::value;
+            float al[K][NP][L], oG[K][NP][L];
+            V dy[K][NP], Tk[K][NP], Gk[K][NP], rk[K][NP], dk[K][NP];
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                const V4<V> sa = S.a[j + i], sb = S.b[j + i];
+#pragma unroll
+                for (int h = 0; h < NP; ++h) {
+                    bool use[L];
+#pragma unroll
+                    for (int l = 0; l < L; ++l) use[l] = j + i >= from[L * h + l];
+                    alphas<L, V>(fx, fy[h], sa, sb, al[i][h], use, dy[i][h], oG[i][h]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                const V4<V> sb = S.b[j + i];
+                const V blue = S.blue[j + i];
+#pragma unroll
+                for (int h = 0; h < NP; ++h) {
+                    V a;
+                    v_set(a, al[i][h]);
+                    float om[L];
+                    v_get(v_sub(one, a), om);
+#pragma unroll
+                    for (int l = 0; l < L; ++l) om[l] = rcp_ftz(om[l]);
+                    v_set(rk[i][h], om);
+                    T[h] = v_mul(T[h], rk[i][h]);
+                    dk[i][h] = v_fma(d2[h], blue, v_fma(d1[h], sb.w, v_mul(d0[h], sb.z)));
+                    Tk[i][h] = T[h];
+                    Gk[i][h] = G[h];
+                    G[h] = v_fma(v_mul(dk[i][h], a), T[h], G[h]);
+                }
+            }
+            // the nine sums of splat i over this thread's pixels; false if none uses it
+            auto sums = [&](int i, float (&g)[9]) -> bool {
+                const V4<V> sa = S.a[j + i], sb = S.b[j + i];
+                auto total = [](V v) -> float {
+                    float e[L];
+                    v_get(v, e);
+                    return L == 2 ? e[0] + e[L - 1] : e[0];
+                };
+                bool any = false;
+                const bool capped = v_lo(sb.y) > kAlphaMax;  // uniform: only such a splat can be capped
+                float s0 = 0.f, s1 = 0.f, s2 = 0.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
+#pragma unroll
+                for (int h = 0; h < NP; ++h) {
+                    V w, ge;
+                    v_set(w, al[i][h]);
+                    w = v_mul(w, Tk[i][h]);
+                    float e[L];
+#pragma unroll
+                    for (int l = 0; l < L; ++l) {
+                        any = any || al[i][h][l] > 0.f;
+                        e[l] = al[i][h][l];
+                    }
+                    if (capped) {  // no gradient through the cap
+#pragma unroll
+                        for (int l = 0; l < L; ++l) e[l] = oG[i][h][l] > kAlphaMax ? 0.f : e[l];
+                    }
+                    v_set(ge, e);
+                    const V dA = v_sub(v_mul(Tk[i][h], dk[i][h]), v_mul(Gk[i][h], rk[i][h]));
+                    const V dp = v_mul(dA, ge), ydp = v_mul(dy[i][h], dp);
+                    s0 += total(dp);
+                    s1 += total(ydp);
+                    s2 += total(v_mul(dy[i][h], ydp));
+                    c0 += total(v_mul(w, d0[h]));
+                    c1 += total(v_mul(w, d1[h]));
+                    c2 += total(v_mul(w, d2[h]));
+                }
+                const float dx = __fsub_rn(v_lo(sa.x), fpx), mx = dx * s0;
+                // -(a mx + b s1), -(b mx + c s1) from the staged -a/2, -b, -c/2
+                g[0] = fmaf(v_lo(sa.z), mx + mx, v_lo(sa.w) * s1);
+                g[1] = fmaf(v_lo(sb.x), s1 + s1, v_lo(sa.w) * mx);
+                g[2] = dx * mx;
+                g[3] = dx * s1;
+                g[4] = s2; g[5] = s0; g[6] = c0; g[7] = c1; g[8] = c2;
+                return any;
+            };
+            const unsigned f = (fz >> j) & ((1u << K) - 1u);
+            if (f == (1u << K) - 1u) return;  // frozen
+            if (K == 2 && f == 0u) {
+                float g[9], g2[9];
+                bool any = sums(0, g);
+                any = sums(K - 1, g2) || any;
+                if (!__any_sync(kFull, any)) return;
+                const int i = lane < 16 ? j : j + K - 1;
+                give(sum9_pair(g, g2, lane), gid[i], v_lo(S.b[i].y), slot >= 0);
+                return;
+            }
+            float g[9];
+            const int i = K == 2 && f == 1u ? K - 1 : 0;  // the unfrozen one
+            const bool any = i ? sums(K - 1, g) : sums(0, g);
+            if (!__any_sync(kFull, any)) return;
+            if (waiting) {
+                give(sum9_pair(pend, g, lane), lane < 16 ? pend_g : gid[j + i], lane < 16 ? pend_o : v_lo(S.b[j + i].y),
+                     slot >= 0);
+            } else {
+#pragma unroll
+                for (int q = 0; q < 9; ++q) pend[q] = g[q];
+                pend_g = gid[j + i];
+                pend_o = v_lo(S.b[j + i].y);
+            }
+            waiting = !waiting;
+        };
+        if (packed) {
+            int j = 0;
+            for (; j + 2 <= cnt; j += 2) steps(IntC<2>(), j);
+            if (j < cnt) steps(IntC<1>(), j);
+        } else {
+            PixBwd p[PPT];
+#pragma unroll
+            for (int h = 0; h < NP; ++h) {
+                float e[5][L];
+                v_get(T[h], e[0]); v_get(G[h], e[1]); v_get(d0[h], e[2]); v_get(d1[h], e[3]); v_get(d2[h], e[4]);
+#pragma unroll
+                for (int l = 0; l < L; ++l)
+                    p[L * h + l] = PixBwd{e[0][l], e[2][l], e[3][l], e[4][l], e[1][l], from[L * h + l]};
+            }
+            scalar_steps<PPT, V>(p, S, gid, cnt, fz, fpx, (float)py0, grad2d);
+#pragma unroll
+            for (int h = 0; h < NP; ++h) {
+                float t_[L], g_[L];
+#pragma unroll
+                for (int l = 0; l < L; ++l) { t_[l] = p[L * h + l].T; g_[l] = p[L * h + l].G; }
+                v_set(T[h], t_); v_set(G[h], g_);
+            }
+        }
+        __syncwarp();  // the staged splats are no longer read
+    }
+    if (waiting) give(sum9_one(pend, lane), pend_g, pend_o, slot >= 0 && lane < 16);
 }
 
-template <int TS, int PPT, int B>
-__global__ void __launch_bounds__(TS * TS / PPT) k_raster_bwd(const float *__restrict__ splats,
-                                                              const uint32_t *__restrict__ vals,
-                                                              const uint32_t *__restrict__ ranges, DevCam cam,
-                                                              const float *__restrict__ t_final,
-                                                              const int32_t *__restrict__ n_last,
-                                                              const float *__restrict__ dl_dimage,
-                                                              const uint8_t *__restrict__ frozen,
-                                                              float *__restrict__ grad2d,
-                                                              const float4 *__restrict__ resume,
-                                                              const int32_t *__restrict__ resume_pos) {
+// Warps to keep resident per SM: 24 with one pixel per thread (78 registers), 16
+// with two (1M Gaussians, 1237x822, nothing frozen: 349 us against 362 without
+// the bound, which takes 132 registers and 12 warps, and 361 at 20 warps).
+template <int TS, int PPT>
+constexpr int bwd_blocks() {
+    constexpr int warps = PPT == 1 ? 24 : PPT == 2 ? 16 : 1, per = TS * TS / PPT / 32;
+    return warps / per > 1 ? warps / per : 1;
+}
+
+template <int TS, int PPT>
+__global__ void __launch_bounds__(TS * TS / PPT, bwd_blocks<TS, PPT>())
+    k_raster_bwd(const float *__restrict__ splats, const uint32_t *__restrict__ vals, const uint32_t *__restrict__ ranges,
+                 DevCam cam, const float *__restrict__ t_final, const int32_t *__restrict__ n_last,
+                 const float *__restrict__ dl_dimage, const uint8_t *__restrict__ frozen, float *__restrict__ grad2d,
+                 const float4 *__restrict__ resume, const int32_t *__restrict__ resume_pos) {
     wait_prior_grid();
-    raster_bwd_tile<TS, PPT, B>(splats, vals, ranges, cam, t_final, n_last, dl_dimage, frozen, grad2d, blockIdx.x,
-                                resume, resume_pos);
+    raster_bwd_tile<TS, PPT>(splats, vals, ranges, cam, t_final, n_last, dl_dimage, frozen, grad2d, blockIdx.x, resume,
+                             resume_pos);
 }
 
 // ---- measurement support: the (pixel, splat) pairs the backward visits ----
@@ -874,7 +1082,7 @@ __global__ void __launch_bounds__(TS * TS / PPT) k_render_fwd_batch(const gs_ras
     }
 }
 
-template <int TS, int PPT, int B>
+template <int TS, int PPT>
 __global__ void __launch_bounds__(TS * TS / PPT) k_raster_bwd_batch(const gs_raster_job *__restrict__ jobs,
                                                                     int W, int H, int tiles_per_job, int total,
                                                                     uint32_t *__restrict__ queue) {
@@ -883,17 +1091,22 @@ __global__ void __launch_bounds__(TS * TS / PPT) k_raster_bwd_batch(const gs_ras
         const gs_raster_job &j = jobs[item / tiles_per_job];
         const DevCam cam = make_cam(&j.cam);
         if (!job_ok(cam, W, H, TS)) continue;
-        raster_bwd_tile<TS, PPT, B>(j.splats, j.vals, j.ranges, cam, j.t_final, j.n_last, j.dl_dimage, j.frozen,
+        raster_bwd_tile<TS, PPT>(j.splats, j.vals, j.ranges, cam, j.t_final, j.n_last, j.dl_dimage, j.frozen,
                                     j.grad2d, item % tiles_per_job);
     }
 }
 
 // Launch shape used when the caller gives none: pixels per thread and batch
-// size of each kernel by tile size (timed on GB300; the autotuner may pick
-// another per workload).
-inline void default_config(int tile, bool bwd, int &ppt, int &batch) {
+// size by tile size (timed on GB300; the autotuner may pick another per
+// workload). The backward of 16-pixel tiles takes one pixel per thread while
+// the tiles are few: below about 2048 the chip has fewer 8 x 8 blocks than
+// warps it can hold, and halving the blocks shortens every chain (100K
+// Gaussians at 512x512, 1024 tiles: 74 us against 88; 50K at 320x240 58
+// against 76); above, two per thread cost fewer instructions (800x800, 2500
+// tiles: 172 against 174; 200K at 1237x822 132 against 154).
+inline void default_config(int tile, int64_t tiles, bool bwd, int &ppt, int &batch) {
     if (tile == 8) { ppt = 1; batch = 64; return; }
-    if (tile == 16) { ppt = bwd ? 2 : 1; batch = 256; return; }
+    if (tile == 16) { ppt = bwd && tiles >= 2048 ? 2 : 1; batch = 256; return; }
     ppt = 2;
     batch = 256;
 }
@@ -922,22 +1135,21 @@ struct BwdArgs {
     const int32_t *resume_pos;
 };
 
-template <int TS, int PPT, bool RES>
-void launch_fwd(int batch, const FwdArgs &a, cudaStream_t s) {
-    launch_chained(k_render_fwd<TS, PPT, RES>, a.cam.tiles_x * a.cam.tiles_y, TS * TS / PPT, s, a.splats, a.vals,
-                   a.ranges, a.cam, a.image, a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos);
+template <int TS, int PPT>
+void launch(int batch, const FwdArgs &a, cudaStream_t s) {
+    const int tiles = a.cam.tiles_x * a.cam.tiles_y;
+    if (a.resume)
+        launch_chained(k_render_fwd<TS, PPT, true>, tiles, TS * TS / PPT, s, a.splats, a.vals, a.ranges, a.cam, a.image,
+                       a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos);
+    else
+        launch_chained(k_render_fwd<TS, PPT, false>, tiles, TS * TS / PPT, s, a.splats, a.vals, a.ranges, a.cam,
+                       a.image, a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos);
 }
 
 template <int TS, int PPT>
-void by_batch(int batch, const FwdArgs &a, cudaStream_t s) {
-    if (a.resume) launch_fwd<TS, PPT, true>(batch, a, s);
-    else launch_fwd<TS, PPT, false>(batch, a, s);
-}
-
-template <int TS, int PPT, int B>
-void launch(const BwdArgs &a, cudaStream_t s) {
-    launch_chained(k_raster_bwd<TS, PPT, B>, a.cam.tiles_x * a.cam.tiles_y, TS * TS / PPT, s, a.splats, a.vals,
-                   a.ranges, a.cam, a.t_final, a.n_last, a.dl, a.frozen, a.grad2d, a.resume, a.resume_pos);
+void launch(int, const BwdArgs &a, cudaStream_t s) {
+    launch_chained(k_raster_bwd<TS, PPT>, a.cam.tiles_x * a.cam.tiles_y, TS * TS / PPT, s, a.splats, a.vals, a.ranges,
+                   a.cam, a.t_final, a.n_last, a.dl, a.frozen, a.grad2d, a.resume, a.resume_pos);
 }
 
 struct BatchArgs {
@@ -957,39 +1169,29 @@ int resident_ctas(K kernel, int threads) {
     return (sms > 0 ? sms : 152) * per_sm;
 }
 
-template <int TS, int PPT, int B>
-void launch(const BatchArgs &a, cudaStream_t s) {
+template <int TS, int PPT>
+void launch(int, const BatchArgs &a, cudaStream_t s) {
     constexpr int NT = TS * TS / PPT;
     if (a.bwd) {
-        const int grid = resident_ctas(k_raster_bwd_batch<TS, PPT, B>, NT);
-        k_raster_bwd_batch<TS, PPT, B><<<grid, NT, 0, s>>>(a.jobs, a.W, a.H, a.tiles_per_job, a.total, a.queue);
+        const int grid = resident_ctas(k_raster_bwd_batch<TS, PPT>, NT);
+        k_raster_bwd_batch<TS, PPT><<<grid, NT, 0, s>>>(a.jobs, a.W, a.H, a.tiles_per_job, a.total, a.queue);
     } else {
         const int grid = resident_ctas(k_render_fwd_batch<TS, PPT>, NT);
         k_render_fwd_batch<TS, PPT><<<grid, NT, 0, s>>>(a.jobs, a.W, a.H, a.tiles_per_job, a.total, a.queue);
     }
 }
 
-template <int TS, int PPT, class A>
-void by_batch(int batch, const A &a, cudaStream_t s) {  // backward and batched launches
-    switch (batch) {
-        case 32: launch<TS, PPT, 32>(a, s); break;
-        case 64: launch<TS, PPT, 64>(a, s); break;
-        case 128: launch<TS, PPT, 128>(a, s); break;
-        default: launch<TS, PPT, 256>(a, s); break;
-    }
-}
-
 template <class A>
 int dispatch(int tile, int ppt, int batch, const A &a, cudaStream_t s) {
     switch (tile * 10 + ppt) {
-        case 81: by_batch<8, 1>(batch, a, s); break;
-        case 82: by_batch<8, 2>(batch, a, s); break;
-        case 161: by_batch<16, 1>(batch, a, s); break;
-        case 162: by_batch<16, 2>(batch, a, s); break;
-        case 164: by_batch<16, 4>(batch, a, s); break;
-        case 321: by_batch<32, 1>(batch, a, s); break;
-        case 324: by_batch<32, 4>(batch, a, s); break;
-        default: by_batch<32, 2>(batch, a, s); break;
+        case 81: launch<8, 1>(batch, a, s); break;
+        case 82: launch<8, 2>(batch, a, s); break;
+        case 161: launch<16, 1>(batch, a, s); break;
+        case 162: launch<16, 2>(batch, a, s); break;
+        case 164: launch<16, 4>(batch, a, s); break;
+        case 321: launch<32, 1>(batch, a, s); break;
+        case 324: launch<32, 4>(batch, a, s); break;
+        default: launch<32, 2>(batch, a, s); break;
     }
     note_launches(1);
     return launch_status();
@@ -1018,7 +1220,7 @@ extern "C" int gs_render_fwd_resume(const float *splats, const uint32_t *vals, c
     FwdArgs a{splats, vals, ranges, make_cam(cam), image, t_final, n_last, frozen, reinterpret_cast<float4 *>(resume),
               resume_pos};
     int ppt, batch;
-    default_config(a.cam.tile, false, ppt, batch);
+    default_config(a.cam.tile, (int64_t)a.cam.tiles_x * a.cam.tiles_y, false, ppt, batch);
     if (cfg) { ppt = cfg->pixels_per_thread; batch = cfg->batch; }
     return dispatch(a.cam.tile, ppt, batch, a, as_stream(stream));
 }
@@ -1047,7 +1249,7 @@ extern "C" int gs_raster_bwd_resume(const float *splats, const uint32_t *vals, c
     BwdArgs a{splats, vals, ranges, make_cam(cam), t_final, n_last, dl_dimage, frozen, grad2d,
               reinterpret_cast<const float4 *>(resume), resume_pos};
     int ppt, batch;
-    default_config(a.cam.tile, true, ppt, batch);
+    default_config(a.cam.tile, (int64_t)a.cam.tiles_x * a.cam.tiles_y, true, ppt, batch);
     if (cfg) { ppt = cfg->pixels_per_thread; batch = cfg->batch; }
     return dispatch(a.cam.tile, ppt, batch, a, as_stream(stream));
 }
@@ -1078,7 +1280,7 @@ static int batch_common(const gs_raster_job *jobs_dev, int32_t n_jobs, int32_t w
     if (cudaMemsetAsync(queue_dev, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
     BatchArgs a{jobs_dev, width, height, (int)tiles, (int)(tiles * n_jobs), queue_dev, bwd};
     int ppt, batch;
-    default_config(tile, bwd, ppt, batch);
+    default_config(tile, tiles * n_jobs, bwd, ppt, batch);
     if (cfg) { ppt = cfg->pixels_per_thread; batch = cfg->batch; }
     return dispatch(tile, ppt, batch, a, s);
 }

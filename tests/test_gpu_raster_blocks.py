@@ -117,3 +117,40 @@ def test_one_tile_against_float64(tile, ppt, n, thin):
             assert (got[:, cols] - grad[:, cols]).abs().max() <= 1e-3 * max(float(grad[:, cols].abs().max()), 1e-6), cols
     assert not g2[:, 9:].any() and not got[frozen[:n] != 0].any()
     assert lib.gs_get_device_error() == 0
+
+
+@pytest.mark.parametrize("tile,ppt", [(8, 1), (8, 2), (16, 2), (16, 4), (32, 1)])
+def test_a_pixel_without_a_finite_gradient_stays_by_itself(tile, ppt):
+    """NaN in dL/dC of one pixel reaches the splats blended there and no others
+    (those: equal to the gradient without that pixel, up to float32 rounding
+    of the scalar steps against the packed ones, 1e-5 of the largest value)."""
+    n, W, H = 70, tile, tile
+    cam = lib.camera(synth.pinhole(W, H, 60.0, (0, 0, -4.0), up=(0, 1, 0)), tile=tile)
+    spl = _splats(n, tile, tile + ppt, False)
+    dl = torch.randn((3, H, W), generator=torch.Generator().manual_seed(ppt))
+    y, x = H // 2, W // 3
+    with torch.no_grad():
+        dx, dy = spl[:n, 0].double() - x, spl[:n, 1].double() - y
+        power = -0.5 * (spl[:n, 2] * dx * dx + spl[:n, 4] * dy * dy) - spl[:n, 3] * dx * dy
+        al = torch.clamp(spl[:n, 5] * torch.exp(power), max=0.99)
+    d = lambda t: t.to(DEV).contiguous()  # noqa: E731
+    vals = torch.arange(n, dtype=torch.int32, device=DEV)
+    ranges = torch.tensor([[0, n]], dtype=torch.int32, device=DEV)
+    cfg = lib.raster_config(ppt, 64)
+    img, tf = torch.zeros((3, H, W), device=DEV), torch.zeros((H, W), device=DEV)
+    nl = torch.zeros((H, W), dtype=torch.int32, device=DEV)
+    lib.gs_render_fwd_cfg(d(spl), vals, ranges, cam, cfg, img, tf, nl)
+    got = []
+    for v in (0.0, float("nan")):
+        e = dl.clone()
+        e[:, y, x] = v
+        g2 = torch.zeros((n, 12), device=DEV)
+        lib.gs_raster_bwd_cfg(d(spl), vals, ranges, cam, cfg, tf, nl, d(e), None, g2)
+        got.append(g2.cpu())
+    last = int(nl[y, x].item())
+    apart = (al < 0.999 / 255) | (torch.arange(n) >= last)  # certainly not blended at the pixel
+    there = (al > 1.001 / 255) & (torch.arange(n) < last) & (power < -1e-6)
+    assert apart.any() and there.any()
+    assert torch.isnan(got[1][there, 6:9]).all()
+    for cols in (slice(0, 2), slice(2, 5), slice(5, 6), slice(6, 9)):
+        assert (got[1][apart][:, cols] - got[0][apart][:, cols]).abs().max() <= 1e-5 * got[0][:, cols].abs().max()
