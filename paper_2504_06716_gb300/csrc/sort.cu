@@ -5,8 +5,10 @@
 // bits) generated in Gaussian order, but no (Gaussian, tile) entry is ever
 // sorted:
 //   1. compact the visible Gaussians (ascending index) and LSD-radix-sort
-//      them by the bits of their float32 depth (4 passes of 8 bits over the
-//      visible Gaussians only; stable, so equal depths keep index order);
+//      them by the bits of their float32 depth above the view's smallest (3
+//      passes of 9 bits, or 4 of 8 where the depths span more, over the
+//      visible Gaussians only, one launch each; stable, so equal depths keep
+//      index order);
 //   2. in that depth order, emit one entry per super-tile (8 x 8 tiles) a
 //      Gaussian's tile rectangle meets -- about one per Gaussian -- and
 //      stable-sort those few entries by super-tile id (1-2 radix passes);
@@ -26,12 +28,25 @@ __device__ uint32_t g_sort_flags;
 
 namespace {
 
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 4;
-constexpr int kSortBlock = kSortThreads * kSortItems;  // keys per radix block
 constexpr int kMaxRadixBits = 9;                       // digits of up to 9 bits (512 buckets) per pass
 constexpr int kMaxRadix = 1 << kMaxRadixBits;
 constexpr int kScanBlock = 1024;                       // elements per scan block
+
+// Contiguous chunks of a device-side count that the blocks of a pass own, one
+// per SM of the chip, none under kMinChunk (then the last blocks have none).
+constexpr int kSortGrid = 152;
+constexpr int kMinChunk = 2048;
+
+__host__ __device__ inline uint32_t chunk_len(uint32_t n) {
+    const uint32_t c = (n + kSortGrid - 1) / kSortGrid;
+    return c <= (uint32_t)kMinChunk ? (uint32_t)kMinChunk : (c + 255u) & ~255u;
+}
+
+// Rows of a pass's histogram that a count of at most n can use.
+inline int64_t chunk_rows(int64_t n) {
+    const int64_t r = (n + kMinChunk - 1) / kMinChunk;
+    return r < 1 ? 1 : (r < kSortGrid ? r : kSortGrid);
+}
 
 __device__ __forceinline__ unsigned lanemask_lt() {
     unsigned m;
@@ -70,96 +85,146 @@ __device__ __forceinline__ bool splat_visible(const float *splats, int64_t i) {
     return __float_as_int(__ldg(splats + i * kSplat + 11)) > 0;
 }
 
-// ---- stage 1a: compaction of visible Gaussians ----
-// Also zeroes the sort's counters: `zero` [nzero] words and *total_exact.
-__global__ void __launch_bounds__(kScanBlock) k_count_visible(const float *__restrict__ splats, int64_t n,
-                                                             uint32_t *__restrict__ part, uint32_t *__restrict__ zero,
-                                                             int64_t nzero,
-                                                             unsigned long long *__restrict__ total_exact) {
-    wait_prior_grid();
-    int64_t i = (int64_t)blockIdx.x * kScanBlock + threadIdx.x;
-    for (int64_t z = i; z < nzero; z += (int64_t)gridDim.x * kScanBlock) zero[z] = 0u;
-    if (i == 0) *total_exact = 0ull;
-    int f = (i < n) && splat_visible(splats, i);
-    int c = __syncthreads_count(f);
-    if (threadIdx.x == 0) part[blockIdx.x] = (uint32_t)c;
-}
-
-// Exclusive scan of part[0..nb) in place by one block; total to *total. With
-// clip given: *clip = min(total, capacity), and the capacity flag if the
-// total exceeds it (the super-tile entries kept).
+// Sum of this block's kScanBlock values of v, and the sum before element i of
+// part[0 .. nb) with the whole (every thread gets all).
 template <typename T>
-__global__ void __launch_bounds__(1024) k_scan_parts(T *__restrict__ part, int nb, T *__restrict__ total,
-                                                     uint32_t *__restrict__ clip, int64_t capacity) {
-    wait_prior_grid();
-    __shared__ T ws[32];
-    T carry = 0;
-    for (int base = 0; base < nb; base += 1024) {
-        int j = base + threadIdx.x;
-        T v = j < nb ? part[j] : T(0), tot;
-        T ex = block_scan_excl<T>(v, ws, &tot);
-        if (j < nb) part[j] = carry + ex;
-        carry += tot;
-    }
-    if (threadIdx.x == 0) {
-        *total = carry;
-        if (clip) {
-            const unsigned long long Q = (unsigned long long)carry;
-            *clip = (uint32_t)(Q > (unsigned long long)capacity ? capacity : Q);
-            if (Q > (unsigned long long)capacity) atomicOr(&g_sort_flags, GS_FLAG_CAPACITY);
-        }
-    }
-}
+struct PartSum {
+    T before, total;
+};
 
-// ---- LSD radix pass: histogram, per-digit row scan, stable scatter ----
-// The number of keys lives on the device; the three kernels derive the same
-// block count nbd from it and loop over those blocks with whatever grid the
-// host launched (sized for the device, not for the worst case). hist is
-// [radix][nbd].
-__device__ __forceinline__ int radix_blocks(const uint32_t *count) {
-    return (int)((*count + kSortBlock - 1) / kSortBlock);
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *__restrict__ keys,
-                                                            const uint32_t *__restrict__ count, int shift, int bits,
-                                                            uint32_t *__restrict__ hist) {
-    wait_prior_grid();
-    __shared__ uint32_t h[kMaxRadix];
-    const int radix = 1 << bits;
-    const uint32_t mask = (uint32_t)radix - 1u;
-    const uint32_t n = *count;
-    const int nbd = radix_blocks(count);
-    for (int b = blockIdx.x; b < nbd; b += gridDim.x) {
-        for (int d = threadIdx.x; d < radix; d += kSortThreads) h[d] = 0;
-        __syncthreads();
-        const int64_t base = (int64_t)b * kSortBlock;
+template <typename T>
+__device__ __forceinline__ PartSum<T> part_sum(const T *__restrict__ part, int nb, int i, T *warp_sums) {
+    T b = 0, t = 0;
+    for (int j = threadIdx.x; j < nb; j += blockDim.x) {
+        const T v = part[j];
+        t += v;
+        b += j < i ? v : T(0);
+    }
 #pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
-            int64_t i = base + r * kSortThreads + threadIdx.x;
-            if (i < n) atomicAdd(&h[(keys[i] >> shift) & mask], 1u);
+    for (int o = 16; o > 0; o >>= 1) {
+        b += __shfl_xor_sync(kFull, b, o);
+        t += __shfl_xor_sync(kFull, t, o);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (lane == 0) {
+        warp_sums[warp] = b;
+        warp_sums[32 + warp] = t;
+    }
+    __syncthreads();
+    PartSum<T> r{T(0), T(0)};
+    for (int w = 0; w < nw; ++w) {
+        r.before += warp_sums[w];
+        r.total += warp_sums[32 + w];
+    }
+    __syncthreads();
+    return r;
+}
+
+// ---- stage 1a: compaction of visible Gaussians ----
+// Eight small blocks per SM, each over one contiguous range of the Gaussians,
+// so that the next kernel's blocks can sum the counts in front of their own
+// range and no scan runs between the two.
+constexpr int kVisBlock = 256;
+constexpr int kVisGrid = 8 * kSortGrid;
+
+__host__ __device__ inline int64_t vis_range(int64_t n) {
+    const int64_t r = (n + kVisGrid - 1) / kVisGrid;
+    return (r + kVisBlock - 1) / kVisBlock * kVisBlock;
+}
+
+// What the visible Gaussians' depths span: the depth keys are float32 bits
+// less the smallest, so that views whose depths lie within a factor of about
+// 16 sort on at most 27 bits, three passes of 9 instead of four of 8.
+struct DepthSpan {
+    uint32_t lowest, bits;
+};
+
+// The digit of launch k (of 4) of the depth sort; bits 0: the launch does
+// nothing. With three passes it is the first launch that is left out, so that
+// the order ends in the same buffer.
+__host__ __device__ inline int depth_first(uint32_t bits) { return bits <= 27 ? 1 : 0; }
+
+inline unsigned vis_blocks(int64_t n) { return (unsigned)((n + vis_range(n) - 1) / vis_range(n)); }
+
+// The same for a count known on the device only, at most n: as many blocks as
+// any such count may use.
+inline unsigned entry_blocks(int64_t n) {
+    const int64_t b = (n + kVisBlock - 1) / kVisBlock;
+    return (unsigned)(b < kVisGrid ? b : kVisGrid);
+}
+
+// What the first kernel zeroes for the rest of the sort.
+struct ZeroSpans {
+    uint32_t *p[3];
+    int64_t n[3];
+};
+
+// Per block: its visible Gaussians, and the least and largest depth bits
+// among them (part [3][kVisGrid]).
+__global__ void __launch_bounds__(kVisBlock) k_count_visible(const float *__restrict__ splats, int64_t n,
+                                                            uint32_t *__restrict__ part, ZeroSpans z,
+                                                            unsigned long long *__restrict__ total_exact) {
+    __shared__ uint32_t s_c[kVisBlock / 32], s_lo[kVisBlock / 32], s_hi[kVisBlock / 32];
+    wait_prior_grid();
+    const int64_t range = vis_range(n), lo = (int64_t)blockIdx.x * range, hi = lo + range < n ? lo + range : n;
+    const int64_t t = (int64_t)blockIdx.x * kVisBlock + threadIdx.x, all = (int64_t)gridDim.x * kVisBlock;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        for (int64_t i = t; i < z.n[k]; i += all) z.p[k][i] = 0u;
+    if (t == 0) *total_exact = 0ull;
+    uint32_t c = 0u, kl = 0xffffffffu, kh = 0u;
+#pragma unroll 4
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kVisBlock) {
+        const uint32_t key = __float_as_uint(__ldg(splats + i * kSplat + 9));
+        if (splat_visible(splats, i)) {
+            ++c;
+            kl = min(kl, key);
+            kh = max(kh, key);
         }
-        __syncthreads();
-        for (int d = threadIdx.x; d < radix; d += kSortThreads) hist[(int64_t)d * nbd + b] = h[d];
-        __syncthreads();
+    }
+    c = __reduce_add_sync(kFull, c);
+    kl = __reduce_min_sync(kFull, kl);
+    kh = __reduce_max_sync(kFull, kh);
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) { s_c[warp] = c; s_lo[warp] = kl; s_hi[warp] = kh; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kVisBlock / 32; ++w) {
+            c += s_c[w];
+            kl = min(kl, s_lo[w]);
+            kh = max(kh, s_hi[w]);
+        }
+        part[blockIdx.x] = c;
+        part[kVisGrid + blockIdx.x] = kl;
+        part[2 * kVisGrid + blockIdx.x] = kh;
     }
 }
 
-__global__ void __launch_bounds__(1024) k_radix_rowscan(uint32_t *__restrict__ hist, const uint32_t *__restrict__ count,
-                                                        uint32_t *__restrict__ digit_total) {
-    wait_prior_grid();
-    __shared__ uint32_t ws[32];
-    const int nb = radix_blocks(count);
-    uint32_t *row = hist + (int64_t)blockIdx.x * nb;
-    uint32_t carry = 0;
-    for (int base = 0; base < nb; base += 1024) {
-        int j = base + threadIdx.x;
-        uint32_t v = j < nb ? row[j] : 0u, tot;
-        uint32_t ex = block_scan_excl<uint32_t>(v, ws, &tot);
-        if (j < nb) row[j] = carry + ex;
-        carry += tot;
-    }
-    if (threadIdx.x == 0) digit_total[blockIdx.x] = carry;
-}
+// ---- LSD radix pass, one launch ----
+// The number of keys lives on the device; block b owns the keys of chunk b
+// (chunk_len). hist [kSortGrid][kMaxRadix] holds every chunk's digit counts:
+// they were added up by whoever wrote the keys (the kernel before the first
+// pass, or the pass before), key by key with atomics that nobody waits for, at
+// the chunk each key went to. So a pass needs no histogram and no scan launch
+// of its own: a block sums the rows of the chunks in front of its own (at most
+// 152 x 256 words, read by all 1024 threads) for where its digits begin.
+//
+// Inside the block every warp owns a contiguous piece of the chunk: it counts
+// its digits in a row of its own, one scan over the warps per digit turns the
+// rows into positions, and the warp then goes through its keys in order,
+// ranking each 32 with a match. The keys of a piece (up to 256 at a time) are
+// loaded together before anything waits. Two block barriers in all, whatever
+// the chunk's length; the order is stable.
+//
+// Bound by L2: the rows of counts (156 KB per block on 8 bits), the scattered
+// 8-byte words and the atomics (about 2.5 cycles per SM each). The three
+// launches it replaces (histograms, a scan per digit, a scatter of 1024 keys
+// per block with four barriers per 256) took 20 us a pass and four passes at
+// 551K keys; this takes 13 to 16 us and three passes (five passes with the
+// super-tiles' one: 102 -> 68 us). Putting a chunk in order in shared memory
+// first, to write runs, made it 72 us.
+constexpr int kRadixThreads = 1024;
+constexpr int kRadixWarps = kRadixThreads / 32;
 
 // Where a one-pass sort by super-tile id leaves each super-tile's entries:
 // its digit's range of the output. Given (chunk_base non-null), block 0 of
@@ -173,108 +238,151 @@ struct SegPlan {
     int ns, chunk;
 };
 
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const uint32_t *__restrict__ kin,
-                                                               const uint32_t *__restrict__ vin,
-                                                               uint32_t *__restrict__ kout, uint32_t *__restrict__ vout,
-                                                               const uint32_t *__restrict__ count, int shift, int bits,
-                                                               const uint32_t *__restrict__ hist,
-                                                               const uint32_t *__restrict__ digit_total, SegPlan sp) {
-    wait_prior_grid();
-    constexpr int kWarps = kSortThreads / 32;
-    constexpr int kPer = kMaxRadix / kSortThreads;  // buckets per thread (consecutive)
-    __shared__ uint32_t run[kMaxRadix];
-    __shared__ uint32_t wc[kWarps][kMaxRadix];
+// The digit a pass sorts by, and its histogram rows.
+struct Digit {
+    uint32_t *hist;
+    int shift, bits;
+};
+
+// The digit of launch k of the depth sort, from the span of the keys (bits 0:
+// nothing to do). hist: row blocks of the four launches, `stride` words apart.
+__device__ __forceinline__ Digit depth_digit(uint32_t *hist, size_t stride, uint32_t bits, int k) {
+    const int first = depth_first(bits), passes = 4 - first;
+    if (k < first || k > 3) return Digit{nullptr, 0, 0};
+    const int per = max(1, ((int)bits + passes - 1) / passes);
+    return Digit{hist + (size_t)k * stride, (k - first) * per, per};
+}
+
+// A key that goes to `pos` of n, counted for the pass that sorts by d next.
+__device__ __forceinline__ void count_next(const Digit &d, uint32_t key, uint32_t pos, uint32_t chunk) {
+    const uint32_t v = (key >> d.shift) & ((1u << d.bits) - 1u);
+    atomicAdd(d.hist + (size_t)(pos / chunk) * kMaxRadix + v, 1u);
+}
+
+// With span given, launch k of the depth sort (cur.hist the histograms of all
+// four, next unused, stride their distance); else the digits cur and next.
+//
+// A key and its value travel as one 8-byte word (one scattered store instead
+// of two); the last pass writes the values (vout) and, if asked, the keys
+// (kout) by themselves instead.
+__global__ void __launch_bounds__(kRadixThreads) k_radix_pass(const uint2 *__restrict__ in, uint2 *__restrict__ out,
+                                                              uint32_t *__restrict__ kout, uint32_t *__restrict__ vout,
+                                                              const uint32_t *__restrict__ count, Digit cur, Digit next,
+                                                              const DepthSpan *__restrict__ span, int k, size_t stride,
+                                                              SegPlan sp) {
+    extern __shared__ uint32_t s_cnt[];  // [warps][radix]
+    __shared__ uint4 s_sum[2][kRadixThreads];  // [row group][four digits]
     __shared__ uint32_t ws[32];
-    const uint32_t n = *count;
-    const int nbd = radix_blocks(count);
-    const bool plan = sp.chunk_base && blockIdx.x == 0;
-    if ((int)blockIdx.x >= nbd && !plan) return;
-    const int radix = 1 << bits;
-    const uint32_t mask = (uint32_t)radix - 1u;
-    const int t = threadIdx.x, warp = t >> 5;
-    // exclusive scan of the bucket totals: thread t owns buckets kPer t .. kPer t + kPer - 1
-    uint32_t dtot[kPer], own = 0u, tot;
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-        const int d = kPer * t + q;
-        dtot[q] = d < radix ? digit_total[d] : 0u;
-        own += dtot[q];
+    constexpr int kRounds = 8;
+    wait_prior_grid();
+    const uint32_t n = *count, len = chunk_len(n);
+    const uint32_t lo = (uint32_t)blockIdx.x * len;  // below 2^32: 152 chunks hold at most 2^31 + 152 * 256
+    if (span) {
+        uint32_t *hist = cur.hist;
+        const uint32_t bits = span->bits;
+        cur = depth_digit(hist, stride, bits, k);
+        next = depth_digit(hist, stride, bits, k + 1);
+        if (!cur.hist) return;
     }
-    uint32_t dbase[kPer];
-    dbase[0] = block_scan_excl<uint32_t>(own, ws, &tot);
+    const bool plan = sp.chunk_base && blockIdx.x == 0;
+    if (lo >= n && !plan) return;
+    const int radix = 1 << cur.bits, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const uint32_t mask = (uint32_t)radix - 1u;
+    const uint32_t piece = len / kRadixWarps;
+    const uint32_t b0 = lo + warp * piece, b1 = lo < n ? min(n, b0 + piece) : b0;
+    uint2 kv[kRounds];
+    auto load = [&](uint32_t i0) {
 #pragma unroll
-    for (int q = 1; q < kPer; ++q) dbase[q] = dbase[q - 1] + dtot[q - 1];
-    if (plan) {  // block-uniform
-        uint32_t nc[kPer], ncown = 0u, nctot;
-#pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            const int d = kPer * t + q;
-            nc[q] = d < sp.ns ? (dtot[q] + (uint32_t)sp.chunk - 1u) / (uint32_t)sp.chunk : 0u;
-            ncown += nc[q];
+        for (int r = 0; r < kRounds; ++r) {
+            const uint32_t i = i0 + 32 * r + lane;
+            kv[r] = i < b1 ? in[i] : make_uint2(0u, 0u);
         }
-        uint32_t cb = block_scan_excl<uint32_t>(ncown, ws, &nctot);
+    };
+    load(b0);
+    for (int e = t; e < kRadixWarps * radix; e += kRadixThreads) s_cnt[e] = 0u;
+    // rows in front of this chunk's, and all rows, four digits per thread and
+    // every load in flight (a row's words past the radix are zero)
+    const int used = (int)((n + len - 1) / len), quads = max(1, radix / 4), parts = kRadixThreads / quads;
+    uint4 below4 = make_uint4(0u, 0u, 0u, 0u), total4 = below4;
+    {
+        const uint4 *h4 = reinterpret_cast<const uint4 *>(cur.hist) + (t & (quads - 1));
+#pragma unroll 20
+        for (int r = t / quads; r < used; r += parts) {
+            const uint4 v = h4[(size_t)r * (kMaxRadix / 4)];
+            total4.x += v.x; total4.y += v.y; total4.z += v.z; total4.w += v.w;
+            if (r < (int)blockIdx.x) { below4.x += v.x; below4.y += v.y; below4.z += v.z; below4.w += v.w; }
+        }
+    }
+    s_sum[0][t] = below4;
+    s_sum[1][t] = total4;
+    __syncthreads();
+    uint32_t *row = s_cnt + warp * radix;
+    for (uint32_t i0 = b0; i0 < b1; i0 += 32 * kRounds) {  // this warp's piece, counted
+        if (i0 != b0) load(i0);
 #pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            const int d = kPer * t + q;
-            if (d < sp.ns) {
-                sp.chunk_base[d] = cb;
-                for (uint32_t c = 0; c < nc[q]; ++c)
-                    sp.chunk_rec[cb + c] = make_uint4((uint32_t)d, dbase[q] + c * (uint32_t)sp.chunk,
-                                                      dbase[q] + dtot[q], cb);
-            }
-            cb += nc[q];
+        for (int r = 0; r < kRounds; ++r)
+            if (i0 + 32 * r + lane < b1) atomicAdd(row + ((kv[r].x >> cur.shift) & mask), 1u);
+    }
+    // per digit (threads below radix): totals, their exclusive scan, this chunk's start
+    uint32_t below = 0u, total = 0u;
+    if (t < radix) {
+        const uint32_t *sb = reinterpret_cast<const uint32_t *>(s_sum[0]), *st = reinterpret_cast<const uint32_t *>(s_sum[1]);
+#pragma unroll 8
+        for (int q = 0; q < parts; ++q) {
+            below += sb[t + q * 4 * quads];
+            total += st[t + q * 4 * quads];
+        }
+    }
+    uint32_t all;
+    const uint32_t dbase = block_scan_excl<uint32_t>(total, ws, &all);  // its barriers also order the counts
+    if (plan) {
+        const uint32_t nc = t < sp.ns ? (total + (uint32_t)sp.chunk - 1u) / (uint32_t)sp.chunk : 0u;
+        uint32_t nctot;
+        const uint32_t cb = block_scan_excl<uint32_t>(nc, ws, &nctot);
+        if (t < sp.ns) {
+            sp.chunk_base[t] = cb;
+            for (uint32_t c = 0; c < nc; ++c)
+                sp.chunk_rec[cb + c] =
+                    make_uint4((uint32_t)t, dbase + c * (uint32_t)sp.chunk, dbase + total, cb);
         }
         if (t == 0) sp.chunk_base[sp.ns] = nctot;
-        if ((int)blockIdx.x >= nbd) return;
+        if (lo >= n) return;
     }
-    for (int b = blockIdx.x; b < nbd; b += gridDim.x) {
-        const int64_t base = (int64_t)b * kSortBlock;
-#pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            const int d = kPer * t + q;
-            if (d < radix) run[d] = dbase[q] + hist[(int64_t)d * nbd + b];
+    if (t < radix) {
+        uint32_t c = dbase + below;
+#pragma unroll 8
+        for (int w = 0; w < kRadixWarps; ++w) {
+            const uint32_t x = s_cnt[w * radix + t];
+            s_cnt[w * radix + t] = c;
+            c += x;
         }
-        // all of the block's keys and values in flight at once; then ranked
-        // and written a sub-block of kSortThreads at a time, in order
-        uint32_t kr[kSortItems], vr[kSortItems];
+    }
+    __syncthreads();
+    const unsigned lt = lanemask_lt();
+    const bool held = piece <= 32 * kRounds;  // the registers still hold the whole piece
+    for (uint32_t i0 = b0; i0 < b1; i0 += 32 * kRounds) {
+        if (!held) load(i0);
 #pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
-            const int64_t i = base + r * kSortThreads + t;
-            kr[r] = i < n ? kin[i] : 0u;
-            vr[r] = i < n ? vin[i] : 0u;
-        }
-#pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
-            int64_t i = base + r * kSortThreads + t;
-            bool valid = i < n;
-            uint32_t key = kr[r];
-            uint32_t d = valid ? ((key >> shift) & mask) : 0xffffu;
-            unsigned peers = __match_any_sync(kFull, d);
-            unsigned lrank = __popc(peers & lanemask_lt());
-            for (int e = t; e < radix; e += kSortThreads) {
-#pragma unroll
-                for (int w = 0; w < kWarps; ++w) wc[w][e] = 0u;
-            }
-            __syncthreads();
-            if (valid && lrank == 0) wc[warp][d] = (uint32_t)__popc(peers);
-            __syncthreads();
-            for (int e = t; e < radix; e += kSortThreads) {
-                uint32_t c = run[e];
-#pragma unroll
-                for (int w = 0; w < kWarps; ++w) {
-                    uint32_t x = wc[w][e];
-                    wc[w][e] = c;
-                    c += x;
-                }
-                run[e] = c;
-            }
-            __syncthreads();
+        for (int r = 0; r < kRounds; ++r) {
+            if (i0 + 32 * r >= b1) break;  // uniform
+            const bool valid = i0 + 32 * r + lane < b1;
+            const uint32_t key = kv[r].x;
+            const uint32_t d = valid ? (key >> cur.shift) & mask : 0xffffu;
+            const unsigned peers = __match_any_sync(kFull, d);
+            uint32_t pos = 0u;
+            if (valid) pos = row[d] + __popc(peers & lt);
+            __syncwarp();
+            if (valid && !(peers & lt)) row[d] += (uint32_t)__popc(peers);
+            __syncwarp();
             if (valid) {
-                uint32_t pos = wc[warp][d] + lrank;
-                kout[pos] = key;
-                vout[pos] = vr[r];
+                if (vout) {
+                    if (kout) kout[pos] = key;
+                    vout[pos] = kv[r].y;
+                } else {
+                    out[pos] = kv[r];
+                    count_next(next, key, pos, len);
+                }
             }
-            __syncthreads();
         }
     }
 }
@@ -451,23 +559,100 @@ __device__ __forceinline__ bool cull_rect(const float4 *cull, uint32_t g, int &x
     return x0 < x1 && y0 < y1;
 }
 
-// The depth keys and indices of the visible Gaussians, ascending index, and
-// their cull records.
-__global__ void __launch_bounds__(kScanBlock) k_emit_visible(const float *__restrict__ splats, int64_t n,
-                                                            const uint32_t *__restrict__ part, DevCam cam,
-                                                            uint32_t *__restrict__ keys, uint32_t *__restrict__ vals,
-                                                            float4 *__restrict__ cull) {
+// The items a block takes at once: warp w has consecutive ones, up to four
+// rounds of 32 of them (fewer when the block's range is short, so that every
+// warp has some), a thread's loads in flight together, and one barrier orders
+// the warps.
+constexpr int kVisRounds = 4;
+
+__device__ __forceinline__ int vis_rounds(int64_t range) {
+    return range >= kVisRounds * kVisBlock ? kVisRounds : (int)((range + kVisBlock - 1) / kVisBlock);
+}
+
+// Exclusive sum over the block's warps of v (one value per warp) and the
+// block's total; double-buffered by `turn`, one barrier.
+__device__ __forceinline__ PartSum<uint32_t> warps_before(uint32_t v, uint32_t (*buf)[kVisBlock / 32], int turn) {
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) buf[turn & 1][warp] = v;
+    __syncthreads();
+    PartSum<uint32_t> r{0u, 0u};
+#pragma unroll
+    for (int w = 0; w < kVisBlock / 32; ++w) {
+        const uint32_t x = buf[turn & 1][w];
+        r.before += w < warp ? x : 0u;
+        r.total += x;
+    }
+    return r;
+}
+
+// The depth keys and indices of the visible Gaussians, ascending index, their
+// cull records, and the first radix pass's digit counts.
+__global__ void __launch_bounds__(kVisBlock) k_emit_visible(const float *__restrict__ splats, int64_t n,
+                                                           const uint32_t *__restrict__ part, DevCam cam,
+                                                           uint2 *__restrict__ kv0, uint2 *__restrict__ kv1,
+                                                           float4 *__restrict__ cull, uint32_t *__restrict__ n_vis,
+                                                           DepthSpan *__restrict__ span, uint32_t *__restrict__ hist,
+                                                           size_t stride) {
+    __shared__ uint32_t ps[64];
+    __shared__ uint32_t buf[2][kVisBlock / 32];
+    __shared__ uint32_t s_lo, s_hi;
     wait_prior_grid();
-    __shared__ int ws[32];
-    int64_t i = (int64_t)blockIdx.x * kScanBlock + threadIdx.x;
-    int f = (i < n) && splat_visible(splats, i);
-    int tot;
-    int r = block_scan_excl<int>(f, ws, &tot);
-    if (f) {
-        uint32_t pos = part[blockIdx.x] + (uint32_t)r;
-        keys[pos] = __float_as_uint(__ldg(splats + i * kSplat + 9));
-        vals[pos] = (uint32_t)i;
-        write_cull(splats, (uint32_t)i, cam, cull);
+    if (threadIdx.x == 0) { s_lo = 0xffffffffu; s_hi = 0u; }
+    uint32_t kl = 0xffffffffu, kh = 0u;
+    for (int j = threadIdx.x; j < (int)gridDim.x; j += kVisBlock) {
+        kl = min(kl, part[kVisGrid + j]);
+        kh = max(kh, part[2 * kVisGrid + j]);
+    }
+    kl = __reduce_min_sync(kFull, kl);
+    kh = __reduce_max_sync(kFull, kh);
+    const PartSum<uint32_t> sum = part_sum<uint32_t>(part, (int)gridDim.x, (int)blockIdx.x, ps);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(&s_lo, kl);
+        atomicMax(&s_hi, kh);
+    }
+    __syncthreads();
+    const uint32_t lowest = s_lo, bits = sum.total ? 32u - (uint32_t)__clz(s_hi - lowest) : 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *n_vis = sum.total;
+        span->lowest = lowest;
+        span->bits = bits;
+    }
+    const int first = depth_first(bits);
+    const Digit dig = depth_digit(hist, stride, bits, first);
+    uint2 *kv = first ? kv1 : kv0;
+    const uint32_t chunk = chunk_len(sum.total);
+    uint32_t at = sum.before;
+    const int64_t range = vis_range(n), lo = (int64_t)blockIdx.x * range, hi = lo + range < n ? lo + range : n;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt = lanemask_lt();
+    const int rounds = vis_rounds(range);
+    int turn = 0;
+    for (int64_t base = lo; base < hi; base += (int64_t)rounds * kVisBlock, ++turn) {
+        const int64_t i0 = base + warp * 32 * rounds + lane;
+        unsigned seen[kVisRounds];
+        uint32_t mine = 0u;
+#pragma unroll
+        for (int r = 0; r < kVisRounds; ++r)
+            seen[r] = r < rounds && i0 + 32 * r < hi && splat_visible(splats, i0 + 32 * r);
+#pragma unroll
+        for (int r = 0; r < kVisRounds; ++r) {
+            seen[r] = __ballot_sync(kFull, seen[r] != 0u);
+            mine += (uint32_t)__popc(seen[r]);
+        }
+        const PartSum<uint32_t> w = warps_before(mine, buf, turn);
+        uint32_t pos0 = at + w.before;
+        at += w.total;
+#pragma unroll
+        for (int r = 0; r < kVisRounds; ++r) {
+            if ((seen[r] >> lane) & 1u) {
+                const uint32_t pos = pos0 + (uint32_t)__popc(seen[r] & lt), i = (uint32_t)(i0 + 32 * r);
+                const uint32_t key = __float_as_uint(__ldg(splats + (int64_t)i * kSplat + 9)) - lowest;
+                kv[pos] = make_uint2(key, i);
+                count_next(dig, key, pos, chunk);
+                write_cull(splats, i, cam, cull);
+            }
+            pos0 += (uint32_t)__popc(seen[r]);
+        }
     }
 }
 
@@ -480,17 +665,29 @@ __device__ __forceinline__ unsigned long long super_entries(const float4 *cull, 
     return (unsigned long long)super_rect(x0, y0, x1, y1, sx0, sy0, sx1, sy1);
 }
 
-__global__ void __launch_bounds__(kScanBlock) k_count_entries(const float4 *__restrict__ cull,
+// Range of the depth-ordered Gaussians a block of the two kernels below owns.
+__device__ __forceinline__ void entry_range(uint32_t n_vis, int64_t &lo, int64_t &hi) {
+    const int64_t range = vis_range((int64_t)n_vis);
+    lo = (int64_t)blockIdx.x * range;
+    hi = lo + range < (int64_t)n_vis ? lo + range : (int64_t)n_vis;
+}
+
+__global__ void __launch_bounds__(kVisBlock) k_count_entries(const float4 *__restrict__ cull,
                                                              const uint32_t *__restrict__ order,
                                                              const uint32_t *__restrict__ n_vis,
                                                              unsigned long long *__restrict__ part_s) {
     wait_prior_grid();
     __shared__ unsigned long long ws[32];
-    int64_t k = (int64_t)blockIdx.x * kScanBlock + threadIdx.x;
-    int sx0, sy0, sx1, sy1;
-    const unsigned long long cs = k < *n_vis ? super_entries(cull, order[k], sx0, sy0, sx1, sy1) : 0ull;
+    int64_t lo, hi;
+    entry_range(*n_vis, lo, hi);
+    unsigned long long c = 0ull;
+#pragma unroll 4
+    for (int64_t k = lo + threadIdx.x; k < hi; k += kVisBlock) {
+        int sx0, sy0, sx1, sy1;
+        c += super_entries(cull, order[k], sx0, sy0, sx1, sy1);
+    }
     unsigned long long tot;
-    block_scan_excl<unsigned long long>(cs, ws, &tot);
+    block_scan_excl<unsigned long long>(c, ws, &tot);
     if (threadIdx.x == 0) part_s[blockIdx.x] = tot;
 }
 
@@ -514,20 +711,6 @@ __device__ __forceinline__ void warp_add_total(unsigned long long v, unsigned lo
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(total, v);
 }
 
-__global__ void __launch_bounds__(256) k_count_exact(const float *__restrict__ splats,
-                                                    const uint32_t *__restrict__ order,
-                                                    const uint32_t *__restrict__ n_vis, DevCam cam,
-                                                    const unsigned long long *__restrict__ total_s, int64_t capacity,
-                                                    unsigned long long *__restrict__ total_exact) {
-    wait_prior_grid();
-    if (*total_s <= (unsigned long long)capacity) return;
-    unsigned long long mine = 0ull;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < *n_vis;
-         k += (int64_t)gridDim.x * blockDim.x)
-        mine += exact_tiles(splats, order[k], cam);
-    warp_add_total(mine, total_exact);
-}
-
 // count_dev = P, the number of entries: the sum of the tile counts, or the
 // exact count above when the super-tile entries overflowed.
 __global__ void k_finish_count(const unsigned long long *__restrict__ total_t,
@@ -540,37 +723,85 @@ __global__ void k_finish_count(const unsigned long long *__restrict__ total_t,
     if (P > (unsigned long long)capacity) atomicOr(&g_sort_flags, GS_FLAG_CAPACITY);
 }
 
-__global__ void __launch_bounds__(kScanBlock) k_emit_super(const float *__restrict__ splats,
+// The super-tile entries in depth order, clipped to the capacity (*sclip of
+// them kept, of *total_s), and the first super-tile pass's digit counts.
+__global__ void __launch_bounds__(kVisBlock) k_emit_super(const float *__restrict__ splats,
                                                           const float4 *__restrict__ cull,
                                                           const uint32_t *__restrict__ order,
                                                           const uint32_t *__restrict__ n_vis, DevCam cam,
                                                           int supers_x, const unsigned long long *__restrict__ part_s,
-                                                          const unsigned long long *__restrict__ total_s,
-                                                          int64_t capacity, uint32_t *__restrict__ skeys,
-                                                          uint32_t *__restrict__ svals,
-                                                          unsigned long long *__restrict__ total_exact) {
+                                                          unsigned long long *__restrict__ total_s,
+                                                          uint32_t *__restrict__ sclip, int64_t capacity,
+                                                          uint2 *__restrict__ entries,
+                                                          uint32_t *__restrict__ skeys, uint32_t *__restrict__ svals,
+                                                          unsigned long long *__restrict__ total_exact, Digit first) {
+    __shared__ unsigned long long ps[64];
+    __shared__ uint32_t buf[2][kVisBlock / 32];
     wait_prior_grid();
-    __shared__ unsigned long long ws[32];
-    int64_t k = (int64_t)blockIdx.x * kScanBlock + threadIdx.x;
-    int sx0 = 0, sy0 = 0, sx1 = 0, sy1 = 0;
-    uint32_t g = 0;
-    unsigned long long c = 0ull;
-    if (k < *n_vis) {
-        g = order[k];
-        c = super_entries(cull, g, sx0, sy0, sx1, sy1);
+    const unsigned long long cap = (unsigned long long)capacity;
+    const PartSum<unsigned long long> sum =
+        part_sum<unsigned long long>(part_s, (int)gridDim.x, (int)blockIdx.x, ps);
+    const uint32_t kept = (uint32_t)(sum.total > cap ? cap : sum.total);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *total_s = sum.total;
+        *sclip = kept;
+        if (sum.total > cap) atomicOr(&g_sort_flags, GS_FLAG_CAPACITY);
     }
-    unsigned long long tot;
-    unsigned long long off = part_s[blockIdx.x] + block_scan_excl<unsigned long long>(c, ws, &tot);
-    if (*total_s > (unsigned long long)capacity)  // the super-tile entries overflowed: P counted tile by tile
-        warp_add_total(c ? exact_tiles(splats, g, cam) : 0ull, total_exact);
-    if (c == 0) return;
-    for (int y = sy0; y < sy1; ++y)
-        for (int x = sx0; x < sx1; ++x) {
-            if (off >= (unsigned long long)capacity) return;
-            skeys[off] = (uint32_t)(y * supers_x + x);
-            svals[off] = g;
-            ++off;
+    const uint32_t chunk = chunk_len(kept);
+    unsigned long long at = sum.before;
+    int64_t lo, hi;
+    entry_range(*n_vis, lo, hi);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rounds = vis_rounds(hi - lo);
+    int turn = 0;
+    for (int64_t base = lo; base < hi; base += (int64_t)rounds * kVisBlock, ++turn) {
+        const int64_t k0 = base + warp * 32 * rounds + lane;
+        uint32_t g[kVisRounds], c[kVisRounds], before[kVisRounds], mine = 0u;
+#pragma unroll
+        for (int r = 0; r < kVisRounds; ++r)
+            g[r] = r < rounds && k0 + 32 * r < hi ? order[k0 + 32 * r] : 0xffffffffu;
+        int sx0, sy0, sx1, sy1;
+#pragma unroll
+        for (int r = 0; r < kVisRounds; ++r)
+            c[r] = g[r] != 0xffffffffu ? (uint32_t)super_entries(cull, g[r], sx0, sy0, sx1, sy1) : 0u;
+#pragma unroll
+        for (int r = 0; r < kVisRounds; ++r) {  // at most 1024 x 65536 entries in a batch: 32 bits
+            uint32_t x = c[r];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, x, o);
+                if (lane >= o) x += y;
+            }
+            before[r] = mine + x - c[r];
+            mine += __shfl_sync(kFull, x, 31);
         }
+        const PartSum<uint32_t> w = warps_before(mine, buf, turn);
+        const unsigned long long off0 = at + w.before;
+        at += w.total;
+        if (sum.total > cap) {  // the super-tile entries overflowed: P counted tile by tile
+            unsigned long long m = 0ull;
+            for (int r = 0; r < kVisRounds; ++r) m += c[r] ? exact_tiles(splats, g[r], cam) : 0ull;
+            warp_add_total(m, total_exact);
+        }
+#pragma unroll
+        for (int r = 0; r < kVisRounds; ++r) {
+            if (c[r] == 0u) continue;
+            unsigned long long off = off0 + before[r];
+            super_entries(cull, g[r], sx0, sy0, sx1, sy1);
+            for (int y = sy0; y < sy1; ++y)
+                for (int x = sx0; x < sx1; ++x, ++off) {
+                    if (off >= cap) break;
+                    const uint32_t key = (uint32_t)(y * supers_x + x);
+                    if (first.hist) {
+                        entries[off] = make_uint2(key, g[r]);
+                        count_next(first, key, (uint32_t)off, chunk);
+                    } else {  // one super-tile: already in order
+                        skeys[off] = key;
+                        svals[off] = g[r];
+                    }
+                }
+        }
+    }
 }
 
 // Segments of the super-tile-sorted list: seg_lo / seg_hi [ns] (zero for an
@@ -776,10 +1007,15 @@ __global__ void __launch_bounds__(kChunk) k_chunk_counts(const float *__restrict
 }
 
 // Tile starts (exclusive scan of the tile counts over tile ids) and the
-// ranges, clipped to the capacity: per-block sums, a scan of those, then each
-// block scans its own tiles from its offset; block 0 of the last step also
-// sets count_dev = P, the sum of the tile counts, or the exact count when the
-// super-tile entries overflowed (and the capacity flag if P exceeds it).
+// ranges, clipped to the capacity: each block scans its own 1024 tiles from
+// the sum of those in front, taken from the tile counts themselves while the
+// grid is small (up to kDirectTiles blocks; 24 words per thread at most) and
+// from per-block sums (k_tile_sums, one launch more) for larger ones. The last
+// block also sets count_dev = P, the sum of the tile counts, or the exact
+// count when the super-tile entries overflowed (and the capacity flag if P
+// exceeds it).
+constexpr int kDirectTiles = 24;
+
 __global__ void __launch_bounds__(kScanBlock) k_tile_sums(const uint32_t *__restrict__ tile_count, int64_t tiles,
                                                          unsigned long long *__restrict__ part) {
     wait_prior_grid();
@@ -793,7 +1029,6 @@ __global__ void __launch_bounds__(kScanBlock) k_tile_sums(const uint32_t *__rest
 __global__ void __launch_bounds__(kScanBlock) k_tile_starts(const uint32_t *__restrict__ tile_count, int64_t tiles,
                                                            const unsigned long long *__restrict__ part,
                                                            int64_t capacity,
-                                                           const unsigned long long *__restrict__ total_t,
                                                            const unsigned long long *__restrict__ total_s,
                                                            const unsigned long long *__restrict__ total_exact,
                                                            unsigned long long *__restrict__ tile_start,
@@ -801,10 +1036,20 @@ __global__ void __launch_bounds__(kScanBlock) k_tile_starts(const uint32_t *__re
                                                            int64_t *__restrict__ count_dev) {
     wait_prior_grid();
     __shared__ unsigned long long ws[32];
-    const int64_t j = (int64_t)blockIdx.x * kScanBlock + threadIdx.x;
+    __shared__ unsigned long long ps[64];
+    const int64_t first = (int64_t)blockIdx.x * kScanBlock, j = first + threadIdx.x;
     const unsigned long long n = j < tiles ? tile_count[j] : 0ull;
+    unsigned long long before;
+    if (part) {
+        before = part_sum<unsigned long long>(part, (int)gridDim.x, (int)blockIdx.x, ps).before;
+    } else {
+        unsigned long long b = 0ull;
+#pragma unroll 8
+        for (int64_t q = threadIdx.x; q < first; q += kScanBlock) b += tile_count[q];
+        block_scan_excl<unsigned long long>(b, ws, &before);
+    }
     unsigned long long tot;
-    const unsigned long long st = part[blockIdx.x] + block_scan_excl<unsigned long long>(n, ws, &tot);
+    const unsigned long long st = before + block_scan_excl<unsigned long long>(n, ws, &tot);
     const unsigned long long cap = (unsigned long long)capacity;
     if (j < tiles) {
         const unsigned long long en = st + n;
@@ -813,8 +1058,8 @@ __global__ void __launch_bounds__(kScanBlock) k_tile_starts(const uint32_t *__re
         ranges[2 * j] = n ? (uint32_t)(st < cap ? st : cap) : 0u;
         ranges[2 * j + 1] = n ? (uint32_t)(en < cap ? en : cap) : 0u;
     }
-    if (j == 0) {
-        const unsigned long long P = *total_s > cap ? *total_exact : *total_t;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        const unsigned long long P = *total_s > cap ? *total_exact : before + tot;
         *count_dev = (int64_t)P;
         if (P > cap) atomicOr(&g_sort_flags, GS_FLAG_CAPACITY);
     }
@@ -893,14 +1138,18 @@ __global__ void __launch_bounds__(kChunk) k_expand(const float *__restrict__ spl
 
 // ---- workspace ----
 struct SortWs {
-    uint32_t *keys[2], *vals[2];  // visible Gaussians: depth keys and indices
-    uint32_t *skeys[2], *svals1;  // super-tile entries; the other value buffer is the output
-    uint32_t *hist, *digit_total, *part32;
+    uint2 *kv[2];                 // visible Gaussians: (depth key, index)
+    uint32_t *order;              // [n] their indices in depth order
+    uint2 *entries[2];            // super-tile entries: (super-tile, index); the second shares the masks' place
+    uint32_t *skeys, *svals;      // in super-tile order
+    uint32_t *hist_d, *hist_s;    // digit counts of the depth and super-tile passes (hist_of)
+    uint32_t *part32;
     unsigned long long *part_s, *total_s, *total_t, *total_exact;
     unsigned long long *masks;                 // [capacity] tile mask of each super-tile entry
     unsigned long long *tile_part;             // [tile blocks]
     float4 *cull;                              // [2 n] cull record of each visible Gaussian
     uint32_t *n_vis, *sclip;
+    DepthSpan *span;
     uint32_t *seg_lo, *seg_hi, *chunk_base;    // [ns], [ns], [ns + 1]
     uint32_t *tile_count;                      // [tiles]
     unsigned long long *tile_start;            // [tiles]
@@ -913,33 +1162,36 @@ inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 inline int64_t max_chunks(int64_t cap, int64_t ns) { return (cap + kChunk - 1) / kChunk + ns + 1; }
 
+constexpr int kDepthPasses = 4, kSuperPasses = 2;  // super-tile ids take at most 16 bits
+
+// Digit counts of pass p of a sort whose count is at most n.
+inline uint32_t *hist_of(uint32_t *base, int64_t n, int p) { return base + (size_t)p * chunk_rows(n) * kMaxRadix; }
+
 inline SortWs sort_layout(char *base, int64_t n, int64_t cap, int64_t tiles, int64_t ns) {
     SortWs w;
-    int64_t nbN = (n + kSortBlock - 1) / kSortBlock, nbC = (cap + kSortBlock - 1) / kSortBlock;
-    int64_t nbMax = nbN > nbC ? nbN : nbC;
-    if (nbMax < 1) nbMax = 1;
-    int64_t nbS = (n + kScanBlock - 1) / kScanBlock;
-    if (nbS < 1) nbS = 1;
     size_t off = 0;
     auto take = [&](size_t bytes) -> char * {
         char *p = base ? base + off : nullptr;
         off += align256(bytes);
         return p;
     };
-    for (int k = 0; k < 2; ++k) w.keys[k] = (uint32_t *)take(4 * (size_t)n);
-    for (int k = 0; k < 2; ++k) w.vals[k] = (uint32_t *)take(4 * (size_t)n);
-    for (int k = 0; k < 2; ++k) w.skeys[k] = (uint32_t *)take(4 * (size_t)cap);
-    w.svals1 = (uint32_t *)take(4 * (size_t)cap);
-    w.hist = (uint32_t *)take(4 * (size_t)kMaxRadix * (size_t)nbMax);
-    w.digit_total = (uint32_t *)take(4 * (size_t)kMaxRadix);
-    w.part32 = (uint32_t *)take(4 * (size_t)nbS);
-    w.part_s = (unsigned long long *)take(8 * (size_t)nbS);
+    for (int k = 0; k < 2; ++k) w.kv[k] = (uint2 *)take(8 * (size_t)n);
+    w.order = (uint32_t *)w.kv[0];  // written by the pass that reads kv[1]
+    w.entries[0] = (uint2 *)take(8 * (size_t)cap);
+    w.svals = (uint32_t *)take(4 * (size_t)cap);
+    w.skeys = (uint32_t *)w.entries[0];  // kept only by two passes (the second reads entries[1]) or none
+    w.hist_d = (uint32_t *)take(4 * (size_t)kDepthPasses * kMaxRadix * (size_t)chunk_rows(n));
+    w.hist_s = (uint32_t *)take(4 * (size_t)kSuperPasses * kMaxRadix * (size_t)chunk_rows(cap));
+    w.part32 = (uint32_t *)take(4 * 3 * (size_t)kVisGrid);
+    w.part_s = (unsigned long long *)take(8 * (size_t)kVisGrid);
     w.total_s = (unsigned long long *)take(8);
     w.total_t = (unsigned long long *)take(8);
     w.total_exact = (unsigned long long *)take(8);
     w.masks = (unsigned long long *)take(8 * (size_t)cap);
+    w.entries[1] = (uint2 *)w.masks;  // the masks are made after the sort
     w.cull = (float4 *)take(32 * (size_t)n);
     w.n_vis = (uint32_t *)take(4);
+    w.span = (DepthSpan *)take(sizeof(DepthSpan));
     w.sclip = (uint32_t *)take(4);
     // zeroed together before each sort: segment bounds, then tile counts
     w.seg_lo = (uint32_t *)take(4 * (size_t)(2 * ns + tiles));
@@ -969,29 +1221,25 @@ inline SuperGrid super_grid(int32_t width, int32_t height, int32_t tile) {
     return g;
 }
 
-// One full LSD sort of (keys, vals) over *count (bounded by `bound`) on `bits`
-// low bits; buffers ping-pong between index `in` and 1 - in. The last pass
-// writes the segment plan sp (if given). Returns the index holding the result.
-int radix_sort(uint32_t *const keys[2], uint32_t *const vals[2], int in, const uint32_t *count, int64_t bound,
-               int total_bits, const SortWs &w, cudaStream_t s, SegPlan sp = SegPlan{}) {
-    if (total_bits <= 0) return in;
-    // 8-bit digits, or one pass of up to kMaxRadixBits when that suffices
-    int npass = total_bits <= kMaxRadixBits ? 1 : (total_bits + 7) / 8;
-    int per = (total_bits + npass - 1) / npass;
-    const int64_t nb = (bound + kSortBlock - 1) / kSortBlock, cap = resident_blocks();
-    const int grid = (int)(nb < 1 ? 1 : (nb < cap ? nb : cap));
-    int shift = 0;
-    for (int p = 0; p < npass; ++p) {
-        int bits = per < total_bits - shift ? per : total_bits - shift;
-        launch_chained(k_radix_hist, grid, kSortThreads, s, keys[in], count, shift, bits, w.hist);
-        launch_chained(k_radix_rowscan, 1 << bits, 1024, s, w.hist, count, w.digit_total);
-        launch_chained(k_radix_scatter, grid, kSortThreads, s, keys[in], vals[in], keys[1 - in], vals[1 - in], count,
-                       shift, bits, w.hist, w.digit_total, p == npass - 1 ? sp : SegPlan{});
-        note_launches(3);
-        in = 1 - in;
-        shift += bits;
-    }
-    return in;
+// The digits of a sort on `total_bits` low bits: 8 bits each, or one pass of up
+// to kMaxRadixBits when that suffices.
+inline int radix_passes(int total_bits) {
+    return total_bits <= 0 ? 0 : (total_bits <= kMaxRadixBits ? 1 : (total_bits + 7) / 8);
+}
+
+inline Digit radix_digit(uint32_t *hist, int64_t bound, int total_bits, int p) {
+    const int npass = radix_passes(total_bits);
+    if (p >= npass) return Digit{nullptr, 0, 0};
+    const int per = (total_bits + npass - 1) / npass, shift = p * per;
+    return Digit{hist_of(hist, bound, p), shift, per < total_bits - shift ? per : total_bits - shift};
+}
+
+// A radix pass over a count of at most `bound`, on a digit of at most `bits`.
+template <typename... Args>
+void launch_radix(int bits, int64_t bound, cudaStream_t s, Args &&...args) {
+    const size_t smem = (sizeof(uint32_t) * (size_t)kRadixWarps) << bits;  // 64 KB for a 9-bit digit
+    cudaFuncSetAttribute(k_radix_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);  // beyond 48 KB
+    launch_chained_smem(k_radix_pass, (unsigned)chunk_rows(bound), kRadixThreads, smem, s, static_cast<Args &&>(args)...);
 }
 
 int ceil_log2(int64_t x) {
@@ -1031,7 +1279,6 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
     DevCam dc = make_cam(cam);
     const int64_t tiles = sg.tiles;
     const int ns = (int)sg.ns;
-    const int nbS = (int)((n + kScanBlock - 1) / kScanBlock);
 
     if (n == 0 || capacity == 0) {
         k_zero_u32<<<grid_for(2 * tiles, 256), 256, 0, s>>>(ranges, 2 * tiles);
@@ -1041,56 +1288,67 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
             return launch_status();
         }
     }
+    const int sbits = ceil_log2(sg.ns), npass = radix_passes(sbits);
     // stage 1: visible Gaussians by depth (the first kernel also zeroes the
-    // segment bounds, tile counts and exact count)
-    launch_chained(k_count_visible, nbS, kScanBlock, s, splats, n, w.part32, w.seg_lo, 2 * sg.ns + tiles,
-                   w.total_exact);
-    launch_chained(k_scan_parts<uint32_t>, 1, 1024, s, w.part32, nbS, w.n_vis, nullptr, 0);
-    launch_chained(k_emit_visible, nbS, kScanBlock, s, splats, n, w.part32, dc, w.keys[0], w.vals[0], w.cull);
-    note_launches(3);
-    int cur = radix_sort(w.keys, w.vals, 0, w.n_vis, n, 32, w, s);
+    // segment bounds, tile counts, digit counts and exact count)
+    const ZeroSpans z{{w.seg_lo, w.hist_d, w.hist_s},
+                      {2 * sg.ns + tiles, kDepthPasses * kMaxRadix * chunk_rows(n),
+                       capacity ? npass * kMaxRadix * chunk_rows(capacity) : 0}};
+    const unsigned vgrid = vis_blocks(n), egrid = entry_blocks(n);
+    const size_t hstride = (size_t)chunk_rows(n) * kMaxRadix;
+    launch_chained(k_count_visible, vgrid, kVisBlock, s, splats, n, w.part32, z, w.total_exact);
+    launch_chained(k_emit_visible, vgrid, kVisBlock, s, splats, n, w.part32, dc, w.kv[0], w.kv[1], w.cull,
+                   w.n_vis, w.span, w.hist_d, hstride);
+    for (int k = 0; k < kDepthPasses; ++k)
+        launch_radix(kMaxRadixBits, n, s, w.kv[k & 1], w.kv[1 - (k & 1)], static_cast<uint32_t *>(nullptr),
+                     k == 3 ? w.order : nullptr, w.n_vis, Digit{w.hist_d, 0, 0}, Digit{nullptr, 0, 0}, w.span, k,
+                     hstride, SegPlan{});
+    note_launches(2 + kDepthPasses);
+    const uint32_t *order = w.order;
     // stage 2: super-tile entries in depth order, stable-sorted by super-tile
-    launch_chained(k_count_entries, nbS, kScanBlock, s, w.cull, w.vals[cur], w.n_vis, w.part_s);
-    launch_chained(k_scan_parts<unsigned long long>, 1, 1024, s, w.part_s, nbS, w.total_s, w.sclip, capacity);
-    note_launches(2);
+    launch_chained(k_count_entries, egrid, kVisBlock, s, w.cull, order, w.n_vis, w.part_s);
+    note_launches(1);
+    launch_chained(k_emit_super, egrid, kVisBlock, s, splats, w.cull, order, w.n_vis, dc, sg.supers_x, w.part_s,
+                   w.total_s, w.sclip, capacity, w.entries[0], w.skeys, w.svals, w.total_exact,
+                   capacity ? radix_digit(w.hist_s, capacity, sbits, 0) : Digit{nullptr, 0, 0});
+    note_launches(1);
     if (capacity == 0) {
         cudaMemsetAsync(w.total_t, 0, sizeof(unsigned long long), s);
-        launch_chained(k_count_exact, (unsigned)resident_blocks(), 256, s, splats, w.vals[cur], w.n_vis, dc, w.total_s,
-                       capacity, w.total_exact);
         launch_chained(k_finish_count, 1, 1, s, w.total_t, w.total_s, w.total_exact, capacity, count_dev);
-        note_launches(2);
+        note_launches(1);
         return launch_status();
     }
-    const int sbits = ceil_log2(sg.ns);
-    const int npass = sbits <= 0 ? 0 : (sbits <= kMaxRadixBits ? 1 : (sbits + 7) / 8);
-    uint32_t *sk[2] = {w.skeys[0], w.skeys[1]};
-    uint32_t *sv[2] = {w.svals1, vals};  // the sorted list must end in svals1: vals is written from it
-    const int start = npass % 2;
-    launch_chained(k_emit_super, nbS, kScanBlock, s, splats, w.cull, w.vals[cur], w.n_vis, dc, sg.supers_x, w.part_s,
-                   w.total_s, capacity, sk[start], sv[start], w.total_exact);
-    note_launches(1);
-    // one pass: its digit ranges are the segments, written by the pass itself
-    const SegPlan sp{w.chunk_base, w.chunk_rec, ns, kChunk};
-    // ends in skeys[0] / svals1
-    radix_sort(sk, sv, start, w.sclip, capacity, sbits, w, s, npass == 1 ? sp : SegPlan{});
+    // One pass (up to 512 super-tiles): its digit ranges are the segments, written
+    // by the pass itself. Two: the second leaves the keys, which mark them.
+    for (int p = 0; p < npass; ++p) {
+        const bool last = p == npass - 1;
+        const Digit dg = radix_digit(w.hist_s, capacity, sbits, p);
+        launch_radix(dg.bits, capacity, s, w.entries[p], w.entries[1], last && npass == 2 ? w.skeys : nullptr,
+                     last ? w.svals : nullptr, w.sclip, dg, radix_digit(w.hist_s, capacity, sbits, p + 1),
+                     static_cast<DepthSpan *>(nullptr), 0, size_t(0),
+                     npass == 1 ? SegPlan{w.chunk_base, w.chunk_rec, ns, kChunk} : SegPlan{});
+        note_launches(1);
+    }
     // stage 3: per-tile lists
     const int64_t chunks = max_chunks(capacity, sg.ns), resident = resident_blocks();
     const unsigned cgrid = (unsigned)(chunks < resident ? chunks : resident);
     if (npass != 1) {
-        launch_chained(k_seg_mark, (unsigned)resident, 256, s, w.skeys[0], w.sclip, w.seg_lo, w.seg_hi);
+        launch_chained(k_seg_mark, (unsigned)resident, 256, s, w.skeys, w.sclip, w.seg_lo, w.seg_hi);
         launch_chained(k_super_plan, 1, 1024, s, w.seg_lo, w.seg_hi, ns, w.chunk_base, w.chunk_rec);
         note_launches(2);
     }
-    launch_chained(k_chunk_counts, cgrid, kChunk, s, splats, w.cull, w.svals1, w.chunk_base, w.chunk_rec, ns,
+    launch_chained(k_chunk_counts, cgrid, kChunk, s, splats, w.cull, w.svals, w.chunk_base, w.chunk_rec, ns,
                    sg.supers_x, dc, w.chunk_counts, w.tile_count, w.masks);
     const int tb = (int)((tiles + kScanBlock - 1) / kScanBlock);
-    launch_chained(k_tile_sums, tb, kScanBlock, s, w.tile_count, tiles, w.tile_part);
-    launch_chained(k_scan_parts<unsigned long long>, 1, 1024, s, w.tile_part, tb, w.total_t, nullptr, 0);
-    launch_chained(k_tile_starts, tb, kScanBlock, s, w.tile_count, tiles, w.tile_part, capacity, w.total_t, w.total_s,
-                   w.total_exact, w.tile_start, ranges, count_dev);
-    note_launches(2);
-    launch_chained(k_expand, cgrid, kChunk, s, splats, w.svals1, w.chunk_base, w.chunk_rec, ns, sg.supers_x, dc,
+    const bool direct = tb <= kDirectTiles;
+    if (!direct) {
+        launch_chained(k_tile_sums, tb, kScanBlock, s, w.tile_count, tiles, w.tile_part);
+        note_launches(1);
+    }
+    launch_chained(k_tile_starts, tb, kScanBlock, s, w.tile_count, tiles, direct ? nullptr : w.tile_part, capacity,
+                   w.total_s, w.total_exact, w.tile_start, ranges, count_dev);
+    launch_chained(k_expand, cgrid, kChunk, s, splats, w.svals, w.chunk_base, w.chunk_rec, ns, sg.supers_x, dc,
                    w.chunk_counts, w.tile_start, capacity, w.masks, vals);
-    note_launches(3);
+    note_launches(3);  // chunk counts, tile starts, lists
     return launch_status();
 }
