@@ -501,6 +501,34 @@ __device__ __forceinline__ bool tile_hit(const SplatShape &sh, int tile, int x, 
     return false;
 }
 
+// tile_hit by the edges that face the mean alone: for a mean outside the box the
+// least q over the box lies on one of them, so the other edges can pass only
+// where rounding decides. `none` is a bound above tau beyond which it cannot:
+// 1.01 tau for kappa <= 1e4 (as in cand_rect: q is off by at most 0.24%, the
+// clamped minimiser's own rounding by less), infinite for worse conics; q
+// between tau and `none` goes through all four edges. The same decision as
+// tile_hit, in two evaluations of q instead of four.
+__device__ __forceinline__ bool tile_hit_facing(const SplatShape &sh, float none, int tile, int x, int y) {
+    const float x0 = (float)(x * tile), x1 = (float)(x * tile + tile - 1);
+    const float y0 = (float)(y * tile), y1 = (float)(y * tile + tile - 1);
+    const bool out_x = !(sh.mx >= x0 && sh.mx <= x1), out_y = !(sh.my >= y0 && sh.my <= y1);
+    if (sh.tau < 0.f) return false;
+    if (!out_x && !out_y) return true;
+    const float dx = __fsub_rn(sh.mx > x1 ? x1 : x0, sh.mx);
+    const float yo = __fsub_rn(sh.my, __fmul_rn(sh.bc, dx));
+    const float yy = yo < y0 ? y0 : (yo > y1 ? y1 : yo);
+    const float q1 = quad_f32(sh.a, sh.b, sh.c, dx, __fsub_rn(yy, sh.my));
+    const float dy = __fsub_rn(sh.my > y1 ? y1 : y0, sh.my);
+    const float xo = __fsub_rn(sh.mx, __fmul_rn(sh.ba, dy));
+    const float xx = xo < x0 ? x0 : (xo > x1 ? x1 : xo);
+    const float q2 = quad_f32(sh.a, sh.b, sh.c, __fsub_rn(xx, sh.mx), dy);
+    // a non-facing edge's q is one of the four as well: a pass is a pass
+    if (q1 <= sh.tau || q2 <= sh.tau) return true;
+    const float q = out_x ? (out_y ? fminf(q1, q2) : q1) : q2;
+    if (q > none) return false;
+    return tile_hit(sh, tile, x, y);
+}
+
 // The tiles a splat may be listed in: its 3-sigma rectangle, narrowed to the
 // bounding box of the ellipse q <= tau when that box is provably wide
 // enough. tile_hit evaluates q = a dx^2 + 2 b dx dy + c dy^2 (float32) only
@@ -513,7 +541,8 @@ __device__ __forceinline__ bool tile_hit(const SplatShape &sh, int tile, int x, 
 // widths leaves (plus a pixel). Ill-conditioned conics keep the rectangle.
 // So every tile dropped here fails tile_hit: the lists are unchanged.
 __device__ __forceinline__ int cand_rect(const float *splats, uint32_t g, const DevCam &cam, float tau, int &x0,
-                                         int &y0, int &x1, int &y1) {
+                                         int &y0, int &x1, int &y1, float *none = nullptr) {
+    if (none) *none = __int_as_float(0x7f800000);  // no bound (see tile_hit_facing) for ill-conditioned conics
     if (!splat_rect(splats, g, cam, x0, y0, x1, y1)) return 0;
     const float *r = splats + (int64_t)g * kSplat;
     const float mx = __ldg(r), my = __ldg(r + 1), a = __ldg(r + 2), b = __ldg(r + 3), c = __ldg(r + 4);
@@ -521,6 +550,7 @@ __device__ __forceinline__ int cand_rect(const float *splats, uint32_t g, const 
     if (!(tau >= 0.f) || !(det > 0.f) || !(a > 0.f) || !(c > 0.f)) return 1;
     const float kappa = (a + fabsf(b) + c) * (a + c) / det;
     if (!(kappa <= 1e4f)) return 1;
+    if (none) *none = 1.01f * tau;
     const float hx = sqrtf(tau * c / det) * 1.02f + 1.f;
     const float hy = sqrtf(tau * a / det) * 1.02f + 1.f;
     const float inv = 1.f / (float)cam.tile;  // exact: a power of two
@@ -538,13 +568,14 @@ __device__ __forceinline__ int cand_rect(const float *splats, uint32_t g, const 
 // The tile tests' constants and the candidate rectangle of a visible
 // Gaussian, computed once per sort (k_emit_visible) and read by the
 // depth-ordered passes and the chunk kernels: cull[2 g] = (tau, b / c, b / a,
-// 0), cull[2 g + 1] = (x0 | y0 << 16, x1 | y1 << 16, 0, 0) as integers, the
+// the bound of tile_hit_facing), cull[2 g + 1] = (x0 | y0 << 16, x1 | y1 << 16, 0, 0) as integers, the
 // empty rectangle when no tile can list the splat (255 o < 1).
 __device__ __forceinline__ void write_cull(const float *splats, uint32_t g, const DevCam &cam, float4 *cull) {
     const SplatShape sh = splat_shape(splats, g);
     int x0 = 0, y0 = 0, x1 = 0, y1 = 0;
-    if (!(sh.tau >= 0.f) || !cand_rect(splats, g, cam, sh.tau, x0, y0, x1, y1)) x0 = y0 = x1 = y1 = 0;
-    cull[2 * (int64_t)g] = make_float4(sh.tau, sh.bc, sh.ba, 0.f);
+    float none = 0.f;
+    if (!(sh.tau >= 0.f) || !cand_rect(splats, g, cam, sh.tau, x0, y0, x1, y1, &none)) x0 = y0 = x1 = y1 = 0;
+    cull[2 * (int64_t)g] = make_float4(sh.tau, sh.bc, sh.ba, none);
     reinterpret_cast<uint4 *>(cull)[2 * (int64_t)g + 1] =
         make_uint4((uint32_t)x0 | ((uint32_t)y0 << 16), (uint32_t)x1 | ((uint32_t)y1 << 16), 0u, 0u);
 }
@@ -853,12 +884,17 @@ struct ChunkCtx {
 };
 
 // Scratch of the tile tests (shared memory, one slot per thread): hit
-// masks as two 32-bit halves, the entry's shape and its candidate
-// rectangle packed as lx0 | ly0 << 3 | w << 6 | ceil(512 / w) << 10.
+// masks as two 32-bit halves, the entry's shape, the bound of
+// tile_hit_facing, and its candidate rectangle packed as lx0 | ly0 << 3 |
+// w << 6 | ceil(512 / w) << 10 | first candidate << 20; per warp the bits
+// of the first candidates (2048 of them at most) and the entries that have any.
 struct TestScratch {
-    uint32_t *hit;  // [2 * kChunk]
-    float4 *shape;  // [2 * kChunk]
-    uint32_t *rect; // [kChunk]
+    uint32_t *hit;   // [2 * kChunk]
+    float4 *shape;   // [2 * kChunk]
+    float *none;     // [kChunk]
+    uint32_t *rect;  // [kChunk]
+    uint32_t *starts;  // [kChunk / 32][64]
+    uint8_t *owner;    // [kChunk]
 };
 
 // With masks_in NULL the masks are computed by the tile test (and stored to
@@ -889,6 +925,7 @@ __device__ __forceinline__ void chunk_load(ChunkCtx &cx, uint32_t c, const float
     // tiles from (lx0, ly0) in the super-tile's own tile coordinates
     int lx0 = 0, ly0 = 0, w = 0, h = 0;
     SplatShape sh{};
+    float none = 0.f;
     int x0, y0, x1, y1;
     if (valid) {  // every listed entry's splat has tau >= 0 and a candidate rectangle
         const float *r = splats + (int64_t)cx.g * kSplat;
@@ -897,6 +934,7 @@ __device__ __forceinline__ void chunk_load(ChunkCtx &cx, uint32_t c, const float
         sh.mx = p0.x; sh.my = p0.y; sh.a = p0.z; sh.b = p0.w;
         sh.c = __ldg(r + 4);
         sh.tau = c0.x; sh.bc = c0.y; sh.ba = c0.z;
+        none = c0.w;
         if (cull_rect(cull, cx.g, x0, y0, x1, y1)) {
             lx0 = max(x0 - cx.sx * kSuper, 0);
             ly0 = max(y0 - cx.sy * kSuper, 0);
@@ -907,10 +945,12 @@ __device__ __forceinline__ void chunk_load(ChunkCtx &cx, uint32_t c, const float
     const int cnt = w * h;
     sc.shape[2 * threadIdx.x] = make_float4(sh.mx, sh.my, sh.a, sh.b);
     sc.shape[2 * threadIdx.x + 1] = make_float4(sh.c, sh.tau, sh.bc, sh.ba);
-    // k / w = (k * ceil(512 / w)) >> 9 exactly for k < 64, w <= 8
-    sc.rect[threadIdx.x] = cnt ? (uint32_t)(lx0 | (ly0 << 3) | (w << 6) | (((512 + w - 1) / w) << 10)) : 0u;
+    sc.none[threadIdx.x] = none;
     sc.hit[2 * threadIdx.x] = 0u;
     sc.hit[2 * threadIdx.x + 1] = 0u;
+    uint32_t *starts = sc.starts + warp * 64;
+    uint8_t *owner = sc.owner + warp * 32;
+    starts[lane] = starts[lane + 32] = 0u;
     // the warp's (entry, tile) candidates, spread evenly over its lanes
     int incl = cnt;
 #pragma unroll
@@ -919,27 +959,35 @@ __device__ __forceinline__ void chunk_load(ChunkCtx &cx, uint32_t c, const float
         if (lane >= o) incl += y;
     }
     const int excl = incl - cnt, total = __shfl_sync(kFull, incl, 31);
+    const unsigned some = __ballot_sync(kFull, cnt > 0);
     __syncwarp();
+    if (cnt) {
+        // k / w = (k * ceil(512 / w)) >> 9 exactly for k < 64, w <= 8
+        sc.rect[threadIdx.x] =
+            (uint32_t)(lx0 | (ly0 << 3) | (w << 6) | (((512 + w - 1) / w) << 10)) | ((uint32_t)excl << 20);
+        owner[__popc(some & lanemask_lt())] = (uint8_t)lane;
+        atomicOr(starts + (excl >> 5), 1u << (excl & 31));
+    }
+    __syncwarp();
+    int passed = -1;  // entries that begin before this round, less one
     for (int base = 0; base < total; base += 32) {
+        // candidate j belongs to the last entry that begins at or before it
         const int j = base + lane;
-        int i = 0;  // owner: the last lane whose first candidate index is <= j
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-            const int ex = __shfl_sync(kFull, excl, i + step);
-            if (ex <= j) i += step;
-        }
-        const int k = j - __shfl_sync(kFull, excl, i);
+        const uint32_t word = starts[base >> 5];
+        const int i = owner[min(31, passed + __popc(word & (kFull >> (31 - lane))))];
+        passed += __popc(word);
         if (j < total) {
             const int o = warp * 32 + i;
             const uint32_t pk = sc.rect[o];
+            const int k = j - (int)(pk >> 20);
             const int ow = (int)((pk >> 6) & 15u);
-            const int q = (k * (int)(pk >> 10)) >> 9, r = k - q * ow;
+            const int q = (k * (int)((pk >> 10) & 1023u)) >> 9, r = k - q * ow;
             const int t = ((int)((pk >> 3) & 7u) + q) * kSuper + (int)(pk & 7u) + r;
             const float4 s0 = sc.shape[2 * o], s1 = sc.shape[2 * o + 1];
             SplatShape os;
             os.mx = s0.x; os.my = s0.y; os.a = s0.z; os.b = s0.w;
             os.c = s1.x; os.tau = s1.y; os.bc = s1.z; os.ba = s1.w;
-            if (tile_hit(os, cam.tile, cx.sx * kSuper + (t & 7), cx.sy * kSuper + (t >> 3)))
+            if (tile_hit_facing(os, sc.none[o], cam.tile, cx.sx * kSuper + (t & 7), cx.sy * kSuper + (t >> 3)))
                 atomicOr(&sc.hit[2 * o + (t >> 5)], 1u << (t & 31));  // native 32-bit
         }
     }
@@ -973,6 +1021,10 @@ __device__ __forceinline__ int slot_tile(int t, int sx, int sy, int tiles_x) {
     return (sy * kSuper + (t >> 3)) * tiles_x + sx * kSuper + (t & 7);
 }
 
+// Bound by instruction issue: about 12 candidate tiles per entry, 85
+// instructions per 32 of them (1M Gaussians, 931K entries: 66 -> 61 us with the
+// two-edge test and the owner of a candidate found by a population count
+// instead of a search over the lanes).
 __global__ void __launch_bounds__(kChunk) k_chunk_counts(const float *__restrict__ splats,
                                                         const float4 *__restrict__ cull,
                                                         const uint32_t *__restrict__ svals,
@@ -985,8 +1037,11 @@ __global__ void __launch_bounds__(kChunk) k_chunk_counts(const float *__restrict
     __shared__ uint32_t hit_mask[2 * kChunk];  // per entry, low and high halves
     __shared__ float4 shape[2 * kChunk];
     __shared__ uint32_t rect[kChunk];
+    __shared__ float none[kChunk];
+    __shared__ uint32_t starts[kChunk / 32][64];
+    __shared__ uint8_t owner[kChunk];
     __shared__ uint32_t cnt[kChunk / 32][64];  // per warp and slot: the warp's entries that the slot's tile lists
-    const TestScratch sc{hit_mask, shape, rect};
+    const TestScratch sc{hit_mask, shape, none, rect, &starts[0][0], owner};
     const uint32_t nc = chunk_base[ns];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
@@ -1065,6 +1120,9 @@ __global__ void __launch_bounds__(kScanBlock) k_tile_starts(const uint32_t *__re
     }
 }
 
+// Bound by instruction issue; a slot's place and its lanes are one 8-byte word
+// in shared memory and positions have 32 bits (40 -> 30 us at 931K entries,
+// 4.8M places).
 __global__ void __launch_bounds__(kChunk) k_expand(const float *__restrict__ splats, const uint32_t *__restrict__ svals,
                                                   const uint32_t *__restrict__ chunk_base,
                                                   const uint4 *__restrict__ chunk_rec, int ns, int supers_x,
@@ -1074,18 +1132,19 @@ __global__ void __launch_bounds__(kChunk) k_expand(const float *__restrict__ spl
                                                   uint32_t *__restrict__ vals) {
     wait_prior_grid();
     constexpr int kW = kChunk / 32;
-    __shared__ uint32_t ballots[kW][64];                 // per (warp, slot): lanes whose entry the tile lists
+    // per (warp, slot): where the warp's entries of the slot's tile start in the
+    // final list (clipped to the capacity), and the lanes whose entry it lists
+    __shared__ uint2 place[kW][64];
     __shared__ uint32_t before[kChunk / 64][64];         // partial sums of earlier chunks' counts
-    __shared__ unsigned long long base[kW][64];         // start of (warp, slot) in the final list
-    const uint32_t nc = chunk_base[ns];
+    const uint32_t nc = chunk_base[ns], cap = (uint32_t)capacity;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt = lanemask_lt();
     for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
         ChunkCtx cx;
         chunk_load(cx, c, splats, nullptr, svals, chunk_rec, supers_x, cam, TestScratch{}, masks, nullptr);
         const uint32_t lo = (uint32_t)cx.mask, hi = (uint32_t)(cx.mask >> 32);
-        ballots[warp][lane] = warp_transpose32(lo, lane);
-        ballots[warp][lane + 32] = warp_transpose32(hi, lane);
+        place[warp][lane].y = warp_transpose32(lo, lane);
+        place[warp][lane + 32].y = warp_transpose32(hi, lane);
         {   // entries of each slot in the super-tile's earlier chunks: 4 threads per slot,
             // four independent sums so that the loads overlap
             constexpr int kQ = kChunk / 64;
@@ -1111,10 +1170,11 @@ __global__ void __launch_bounds__(kChunk) k_expand(const float *__restrict__ spl
 #pragma unroll
                 for (int q = 0; q < kChunk / 64; ++q) run += before[q][t];
             }
+            uint32_t at = (uint32_t)(run < (unsigned long long)cap ? run : (unsigned long long)cap);
 #pragma unroll
-            for (int w = 0; w < kW; ++w) {
-                base[w][t] = run;
-                run += (unsigned long long)__popc(ballots[w][t]);
+            for (int w = 0; w < kW; ++w) {  // below 2^31 + 256 + ...: 32 bits hold it
+                place[w][t].x = at;
+                at += (uint32_t)__popc(place[w][t].y);
             }
         }
         __syncthreads();
@@ -1122,15 +1182,19 @@ __global__ void __launch_bounds__(kChunk) k_expand(const float *__restrict__ spl
         // lanes before it that tile t lists. Written slot by slot over the
         // slots some lane has (a warp's entries of one tile go to consecutive
         // words) or, when that takes more rounds, each lane over its own slots.
-        const unsigned long long any = ((unsigned long long)__reduce_or_sync(kFull, hi) << 32) |
-                                       __reduce_or_sync(kFull, lo);
-        const int by_slot = __popcll(any), by_lane = (int)__reduce_max_sync(kFull, (unsigned)__popcll(cx.mask));
-        for (unsigned long long u = by_lane < by_slot ? cx.mask : any; u; u &= u - 1ull) {
-            const int t = __ffsll((long long)u) - 1;
-            if ((cx.mask >> t) & 1ull) {
-                const unsigned long long pos =
-                    base[warp][t] + (unsigned long long)__popc(ballots[warp][t] & lt);
-                if (pos < (unsigned long long)capacity) vals[pos] = cx.g;
+        const unsigned any_lo = __reduce_or_sync(kFull, lo), any_hi = __reduce_or_sync(kFull, hi);
+        const int by_slot = __popc(any_lo) + __popc(any_hi);
+        const bool by_lane = (int)__reduce_max_sync(kFull, (unsigned)__popcll(cx.mask)) < by_slot;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const uint32_t mine = half ? hi : lo;
+            for (uint32_t u = by_lane ? mine : (half ? any_hi : any_lo); u; u &= u - 1u) {
+                const int t = __ffs((int)u) - 1;
+                if ((mine >> t) & 1u) {
+                    const uint2 p = place[warp][32 * half + t];
+                    const uint32_t pos = p.x + (uint32_t)__popc(p.y & lt);
+                    if (pos < cap) vals[pos] = cx.g;
+                }
             }
         }
     }
