@@ -4,11 +4,11 @@
 // SSIM uses the 11x11 Gaussian window (sigma 1.5) as two 1-D passes in
 // shared memory (Sec. 3.3, "Accelerated SSIM loss calculation"): one kernel
 // builds the five window moments of a 32x32 tile plus its 5-pixel halo and
-// emits the SSIM map's three partial-derivative maps; a second kernel runs
-// the same separable window over those maps (the window is symmetric, so it
-// is its own adjoint) and combines them with the L1 term into dL/dimage.
-// Block partial sums are reduced in a fixed order, so the loss is
-// deterministic.
+// emits the SSIM map's three partial-derivative maps (two of them as one array
+// of pairs); a second kernel runs the same separable window over those maps
+// (the window is symmetric, so it is its own adjoint) and combines them with
+// the L1 term into dL/dimage. Block partial sums are reduced in a fixed order,
+// so the loss is deterministic.
 #include "common.cuh"
 
 namespace gs {
@@ -29,22 +29,70 @@ struct Win {
 
 // Each pass gives a thread kV = 4 consecutive outputs, so that it reads the
 // kV + 10 inputs of their windows once from shared memory instead of
-// 11 per output. Horizontal items: (row of the haloed tile, 4 columns);
-// vertical items: (column, 4 rows), one per thread, a warp on 32 columns.
+// 11 per output. Horizontal items: (4 columns, row of the haloed tile), a warp
+// on 32 rows; vertical items: (column, 4 rows), one per thread, a warp on 32
+// columns.
+//
+// Quantities that share a weight go in pairs through the packed FP32
+// instructions -- (x, y) and (x^2, y^2) with x y beside them in the forward,
+// the first two maps with the third in the backward -- and lie interleaved in
+// shared memory, so that a load brings a ready pair and no instruction is
+// spent on packing. Every rounded operation is the scalar one's. Row strides
+// of the arrays are 4 words times an odd number: 16-byte accesses of eight
+// consecutive rows meet all 32 banks. The loss is reduced from the forward's
+// partial sums by the backward's first block, so that the forward counts no
+// blocks, fences nothing and no counter has to be cleared before it.
+//
+// Bound by instruction issue (66-71%) and, at its four blocks per SM, by the
+// two barriers between the passes. 3 x 822 x 1237: 68.4 us with scalar passes, a
+// counted last block and a cleared counter; 61.8 us with packed passes; 50.0 us
+// with the reduction in the backward.
 constexpr int kV = 4;
 constexpr int kSeg = kT / kV;              // 8 segments per row / column
 constexpr int kHItems = kE * kSeg;         // 336 horizontal items
+constexpr int kH2 = kT + 2;                // pairs per row of the horizontal sums (68 words)
+constexpr int kH1 = kT + 4;                // words per row of the third one (36)
+constexpr int kE1 = kE + 2;                // words per row of a haloed single map (44); pairs need no padding (84)
 static_assert(kT * kSeg == kLossThreads, "one vertical item per thread");
 
-// The loss from the per-block partial sums (L1 sum, SSIM sum), by the last
-// block to finish: every thread sums a fixed stride of them in double, then a
-// fixed-shape tree, so the result does not depend on the block order.
+// Window sums of kV outputs from kV + 10 inputs, N packed quantities and one
+// scalar: in(q, pairs, scalar) gives input q.
+template <int N, class In>
+__device__ __forceinline__ void window(const Win &win, In in, f32x2 (&p)[N][kV], float (&s)[kV]) {
+#pragma unroll
+    for (int v = 0; v < kV; ++v) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) p[k][v] = f2_pack(0.f, 0.f);
+        s[v] = 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < kV + 10; ++q) {
+        f32x2 x[N];
+        float z;
+        in(q, x, z);
+#pragma unroll
+        for (int v = 0; v < kV; ++v) {
+            const int t = q - v;  // tap of input q in output v's window
+            if (t >= 0 && t < 11) {
+                const float w = win.w[t];
+                const f32x2 w2 = f2_pack(w, w);
+#pragma unroll
+                for (int k = 0; k < N; ++k) p[k][v] = f2_fma(w2, x[k], p[k][v]);
+                s[v] = __fmaf_rn(w, z, s[v]);
+            }
+        }
+    }
+}
+
+// The loss from the forward's per-block partial sums (L1 sum, SSIM sum), by the
+// backward's first block: every thread sums a fixed stride of them in double,
+// then a fixed-shape tree.
 __device__ void loss_from_parts(const float2 *part, int nparts, int64_t N, float lambda, float *loss,
                                 double *scratch /* shared, 2 * kLossThreads */) {
     double *r1 = scratch, *r2 = scratch + kLossThreads;
     double a = 0.0, b = 0.0;
     for (int k = threadIdx.x; k < nparts; k += kLossThreads) {
-        const float2 v = __ldcg(part + k);
+        const float2 v = part[k];
         a += (double)v.x;
         b += (double)v.y;
     }
@@ -68,15 +116,12 @@ __device__ void loss_from_parts(const float2 *part, int nparts, int64_t N, float
 
 __global__ void __launch_bounds__(kLossThreads) k_ssim_fwd(const float *__restrict__ img,
                                                           const float *__restrict__ gt, int H, int W, Win win,
-                                                          float *__restrict__ mapA, float *__restrict__ mapB,
-                                                          float *__restrict__ mapC, float2 *__restrict__ part,
-                                                          unsigned int *__restrict__ done, float lambda,
-                                                          float *__restrict__ loss) {
-    __shared__ float sx[kE][kE + 1], sy[kE][kE + 1];
-    __shared__ __align__(16) float h[5][kE][kT + 1];  // also the last block's reduction scratch
+                                                          f32x2 *__restrict__ mapAB, float *__restrict__ mapC,
+                                                          float2 *__restrict__ part) {
+    __shared__ __align__(16) f32x2 sxy[kE][kE];
+    __shared__ __align__(16) f32x2 h[2][kE][kH2];
+    __shared__ __align__(16) float hxy[kE][kH1];
     __shared__ float red[2][kLossThreads / 32];
-    __shared__ bool last;
-    static_assert(sizeof(h) >= 2 * kLossThreads * sizeof(double), "scratch fits");
     wait_prior_grid();
     const int ch = blockIdx.z;
     const int64_t HW = (int64_t)H * W;
@@ -92,36 +137,37 @@ __global__ void __launch_bounds__(kLossThreads) k_ssim_fwd(const float *__restri
                 const int gy = oy + r;
                 const bool in = col_in && gy >= 0 && gy < H;
                 const int64_t o = (int64_t)gy * W + gx;
-                sx[r][c] = in ? __ldg(x + o) : 0.f;
-                sy[r][c] = in ? __ldg(y + o) : 0.f;
+                sxy[r][c] = f2_pack(in ? __ldg(x + o) : 0.f, in ? __ldg(y + o) : 0.f);
             }
         }
     }
     __syncthreads();
-    // horizontal: window sums of x, y, x^2, y^2, x y along the rows
+    // horizontal: window sums of (x, y), (x^2, y^2), x y along the rows
     for (int it = threadIdx.x; it < kHItems; it += kLossThreads) {
-        const int r = it / kSeg, c0 = (it % kSeg) * kV;
-        float a[kV], b[kV], aa[kV], bb[kV], ab[kV];
+        const int r = it % kE, c0 = (it / kE) * kV;
+        f32x2 in2[kV + 10];
 #pragma unroll
-        for (int v = 0; v < kV; ++v) a[v] = b[v] = aa[v] = bb[v] = ab[v] = 0.f;
-#pragma unroll
-        for (int q = 0; q < kV + 10; ++q) {
-            const float xv = sx[r][c0 + q], yv = sy[r][c0 + q];
-            const float xx = xv * xv, yy = yv * yv, xy = xv * yv;
-#pragma unroll
-            for (int v = 0; v < kV; ++v) {
-                const int t = q - v;  // tap of input q in output v's window
-                if (t >= 0 && t < 11) {
-                    const float w = win.w[t];
-                    a[v] += w * xv; b[v] += w * yv; aa[v] += w * xx; bb[v] += w * yy; ab[v] += w * xy;
-                }
-            }
+        for (int q = 0; q < kV + 10; q += 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&sxy[r][c0 + q]);
+            in2[q] = v.x;
+            in2[q + 1] = v.y;
         }
+        f32x2 p[2][kV];
+        float s[kV];
+        window<2>(win, [&](int q, f32x2 (&o)[2], float &z) {
+            float xv, yv;
+            f2_unpack(in2[q], xv, yv);
+            o[0] = in2[q];
+            o[1] = f2_mul(in2[q], in2[q]);
+            z = xv * yv;
+        }, p, s);
 #pragma unroll
-        for (int v = 0; v < kV; ++v) {
-            h[0][r][c0 + v] = a[v]; h[1][r][c0 + v] = b[v]; h[2][r][c0 + v] = aa[v];
-            h[3][r][c0 + v] = bb[v]; h[4][r][c0 + v] = ab[v];
+        for (int k = 0; k < 2; ++k) {
+#pragma unroll
+            for (int v = 0; v < kV; v += 2)
+                *reinterpret_cast<ulonglong2 *>(&h[k][r][c0 + v]) = make_ulonglong2(p[k][v], p[k][v + 1]);
         }
+        *reinterpret_cast<float4 *>(&hxy[r][c0]) = make_float4(s[0], s[1], s[2], s[3]);
     }
     __syncthreads();
     // vertical, then the SSIM map and its partial derivatives
@@ -129,30 +175,25 @@ __global__ void __launch_bounds__(kLossThreads) k_ssim_fwd(const float *__restri
     float l1 = 0.f, ss = 0.f;
     {
         const int c = threadIdx.x % kT, r0 = (threadIdx.x / kT) * kV;
-        float mx[kV], my[kV], xx[kV], yy[kV], xy[kV];
-#pragma unroll
-        for (int v = 0; v < kV; ++v) mx[v] = my[v] = xx[v] = yy[v] = xy[v] = 0.f;
-#pragma unroll
-        for (int q = 0; q < kV + 10; ++q) {
-            const float h0 = h[0][r0 + q][c], h1 = h[1][r0 + q][c], h2 = h[2][r0 + q][c];
-            const float h3 = h[3][r0 + q][c], h4 = h[4][r0 + q][c];
-#pragma unroll
-            for (int v = 0; v < kV; ++v) {
-                const int t = q - v;
-                if (t >= 0 && t < 11) {
-                    const float w = win.w[t];
-                    mx[v] += w * h0; my[v] += w * h1; xx[v] += w * h2; yy[v] += w * h3; xy[v] += w * h4;
-                }
-            }
-        }
+        f32x2 p[2][kV];
+        float xy[kV];
+        window<2>(win, [&](int q, f32x2 (&o)[2], float &z) {
+            o[0] = h[0][r0 + q][c];
+            o[1] = h[1][r0 + q][c];
+            z = hxy[r0 + q][c];
+        }, p, xy);
 #pragma unroll
         for (int v = 0; v < kV; ++v) {
             const int r = r0 + v;
             const int gy = blockIdx.y * kT + r, gx = blockIdx.x * kT + c;
             if (gy >= H || gx >= W) continue;
-            const float vx = xx[v] - mx[v] * mx[v], vy = yy[v] - my[v] * my[v], cxy = xy[v] - mx[v] * my[v];
-            const float n1 = 2.f * mx[v] * my[v] + C1, n2 = 2.f * cxy + C2;
-            const float d1 = mx[v] * mx[v] + my[v] * my[v] + C1, d2 = vx + vy + C2;
+            float mx, my, xx, yy, xc, yc;
+            f2_unpack(p[0][v], mx, my);
+            f2_unpack(p[1][v], xx, yy);
+            f2_unpack(sxy[r + kR][c + kR], xc, yc);
+            const float vx = xx - mx * mx, vy = yy - my * my, cxy = xy[v] - mx * my;
+            const float n1 = 2.f * mx * my + C1, n2 = 2.f * cxy + C2;
+            const float d1 = mx * mx + my * my + C1, d2 = vx + vy + C2;
             // d1 >= C1 and d2 >= C2 (up to rounding of the variances): the map
             // and its partials are formed without dividing by n1 or n2, which
             // may be zero (m / n2 = n1 / (d1 d2), m / n1 = n2 / (d1 d2))
@@ -161,12 +202,11 @@ __global__ void __launch_bounds__(kLossThreads) k_ssim_fwd(const float *__restri
             const float m_n1 = n2 * qd, m_n2 = n1 * qd;
             const float m = n1 * m_n1;
             ss += m;
-            l1 += fabsf(sx[r + kR][c + kR] - sy[r + kR][c + kR]);
+            l1 += fabsf(xc - yc);
             // partials of the map value w.r.t. the window means of x, x^2 and x*y
-            const int64_t p = ch * HW + (int64_t)gy * W + gx;
-            mapA[p] = 2.f * my[v] * (m_n1 - m_n2) + 2.f * mx[v] * m * (rd2 - rd1);
-            mapB[p] = -m * rd2;
-            mapC[p] = 2.f * m_n2;
+            const int64_t o = ch * HW + (int64_t)gy * W + gx;
+            mapAB[o] = f2_pack(2.f * my * (m_n1 - m_n2) + 2.f * mx * m * (rd2 - rd1), -m * rd2);
+            mapC[o] = 2.f * m_n2;
         }
     }
     // block sums
@@ -177,34 +217,34 @@ __global__ void __launch_bounds__(kLossThreads) k_ssim_fwd(const float *__restri
     }
     if ((threadIdx.x & 31) == 0) { red[0][threadIdx.x >> 5] = l1; red[1][threadIdx.x >> 5] = ss; }
     __syncthreads();
-    const unsigned int nblk = gridDim.x * gridDim.y * gridDim.z;
     if (threadIdx.x == 0) {
         float a = 0.f, b = 0.f;
         for (int w = 0; w < kLossThreads / 32; ++w) { a += red[0][w]; b += red[1][w]; }
         int64_t blk = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
         part[blk] = make_float2(a, b);
-        __threadfence();  // the partial is visible before this block is counted
-        last = atomicAdd(done, 1u) == nblk - 1;
-    }
-    __syncthreads();
-    if (last) {
-        __threadfence();
-        loss_from_parts(part, (int)nblk, 3 * HW, lambda, loss, reinterpret_cast<double *>(&h[0][0][0]));
     }
 }
 
 __global__ void __launch_bounds__(kLossThreads, 5) k_ssim_bwd(const float *__restrict__ img,
                                                           const float *__restrict__ gt, int H, int W, Win win,
-                                                          float lambda, const float *__restrict__ mapA,
-                                                          const float *__restrict__ mapB,
-                                                          const float *__restrict__ mapC, float *__restrict__ dl) {
-    __shared__ float sm[3][kE][kE + 1];
-    __shared__ float h[3][kE][kT + 1];
+                                                          float lambda, const f32x2 *__restrict__ mapAB,
+                                                          const float *__restrict__ mapC,
+                                                          const float2 *__restrict__ part, float *__restrict__ loss,
+                                                          float *__restrict__ dl) {
+    __shared__ __align__(16) f32x2 sab[kE][kE];
+    __shared__ __align__(16) float sc[kE][kE1];
+    __shared__ __align__(16) f32x2 h[kE][kH2];  // also the first block's reduction scratch
+    __shared__ __align__(16) float hc[kE][kH1];
+    static_assert(sizeof(h) >= 2 * kLossThreads * sizeof(double), "scratch fits");
     wait_prior_grid();
     const int ch = blockIdx.z;
     const int64_t HW = (int64_t)H * W;
+    if (blockIdx.x + blockIdx.y + blockIdx.z == 0)  // h is written again behind the next barrier
+        loss_from_parts(part, (int)(gridDim.x * gridDim.y * gridDim.z), 3 * HW, lambda, loss,
+                        reinterpret_cast<double *>(&h[0][0]));
     const int oy = blockIdx.y * kT - kR, ox = blockIdx.x * kT - kR;
-    const float *a = mapA + ch * HW, *b = mapB + ch * HW, *c = mapC + ch * HW;
+    const f32x2 *ab = mapAB + ch * HW;
+    const float *c = mapC + ch * HW;
     {
         const int q = (int)threadIdx.x % kE, r0 = (int)threadIdx.x / kE;
         const int gx = ox + q;
@@ -215,51 +255,41 @@ __global__ void __launch_bounds__(kLossThreads, 5) k_ssim_bwd(const float *__res
                 const int gy = oy + r;
                 const bool in = col_in && gy >= 0 && gy < H;
                 const int64_t o = (int64_t)gy * W + gx;
-                sm[0][r][q] = in ? __ldg(a + o) : 0.f;
-                sm[1][r][q] = in ? __ldg(b + o) : 0.f;
-                sm[2][r][q] = in ? __ldg(c + o) : 0.f;
+                sab[r][q] = in ? __ldg(ab + o) : 0ull;
+                sc[r][q] = in ? __ldg(c + o) : 0.f;
             }
         }
     }
     __syncthreads();
     for (int it = threadIdx.x; it < kHItems; it += kLossThreads) {
-        const int r = it / kSeg, c0 = (it % kSeg) * kV;
-        float s0[kV], s1[kV], s2[kV];
+        const int r = it % kE, c0 = (it / kE) * kV;
+        f32x2 p[1][kV], in2[kV + 10];
+        float s[kV], in1[kV + 12];
 #pragma unroll
-        for (int v = 0; v < kV; ++v) s0[v] = s1[v] = s2[v] = 0.f;
-#pragma unroll
-        for (int q = 0; q < kV + 10; ++q) {
-            const float m0 = sm[0][r][c0 + q], m1 = sm[1][r][c0 + q], m2 = sm[2][r][c0 + q];
-#pragma unroll
-            for (int v = 0; v < kV; ++v) {
-                const int t = q - v;
-                if (t >= 0 && t < 11) {
-                    const float w = win.w[t];
-                    s0[v] += w * m0; s1[v] += w * m1; s2[v] += w * m2;
-                }
-            }
+        for (int q = 0; q < kV + 10; q += 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&sab[r][c0 + q]);
+            in2[q] = v.x;
+            in2[q + 1] = v.y;
         }
 #pragma unroll
-        for (int v = 0; v < kV; ++v) { h[0][r][c0 + v] = s0[v]; h[1][r][c0 + v] = s1[v]; h[2][r][c0 + v] = s2[v]; }
+        for (int q = 0; q < kV + 10; q += 4) {  // the last two words are the row's padding
+            const float4 v = *reinterpret_cast<const float4 *>(&sc[r][c0 + q]);
+            in1[q] = v.x; in1[q + 1] = v.y; in1[q + 2] = v.z; in1[q + 3] = v.w;
+        }
+        window<1>(win, [&](int q, f32x2 (&o)[1], float &z) { o[0] = in2[q]; z = in1[q]; }, p, s);
+#pragma unroll
+        for (int v = 0; v < kV; v += 2)
+            *reinterpret_cast<ulonglong2 *>(&h[r][c0 + v]) = make_ulonglong2(p[0][v], p[0][v + 1]);
+        *reinterpret_cast<float4 *>(&hc[r][c0]) = make_float4(s[0], s[1], s[2], s[3]);
     }
     __syncthreads();
     const float invN = 1.f / (3.f * (float)HW);
     const int cc = threadIdx.x % kT, r0 = (threadIdx.x / kT) * kV;
+    f32x2 p[1][kV];
     float s0[kV], s1[kV], s2[kV];
+    window<1>(win, [&](int q, f32x2 (&o)[1], float &z) { o[0] = h[r0 + q][cc]; z = hc[r0 + q][cc]; }, p, s2);
 #pragma unroll
-    for (int v = 0; v < kV; ++v) s0[v] = s1[v] = s2[v] = 0.f;
-#pragma unroll
-    for (int q = 0; q < kV + 10; ++q) {
-        const float h0 = h[0][r0 + q][cc], h1 = h[1][r0 + q][cc], h2 = h[2][r0 + q][cc];
-#pragma unroll
-        for (int v = 0; v < kV; ++v) {
-            const int t = q - v;
-            if (t >= 0 && t < 11) {
-                const float w = win.w[t];
-                s0[v] += w * h0; s1[v] += w * h1; s2[v] += w * h2;
-            }
-        }
-    }
+    for (int v = 0; v < kV; ++v) f2_unpack(p[0][v], s0[v], s1[v]);
 #pragma unroll
     for (int v = 0; v < kV; ++v) {
         const int gy = blockIdx.y * kT + r0 + v, gx = blockIdx.x * kT + cc;
@@ -362,17 +392,14 @@ extern "C" int gs_loss(const float *image, const float *gt, int32_t H, int32_t W
     if (ws_bytes < gs_loss_workspace_bytes(H, W) || (reinterpret_cast<uintptr_t>(ws) & 255)) return GS_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
     const int64_t HW = (int64_t)H * W;
-    float *mapA = static_cast<float *>(ws);
-    float *mapB = mapA + 3 * HW, *mapC = mapB + 3 * HW;
+    f32x2 *mapAB = static_cast<f32x2 *>(ws);
+    float *mapC = reinterpret_cast<float *>(mapAB + 3 * HW);
     float2 *part = reinterpret_cast<float2 *>(static_cast<char *>(ws) + align256(9 * (size_t)HW * sizeof(float)));
     LossGrid g = loss_grid(H, W);
-    unsigned int *done = reinterpret_cast<unsigned int *>(reinterpret_cast<char *>(part) +
-                                                          align256(sizeof(float2) * (size_t)g.nparts));
     Win win = make_window();
-    if (cudaMemsetAsync(done, 0, sizeof(unsigned int), s) != cudaSuccess) return GS_ERR_CUDA;
-    launch_chained(k_ssim_fwd, g.grid, kLossThreads, s, image, gt, H, W, win, mapA, mapB, mapC, part, done, lambda,
-                   loss_dev);
-    launch_chained(k_ssim_bwd, g.grid, kLossThreads, s, image, gt, H, W, win, lambda, mapA, mapB, mapC, dl_dimage);
+    launch_chained(k_ssim_fwd, g.grid, kLossThreads, s, image, gt, H, W, win, mapAB, mapC, part);
+    launch_chained(k_ssim_bwd, g.grid, kLossThreads, s, image, gt, H, W, win, lambda, mapAB, mapC, part, loss_dev,
+                   dl_dimage);
     note_launches(2);
     return launch_status();
 }
