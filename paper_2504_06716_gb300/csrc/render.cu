@@ -520,14 +520,14 @@ __device__ __forceinline__ float keep_half(bool upper, float lo, float hi, int m
     return (upper ? hi : lo) + __shfl_xor_sync(kFull, upper ? lo : hi, mask);
 }
 
-// Which of the nine values lane l holds after sum9 (-1: none): the levels 8,
-// 4, 2 and 1 split them as {0-4 | 5-8}, {0-2 | 3-4} and {5-7 | 8}, ...
+// Which of a splat's nine gradient values lane l holds after sum_columns (-1:
+// none): lanes with bit 3 clear hold the six of mean, conic and opacity, split
+// by bit 2 as {0-2 | 3-5} and by bits 1 and 0 as {0, 1 | 2}; lanes with bit 3
+// set the colour's three.
 __device__ __forceinline__ int slot_of(int lane) {
-    const int h3 = lane & 8, h2 = lane & 4, q = lane & 3;
-    if (q == 3) return -1;
-    if (!h2) return (h3 ? 5 : 0) + q;
-    if (h3) return q == 0 ? 8 : -1;
-    return q < 2 ? 3 + q : -1;
+    const int q = lane & 3;
+    if (q == 3 || (lane & 12) == 12) return -1;
+    return (lane & 8 ? 6 : lane & 4 ? 3 : 0) + q;
 }
 
 // What the totals of slot are multiplied by: rows of grad2d hold dL/d(mean,
@@ -536,35 +536,51 @@ __device__ __forceinline__ float grad_scale(int slot) {
     return slot == 2 || slot == 4 ? -0.5f : slot == 3 ? -1.f : 1.f;
 }
 
-// The nine values of each half-warp summed over its 16 lanes: lane l gets the
-// total of value slot_of(l).
-__device__ __forceinline__ float sum9_half(const float (&g)[9], int lane) {
+// What a splat's gradient takes from its record, by the lanes that sum it.
+struct SplatSum {
+    float x, ha, nb, hc;  // mean's column, -a/2, -b, -c/2
+};
+
+// The sums of one splat over a block of 8 columns, from the six sums of each
+// thread's own pixels: s0, s1, s2 (dL/dpower, times dy and dy^2) and the
+// colour's three, held by the 16 lanes of half a warp, two rows of pixels. The
+// four rows of a column share dx: the six are summed over the rows first, and
+// only then turned into the moments of dx, half of the lanes with s0-s2 and half
+// with the colour; the columns are summed last. Lane l gets the total of value
+// slot_of(l).
+__device__ __forceinline__ float sum_columns(const float (&r)[6], const SplatSum &sp, float fpx, int lane) {
     const bool h3 = lane & 8, h2 = lane & 4, h1 = lane & 2, h0 = lane & 1;
-    float r[5], s[3];
+    float q[3], w[3];
 #pragma unroll
-    for (int j = 0; j < 5; ++j) r[j] = keep_half(h3, g[j], j < 4 ? g[5 + j] : 0.f, 8);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) s[j] = keep_half(h2, r[j], j < 2 ? r[3 + j] : 0.f, 4);
-    const float u0 = keep_half(h1, s[0], s[2], 2), u1 = keep_half(h1, s[1], 0.f, 2);
+    for (int j = 0; j < 3; ++j) q[j] = keep_half(h3, r[j], r[3 + j], 8);
+    // -(a mx + b s1), -(b mx + c s1), dx^2 s0 | dx s1, s2, s0
+    const float dx = __fsub_rn(sp.x, fpx), mx = dx * q[0];
+    const float v0 = h3 ? q[0] : fmaf(sp.ha, mx + mx, sp.nb * q[1]);
+    const float v1 = h3 ? q[1] : fmaf(sp.hc, q[1] + q[1], sp.nb * mx);
+    const float v2 = h3 ? q[2] : dx * mx;
+    w[0] = keep_half(h2, v0, dx * q[1], 4);
+    w[1] = keep_half(h2, v1, q[2], 4);
+    w[2] = keep_half(h2, v2, q[0], 4);
+    const float u0 = keep_half(h1, w[0], w[2], 2), u1 = w[1] + __shfl_xor_sync(kFull, w[1], 2);
     return keep_half(h0, u0, u1, 1);
 }
 
-// Two splats' nine values at once: lanes 0-15 get the totals of a, lanes 16-31
-// those of b (20 shuffles for both; one splat alone takes 18).
-__device__ __forceinline__ float sum9_pair(const float (&a)[9], const float (&b)[9], int lane) {
-    const bool h4 = lane & 16;
-    float g[9];
+// Two splats' sums at once: lanes 0-15 get the totals of a, lanes 16-31 those of
+// b, sp being each lane's own.
+__device__ __forceinline__ float sum_pair(const float (&a)[6], const float (&b)[6], const SplatSum &sp, float fpx,
+                                          int lane) {
+    float r[6];
 #pragma unroll
-    for (int j = 0; j < 9; ++j) g[j] = keep_half(h4, a[j], b[j], 16);
-    return sum9_half(g, lane);
+    for (int j = 0; j < 6; ++j) r[j] = keep_half(lane & 16, a[j], b[j], 16);
+    return sum_columns(r, sp, fpx, lane);
 }
 
-// One splat's nine values: both half-warps get its totals.
-__device__ __forceinline__ float sum9_one(const float (&a)[9], int lane) {
-    float g[9];
+// One splat's: both half-warps get its totals.
+__device__ __forceinline__ float sum_one(const float (&a)[6], const SplatSum &sp, float fpx, int lane) {
+    float r[6];
 #pragma unroll
-    for (int j = 0; j < 9; ++j) g[j] = a[j] + __shfl_xor_sync(kFull, a[j], 16);
-    return sum9_half(g, lane);
+    for (int j = 0; j < 6; ++j) r[j] = a[j] + __shfl_xor_sync(kFull, a[j], 16);
+    return sum_columns(r, sp, fpx, lane);
 }
 
 // Backward state of one pixel: recovered transmittance T, dL/dC, and the
@@ -640,7 +656,7 @@ __device__ __forceinline__ void pix_load(PixBwd &p, bool inside, int64_t pix, in
 template <int PPT, class V>
 __device__ __noinline__ void scalar_steps(PixBwd *p, const Stage<V> &S, const uint32_t *gid, int cnt, unsigned fz,
                                           float fpx, float fpy0, float *grad2d) {
-    const int lane = threadIdx.x & 31, slot = slot_of(lane);
+    const int lane = threadIdx.x & 31;
     for (int j = 0; j < cnt; ++j) {
         const float dx = __fsub_rn(v_lo(S.a[j].x), fpx), ha = v_lo(S.a[j].z), nb = v_lo(S.a[j].w), hc = v_lo(S.b[j].x);
         SplatRow row;
@@ -658,9 +674,15 @@ __device__ __noinline__ void scalar_steps(PixBwd *p, const Stage<V> &S, const ui
             const float mx = dx * g[0];
             const float e[9] = {fmaf(ha, mx + mx, nb * g[1]), fmaf(hc, g[1] + g[1], nb * mx), dx * mx, dx * g[1], g[2],
                                 g[5], g[6], g[7], g[8]};
-            const float tot = sum9_one(e, lane) * grad_scale(slot);
-            if (slot >= 0 && lane < 16 && tot != 0.f)
-                atomicAdd(grad2d + (int64_t)(gid[j] & 0x7fffffffu) * kG2d + slot, tot);
+            float tot = 0.f;  // lane l: the total of value l
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                float t = e[q];
+#pragma unroll
+                for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+                if (lane == q) tot = t * grad_scale(q);
+            }
+            if (lane < 9 && tot != 0.f) atomicAdd(grad2d + (int64_t)(gid[j] & 0x7fffffffu) * kG2d + lane, tot);
         }
     }
 }
@@ -672,14 +694,15 @@ __device__ __noinline__ void scalar_steps(PixBwd *p, const Stage<V> &S, const ui
 // much longer than the others', by that tile's chain of splats: two splats are
 // gone through together so that their latencies overlap.
 //
-// An unfrozen splat needs nine sums over the block: the moments s0 = sum of
-// dL/dpower, s1 and s2 (times dy and dy^2, formed per pixel), turned per lane
-// into the gradients of mean and conic; the opacity's, which is s0 / opacity
-// (dL/dpower = dL/dalpha alpha where alpha is not capped); the three of the
-// colour. Two unfrozen splats are summed over the warp together and added to
-// grad2d by the lanes that hold the totals, 18 adds to two rows in one
-// instruction: no shared accumulator, and per splat and block two sectors of
-// atomics instead of nine scattered words.
+// An unfrozen splat needs nine sums over the block: mean's two and the conic's
+// three from the moments of dL/dpower; the opacity's, which is the zeroth moment
+// / opacity (dL/dpower = dL/dalpha alpha where alpha is not capped); the three of
+// the colour. Two unfrozen splats are summed over the warp together, six sums of
+// each over the rows first and nine over the columns (sum_columns: 15 shuffles
+// for both, and the moments of dx are formed once per column; nine sums over
+// all lanes took 20), and added to grad2d by the lanes that hold the totals, 18
+// adds to two rows in one instruction: no shared accumulator, and per splat and
+// block two sectors of atomics instead of nine scattered words.
 //
 // A frozen splat only moves T and G, a uniform branch.
 //
@@ -691,9 +714,9 @@ __device__ __noinline__ void scalar_steps(PixBwd *p, const Stage<V> &S, const ui
 // Measured against the kernel before it (a barrier-separated batch per CTA,
 // scalar steps with divisions, one splat's sums at a time into a shared
 // accumulator by atomics): 1M Gaussians, 1237x822, 8-pixel tiles, two pixels
-// per thread, nothing frozen 492 -> 349 us, 95% frozen 220 -> 157 us (one
-// pixel per thread 208 -> 138 us); 400K at 800x800, 16-pixel tiles, half frozen
-// 445 -> 172 us; 2K at 128x128 114 -> 33 us.
+// per thread, nothing frozen 492 -> 324 us (348 with nine sums over all lanes),
+// 95% frozen 220 -> 156 us (one pixel per thread 208 -> 138 us); 400K at 800x800,
+// 16-pixel tiles, half frozen 445 -> 168 us; 2K at 128x128 114 -> 28 us.
 template <int TS, int PPT>
 __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats, const uint32_t *__restrict__ vals,
                                                 const uint32_t *__restrict__ ranges, const DevCam &cam,
@@ -744,7 +767,8 @@ __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats
 
     const int slot = slot_of(lane);
     const float scale = grad_scale(slot);
-    float pend[9];  // the sums of an unfrozen splat that waits for a second one
+    float pend[6];  // the sums of an unfrozen splat that waits for a second one
+    SplatSum pend_s = {};
     uint32_t pend_g = 0;
     float pend_o = 1.f;
     bool waiting = false;
@@ -834,9 +858,9 @@ __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats
                     G[h] = v_fma(v_mul(dk[i][h], a), T[h], G[h]);
                 }
             }
-            // the nine sums of splat i over this thread's pixels; false if none uses it
-            auto sums = [&](int i, float (&g)[9]) -> bool {
-                const V4<V> sa = S.a[j + i], sb = S.b[j + i];
+            // the six sums of splat i over this thread's pixels; false if none uses it
+            auto sums = [&](int i, float (&g)[6]) -> bool {
+                const V4<V> sb = S.b[j + i];
                 auto total = [](V v) -> float {
                     float e[L];
                     v_get(v, e);
@@ -870,38 +894,41 @@ __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats
                     c1 += total(v_mul(w, d1[h]));
                     c2 += total(v_mul(w, d2[h]));
                 }
-                const float dx = __fsub_rn(v_lo(sa.x), fpx), mx = dx * s0;
-                // -(a mx + b s1), -(b mx + c s1) from the staged -a/2, -b, -c/2
-                g[0] = fmaf(v_lo(sa.z), mx + mx, v_lo(sa.w) * s1);
-                g[1] = fmaf(v_lo(sb.x), s1 + s1, v_lo(sa.w) * mx);
-                g[2] = dx * mx;
-                g[3] = dx * s1;
-                g[4] = s2; g[5] = s0; g[6] = c0; g[7] = c1; g[8] = c2;
+                g[0] = s0; g[1] = s1; g[2] = s2; g[3] = c0; g[4] = c1; g[5] = c2;
                 return any;
+            };
+            auto part = [&](int i) {
+                return SplatSum{v_lo(S.a[i].x), v_lo(S.a[i].z), v_lo(S.a[i].w), v_lo(S.b[i].x)};
             };
             const unsigned f = (fz >> j) & ((1u << K) - 1u);
             if (f == (1u << K) - 1u) return;  // frozen
             if (K == 2 && f == 0u) {
-                float g[9], g2[9];
+                float g[6], g2[6];
                 bool any = sums(0, g);
                 any = sums(K - 1, g2) || any;
                 if (!__any_sync(kFull, any)) return;
                 const int i = lane < 16 ? j : j + K - 1;
-                give(sum9_pair(g, g2, lane), gid[i], v_lo(S.b[i].y), slot >= 0);
+                give(sum_pair(g, g2, part(i), fpx, lane), gid[i], v_lo(S.b[i].y), slot >= 0);
                 return;
             }
-            float g[9];
+            float g[6];
             const int i = K == 2 && f == 1u ? K - 1 : 0;  // the unfrozen one
             const bool any = i ? sums(K - 1, g) : sums(0, g);
             if (!__any_sync(kFull, any)) return;
+            const SplatSum own = part(j + i);
+            const uint32_t own_g = gid[j + i];
+            const float own_o = v_lo(S.b[j + i].y);
             if (waiting) {
-                give(sum9_pair(pend, g, lane), lane < 16 ? pend_g : gid[j + i], lane < 16 ? pend_o : v_lo(S.b[j + i].y),
-                     slot >= 0);
+                const bool first = lane < 16;
+                const SplatSum sp{first ? pend_s.x : own.x, first ? pend_s.ha : own.ha, first ? pend_s.nb : own.nb,
+                                  first ? pend_s.hc : own.hc};
+                give(sum_pair(pend, g, sp, fpx, lane), first ? pend_g : own_g, first ? pend_o : own_o, slot >= 0);
             } else {
 #pragma unroll
-                for (int q = 0; q < 9; ++q) pend[q] = g[q];
-                pend_g = gid[j + i];
-                pend_o = v_lo(S.b[j + i].y);
+                for (int q = 0; q < 6; ++q) pend[q] = g[q];
+                pend_s = own;
+                pend_g = own_g;
+                pend_o = own_o;
             }
             waiting = !waiting;
         };
@@ -930,12 +957,13 @@ __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats
         }
         __syncwarp();  // the staged splats are no longer read
     }
-    if (waiting) give(sum9_one(pend, lane), pend_g, pend_o, slot >= 0 && lane < 16);
+    if (waiting) give(sum_one(pend, pend_s, fpx, lane), pend_g, pend_o, slot >= 0 && lane < 16);
 }
 
 // Warps to keep resident per SM: 24 with one pixel per thread (78 registers), 16
-// with two (1M Gaussians, 1237x822, nothing frozen: 349 us against 362 without
-// the bound, which takes 132 registers and 12 warps, and 361 at 20 warps).
+// with two (1M Gaussians, 1237x822, nothing frozen, with nine sums over all lanes:
+// 349 us against 362 without the bound, at 132 registers and 12 warps, and 361 at
+// 20 warps; 324 us now at 111 registers and 18 warps).
 template <int TS, int PPT>
 constexpr int bwd_blocks() {
     constexpr int warps = PPT == 1 ? 24 : PPT == 2 ? 16 : 1, per = TS * TS / PPT / 32;
