@@ -121,11 +121,14 @@ __device__ __forceinline__ PartSum<T> part_sum(const T *__restrict__ part, int n
 }
 
 // ---- stage 1a: compaction of visible Gaussians ----
-// Eight small blocks per SM, each over one contiguous range of the Gaussians,
-// so that the next kernel's blocks can sum the counts in front of their own
-// range and no scan runs between the two.
+// Five small blocks per SM, each over one contiguous range of the Gaussians, so
+// that the next kernel's blocks can sum the counts in front of their own range
+// and no scan runs between the two. Five fit at the emitting kernels' 48
+// registers: one wave, each block with the same share (eight per SM, in a second
+// wave of a few: the emitting kernels 25.5 + 27.8 us against 24.5 + 21.3 at 1M
+// Gaussians, 12.9 + 12.1 against 10.9 + 10.8 at 250K).
 constexpr int kVisBlock = 256;
-constexpr int kVisGrid = 8 * kSortGrid;
+constexpr int kVisGrid = 5 * kSortGrid;
 
 __host__ __device__ inline int64_t vis_range(int64_t n) {
     const int64_t r = (n + kVisGrid - 1) / kVisGrid;
@@ -689,7 +692,7 @@ __device__ __forceinline__ PartSum<uint32_t> warps_before(uint32_t v, uint32_t (
 
 // The depth keys and indices of the visible Gaussians, ascending index, their
 // cull records, and the first radix pass's digit counts.
-__global__ void __launch_bounds__(kVisBlock) k_emit_visible(const float *__restrict__ splats, int64_t n,
+__global__ void __launch_bounds__(kVisBlock, 5) k_emit_visible(const float *__restrict__ splats, int64_t n,
                                                            const uint32_t *__restrict__ part, DevCam cam,
                                                            uint2 *__restrict__ kv0, uint2 *__restrict__ kv1,
                                                            float4 *__restrict__ cull, uint32_t *__restrict__ n_vis,
@@ -827,7 +830,7 @@ __global__ void k_finish_count(const unsigned long long *__restrict__ total_t,
 
 // The super-tile entries in depth order, clipped to the capacity (*sclip of
 // them kept, of *total_s), and the first super-tile pass's digit counts.
-__global__ void __launch_bounds__(kVisBlock) k_emit_super(const float *__restrict__ splats,
+__global__ void __launch_bounds__(kVisBlock, 5) k_emit_super(const float *__restrict__ splats,
                                                           const float4 *__restrict__ cull,
                                                           const uint32_t *__restrict__ order,
                                                           const uint32_t *__restrict__ n_vis, DevCam cam,
@@ -1097,7 +1100,7 @@ __device__ __forceinline__ int slot_tile(int t, int sx, int sy, int tiles_x) {
 // through the test. 1M Gaussians, 931K entries: 66 us with the four-edge test of
 // every tile, 61 with two edges and the owner found by a population count, 42 by
 // rows (22M instead of 40M instructions); 3M Gaussians 117 -> 88 us.
-__global__ void __launch_bounds__(kChunk) k_chunk_counts(const float *__restrict__ splats,
+__global__ void __launch_bounds__(kChunk, 5) k_chunk_counts(const float *__restrict__ splats,
                                                         const float4 *__restrict__ cull,
                                                         const uint32_t *__restrict__ svals,
                                                         const uint32_t *__restrict__ chunk_base,
