@@ -231,6 +231,21 @@ int gs_raster_bwd_resume(const float *splats, const uint32_t *vals, const uint32
                          const float *dl_dimage, const uint8_t *frozen, const float *resume,
                          const int32_t *resume_pos, float *grad2d, gs_stream_t stream);
 
+/* Sec. 3.1 and Sec. 3.2.4: gs_render_fwd_resume and gs_raster_bwd_resume (same results) with the tiles taken
+ * longest list first, in the order that gs_sort left in its workspace for
+ * these lists: sort_ws of sort_ws_bytes, unchanged since that call. A NULL, too
+ * small or unaligned workspace, or one whose last sort was for another grid, means
+ * ascending tiles. */
+int gs_render_fwd_sorted(const float *splats, const uint32_t *vals, const uint32_t *ranges, const gs_camera *cam,
+                         const gs_raster_config *cfg, const uint8_t *frozen, float *image, float *t_final,
+                         int32_t *n_last, float *resume, int32_t *resume_pos, const void *sort_ws,
+                         size_t sort_ws_bytes, gs_stream_t stream);
+int gs_raster_bwd_sorted(const float *splats, const uint32_t *vals, const uint32_t *ranges, const gs_camera *cam,
+                         const gs_raster_config *cfg, const float *t_final, const int32_t *n_last,
+                         const float *dl_dimage, const uint8_t *frozen, const float *resume,
+                         const int32_t *resume_pos, float *grad2d, const void *sort_ws, size_t sort_ws_bytes,
+                         gs_stream_t stream);
+
 /* Several scenes in one launch. The paper trains one scene at a time and
  * has no counterpart; each job computes what gs_render_fwd (Sec. 3.1,
  * Eq. 2) or gs_raster_bwd (Sec. 3.2.4) computes for one view.

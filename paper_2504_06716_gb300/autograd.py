@@ -37,7 +37,7 @@ class RasterizeGaussians(torch.autograd.Function):
         image = torch.empty((3, H, W), dtype=torch.float32, device=dev)
         t_final = torch.empty((H, W), dtype=torch.float32, device=dev)
         n_last = torch.empty((H, W), dtype=torch.int32, device=dev)
-        lib.gs_render_fwd(splats, vals, ranges, cam, image, t_final, n_last)
+        lib.gs_render_fwd_sorted(splats, vals, ranges, cam, None, None, image, t_final, n_last, None, None, ws)
         ctx.save_for_backward(P, splats, vals, ranges, t_final, n_last)
         ctx.cam, ctx.sh_degree, ctx.frozen = cam, sh_degree, frozen
         ctx.mark_non_differentiable(t_final, n_last)

@@ -6,6 +6,16 @@
 namespace gs {
 static std::atomic<unsigned long long> g_launches{0};
 void note_launches(int k) { g_launches.fetch_add((unsigned long long)k, std::memory_order_relaxed); }
+int render_fwd_ordered(const float *splats, const uint32_t *vals, const uint32_t *ranges, const gs_camera *cam,
+                       const gs_raster_config *cfg, const uint8_t *frozen, float *image, float *t_final,
+                       int32_t *n_last, float *resume, int32_t *resume_pos, const TileOrder &order, int32_t *depth,
+                       gs_stream_t stream);
+int raster_bwd_ordered(const float *splats, const uint32_t *vals, const uint32_t *ranges, const gs_camera *cam,
+                       const gs_raster_config *cfg, const float *t_final, const int32_t *n_last,
+                       const float *dl_dimage, const uint8_t *frozen, const float *resume, const int32_t *resume_pos,
+                       float *grad2d, const TileOrder &order, gs_stream_t stream);
+int loss_ordering(const float *image, const float *gt, int32_t H, int32_t W, float lambda, void *ws, size_t ws_bytes,
+                  float *loss_dev, float *dl_dimage, int tiles, const SortFront &front, gs_stream_t stream);
 uint32_t take_sort_flags();
 uint32_t take_loss_flags();
 uint32_t take_render_flags();
@@ -33,18 +43,32 @@ extern "C" int gs_train_step(const gs_step *s, const gs_camera *cam, const float
     if (st == GS_OK)
         st = gs_sort(s->splats, s->n, cam, s->sort_ws, s->sort_ws_bytes, s->capacity, s->vals, s->ranges,
                      s->count_dev, stream);
+    // the tiles' orders: the forward's by list length, as the sort just left it, the
+    // backward's by the depth that the forward reaches
+    TileOrder by_length{}, by_depth{};
+    SortFront front{};
+    int tiles = 0;  // 0: not ordered
+    if (st == GS_OK && s->n > 0 && s->capacity > 0) {
+        const DevCam dc = make_cam(cam);
+        if (dc.tiles_x * dc.tiles_y >= kOrderMinTiles) {
+            tiles = dc.tiles_x * dc.tiles_y;
+            front = sort_front(s->sort_ws, tiles);
+            by_length.order = front.order;
+            by_depth.order = front.order_deep;
+        }
+    }
     if (st == GS_OK)
-        st = gs_render_fwd_resume(s->splats, s->vals, s->ranges, cam, fwd, s->frozen, s->image, s->t_final, s->n_last,
-                                  s->resume, s->resume_pos, stream);
+        st = render_fwd_ordered(s->splats, s->vals, s->ranges, cam, fwd, s->frozen, s->image, s->t_final, s->n_last,
+                                s->resume, s->resume_pos, by_length, front.depth, stream);
     if (st == GS_OK)
-        st = gs_loss(s->image, gt, cam->height, cam->width, s->lambda_ssim, s->loss_ws, s->loss_ws_bytes, s->loss_dev,
-                     s->dl_dimage, stream);
+        st = loss_ordering(s->image, gt, cam->height, cam->width, s->lambda_ssim, s->loss_ws, s->loss_ws_bytes,
+                           s->loss_dev, s->dl_dimage, tiles, front, stream);
     cudaStream_t cs = as_stream(stream);
     if (st == GS_OK && s->bwd_events[0] && cudaEventRecord(static_cast<cudaEvent_t>(s->bwd_events[0]), cs) != cudaSuccess)
         st = GS_ERR_CUDA;
     if (st == GS_OK)
-        st = gs_raster_bwd_resume(s->splats, s->vals, s->ranges, cam, bwd, s->t_final, s->n_last, s->dl_dimage,
-                                  s->frozen, s->resume, s->resume_pos, s->grad2d, stream);
+        st = raster_bwd_ordered(s->splats, s->vals, s->ranges, cam, bwd, s->t_final, s->n_last, s->dl_dimage,
+                                s->frozen, s->resume, s->resume_pos, s->grad2d, by_depth, stream);
     if (st == GS_OK && s->bwd_events[1] && cudaEventRecord(static_cast<cudaEvent_t>(s->bwd_events[1]), cs) != cudaSuccess)
         st = GS_ERR_CUDA;
     if (st == GS_OK)

@@ -114,15 +114,32 @@ __device__ void loss_from_parts(const float2 *part, int nparts, int64_t N, float
     }
 }
 
+// Inside a training step the first blocks of the two kernels also make the order in
+// which the rasteriser's backward takes the tiles: by the depth their walk
+// reached in the forward, longest first, 256 tiles per block (one block for all
+// of 16K tiles took 40 us longer than the kernel's others).
+struct DepthOrder {
+    int tiles;  // 0: none
+    const int32_t *depth;
+    uint32_t *order, *hist, *next;
+
+    __device__ int block() const { return (int)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x); }
+    __device__ bool mine() const { return block() < (tiles + kLenBuckets - 1) / kLenBuckets; }
+};
+static_assert(kLossThreads == kLenBuckets, "a bucket per thread");
+
 __global__ void __launch_bounds__(kLossThreads) k_ssim_fwd(const float *__restrict__ img,
                                                           const float *__restrict__ gt, int H, int W, Win win,
                                                           f32x2 *__restrict__ mapAB, float *__restrict__ mapC,
-                                                          float2 *__restrict__ part) {
+                                                          float2 *__restrict__ part, DepthOrder deep) {
     __shared__ __align__(16) f32x2 sxy[kE][kE];
     __shared__ __align__(16) f32x2 h[2][kE][kH2];
     __shared__ __align__(16) float hxy[kE][kH1];
     __shared__ float red[2][kLossThreads / 32];
     wait_prior_grid();
+    if (deep.mine())
+        count_buckets<1>(deep.block(), deep.tiles, [&](int t) { return (uint32_t)deep.depth[t]; },
+                         reinterpret_cast<uint32_t *>(&hxy[0][0]), deep.hist);
     const int ch = blockIdx.z;
     const int64_t HW = (int64_t)H * W;
     const float *x = img + ch * HW, *y = gt + ch * HW;
@@ -230,7 +247,7 @@ __global__ void __launch_bounds__(kLossThreads, 5) k_ssim_bwd(const float *__res
                                                           float lambda, const f32x2 *__restrict__ mapAB,
                                                           const float *__restrict__ mapC,
                                                           const float2 *__restrict__ part, float *__restrict__ loss,
-                                                          float *__restrict__ dl) {
+                                                          float *__restrict__ dl, DepthOrder deep) {
     __shared__ __align__(16) f32x2 sab[kE][kE];
     __shared__ __align__(16) float sc[kE][kE1];
     __shared__ __align__(16) f32x2 h[kE][kH2];  // also the first block's reduction scratch
@@ -239,6 +256,10 @@ __global__ void __launch_bounds__(kLossThreads, 5) k_ssim_bwd(const float *__res
     wait_prior_grid();
     const int ch = blockIdx.z;
     const int64_t HW = (int64_t)H * W;
+    if (deep.mine())
+        place_buckets<1>(deep.block(), deep.tiles, [&](int t) { return (uint32_t)deep.depth[t]; },
+                         [&](int t, uint32_t at) { deep.order[at] = (uint32_t)t; }, deep.hist, deep.next,
+                         reinterpret_cast<uint32_t *>(&hc[0][0]));
     if (blockIdx.x + blockIdx.y + blockIdx.z == 0)  // h is written again behind the next barrier
         loss_from_parts(part, (int)(gridDim.x * gridDim.y * gridDim.z), 3 * HW, lambda, loss,
                         reinterpret_cast<double *>(&h[0][0]));
@@ -385,8 +406,9 @@ extern "C" size_t gs_loss_workspace_bytes(int32_t H, int32_t W) {
     return align256(maps) + align256(sizeof(float2) * (size_t)loss_grid(H, W).nparts) + 256;
 }
 
-extern "C" int gs_loss(const float *image, const float *gt, int32_t H, int32_t W, float lambda, void *ws,
-                       size_t ws_bytes, float *loss_dev, float *dl_dimage, gs_stream_t stream) {
+namespace gs {
+int loss_ordering(const float *image, const float *gt, int32_t H, int32_t W, float lambda, void *ws, size_t ws_bytes,
+                  float *loss_dev, float *dl_dimage, int tiles, const SortFront &front, gs_stream_t stream) {
     if (H <= 0 || W <= 0 || H > 16384 || W > 16384 || !(lambda >= 0.f && lambda <= 1.f)) return GS_ERR_INVALID_ARG;
     if (!image || !gt || !ws || !loss_dev || !dl_dimage) return GS_ERR_INVALID_ARG;
     if (ws_bytes < gs_loss_workspace_bytes(H, W) || (reinterpret_cast<uintptr_t>(ws) & 255)) return GS_ERR_INVALID_ARG;
@@ -397,11 +419,19 @@ extern "C" int gs_loss(const float *image, const float *gt, int32_t H, int32_t W
     float2 *part = reinterpret_cast<float2 *>(static_cast<char *>(ws) + align256(9 * (size_t)HW * sizeof(float)));
     LossGrid g = loss_grid(H, W);
     Win win = make_window();
-    launch_chained(k_ssim_fwd, g.grid, kLossThreads, s, image, gt, H, W, win, mapAB, mapC, part);
+    // 256 tiles of 64 pixels or more and 3 x 1024 pixels a block: there are enough of them
+    const DepthOrder deep{tiles, front.depth, front.order_deep, front.hist, front.next};
+    launch_chained(k_ssim_fwd, g.grid, kLossThreads, s, image, gt, H, W, win, mapAB, mapC, part, deep);
     launch_chained(k_ssim_bwd, g.grid, kLossThreads, s, image, gt, H, W, win, lambda, mapAB, mapC, part, loss_dev,
-                   dl_dimage);
+                   dl_dimage, deep);
     note_launches(2);
     return launch_status();
+}
+}  // namespace gs
+
+extern "C" int gs_loss(const float *image, const float *gt, int32_t H, int32_t W, float lambda, void *ws,
+                       size_t ws_bytes, float *loss_dev, float *dl_dimage, gs_stream_t stream) {
+    return loss_ordering(image, gt, H, W, lambda, ws, ws_bytes, loss_dev, dl_dimage, 0, SortFront{}, stream);
 }
 
 extern "C" size_t gs_psnr_workspace_bytes(int32_t S, int32_t H, int32_t W) {

@@ -189,7 +189,8 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
                                             int32_t *__restrict__ n_last, int tile, int batch = 0,
                                             const uint8_t *__restrict__ frozen = nullptr,
                                             float4 *__restrict__ resume = nullptr,
-                                            int32_t *__restrict__ resume_pos = nullptr) {
+                                            int32_t *__restrict__ resume_pos = nullptr,
+                                            int32_t *__restrict__ depth = nullptr) {
     constexpr int L = Lanes<PPT>::L, NP = Lanes<PPT>::NP;
     typedef typename ValueOf<L>::T V;
     constexpr int kWarps = TS * TS / PPT / 32, kH = 4 * PPT;
@@ -470,6 +471,13 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
         }
         if (threadIdx.x == 0) resume_pos[tile] = umax;
     }
+    if (depth) {  // how far the tile's walk got: the backward takes the tiles by it
+        int d = last[0];
+#pragma unroll
+        for (int k = 1; k < PPT; ++k) d = max(d, last[k]);
+        d = __reduce_max_sync(kFull, d);
+        if (lane == 0 && d > 0) atomicMax(depth + tile, d);
+    }
     float4 f[PPT];
     state(f);
     const int64_t HW = (int64_t)cam.W * cam.H;
@@ -508,10 +516,10 @@ __global__ void __launch_bounds__(TS * TS / PPT, fwd_blocks<TS, PPT, RES>())
     k_render_fwd(const float *__restrict__ splats, const uint32_t *__restrict__ vals, const uint32_t *__restrict__ ranges,
                  DevCam cam, float *__restrict__ image, float *__restrict__ t_final, int32_t *__restrict__ n_last,
                  int batch, const uint8_t *__restrict__ frozen, float4 *__restrict__ resume,
-                 int32_t *__restrict__ resume_pos) {
+                 int32_t *__restrict__ resume_pos, TileOrder order, int32_t *__restrict__ depth) {
     wait_prior_grid();
-    render_tile<TS, PPT, RES>(splats, vals, ranges, cam, image, t_final, n_last, blockIdx.x, batch, frozen, resume,
-                              resume_pos);
+    render_tile<TS, PPT, RES>(splats, vals, ranges, cam, image, t_final, n_last, ordered_tile(order), batch, frozen,
+                              resume, resume_pos, depth);
 }
 
 // Sums over a warp by recursive halving: at each xor level a lane keeps half
@@ -975,10 +983,10 @@ __global__ void __launch_bounds__(TS * TS / PPT, bwd_blocks<TS, PPT>())
     k_raster_bwd(const float *__restrict__ splats, const uint32_t *__restrict__ vals, const uint32_t *__restrict__ ranges,
                  DevCam cam, const float *__restrict__ t_final, const int32_t *__restrict__ n_last,
                  const float *__restrict__ dl_dimage, const uint8_t *__restrict__ frozen, float *__restrict__ grad2d,
-                 const float4 *__restrict__ resume, const int32_t *__restrict__ resume_pos) {
+                 const float4 *__restrict__ resume, const int32_t *__restrict__ resume_pos, TileOrder order) {
     wait_prior_grid();
-    raster_bwd_tile<TS, PPT>(splats, vals, ranges, cam, t_final, n_last, dl_dimage, frozen, grad2d, blockIdx.x, resume,
-                             resume_pos);
+    raster_bwd_tile<TS, PPT>(splats, vals, ranges, cam, t_final, n_last, dl_dimage, frozen, grad2d, ordered_tile(order),
+                             resume, resume_pos);
 }
 
 // ---- measurement support: the (pixel, splat) pairs the backward visits ----
@@ -1148,6 +1156,8 @@ struct FwdArgs {
     const uint8_t *frozen;
     float4 *resume;
     int32_t *resume_pos;
+    TileOrder order;
+    int32_t *depth;
 };
 
 struct BwdArgs {
@@ -1161,6 +1171,7 @@ struct BwdArgs {
     float *grad2d;
     const float4 *resume;
     const int32_t *resume_pos;
+    TileOrder order;
 };
 
 template <int TS, int PPT>
@@ -1168,16 +1179,16 @@ void launch(int batch, const FwdArgs &a, cudaStream_t s) {
     const int tiles = a.cam.tiles_x * a.cam.tiles_y;
     if (a.resume)
         launch_chained(k_render_fwd<TS, PPT, true>, tiles, TS * TS / PPT, s, a.splats, a.vals, a.ranges, a.cam, a.image,
-                       a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos);
+                       a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos, a.order, a.depth);
     else
         launch_chained(k_render_fwd<TS, PPT, false>, tiles, TS * TS / PPT, s, a.splats, a.vals, a.ranges, a.cam,
-                       a.image, a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos);
+                       a.image, a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos, a.order, a.depth);
 }
 
 template <int TS, int PPT>
 void launch(int, const BwdArgs &a, cudaStream_t s) {
     launch_chained(k_raster_bwd<TS, PPT>, a.cam.tiles_x * a.cam.tiles_y, TS * TS / PPT, s, a.splats, a.vals, a.ranges,
-                   a.cam, a.t_final, a.n_last, a.dl, a.frozen, a.grad2d, a.resume, a.resume_pos);
+                   a.cam, a.t_final, a.n_last, a.dl, a.frozen, a.grad2d, a.resume, a.resume_pos, a.order);
 }
 
 struct BatchArgs {
@@ -1237,20 +1248,75 @@ inline bool config_ok(const gs_raster_config *c, int tile) {
 
 using namespace gs;
 
-extern "C" int gs_render_fwd_resume(const float *splats, const uint32_t *vals, const uint32_t *ranges,
-                                    const gs_camera *cam, const gs_raster_config *cfg, const uint8_t *frozen,
-                                    float *image, float *t_final, int32_t *n_last, float *resume,
-                                    int32_t *resume_pos, gs_stream_t stream) {
+namespace gs {
+int render_fwd_ordered(const float *splats, const uint32_t *vals, const uint32_t *ranges, const gs_camera *cam,
+                       const gs_raster_config *cfg, const uint8_t *frozen, float *image, float *t_final,
+                       int32_t *n_last, float *resume, int32_t *resume_pos, const TileOrder &order, int32_t *depth,
+                       gs_stream_t stream) {
     if (!camera_ok(cam) || !config_ok(cfg, cam->tile) || !ranges || !image || !t_final || !n_last)
         return GS_ERR_INVALID_ARG;
     if ((resume == nullptr) != (resume_pos == nullptr)) return GS_ERR_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(splats) | reinterpret_cast<uintptr_t>(resume)) & 15) return GS_ERR_INVALID_ARG;
     FwdArgs a{splats, vals, ranges, make_cam(cam), image, t_final, n_last, frozen, reinterpret_cast<float4 *>(resume),
-              resume_pos};
+              resume_pos, order, depth};
     int ppt, batch;
     default_config(a.cam.tile, (int64_t)a.cam.tiles_x * a.cam.tiles_y, false, ppt, batch);
     if (cfg) { ppt = cfg->pixels_per_thread; batch = cfg->batch; }
     return dispatch(a.cam.tile, ppt, batch, a, as_stream(stream));
+}
+
+int raster_bwd_ordered(const float *splats, const uint32_t *vals, const uint32_t *ranges, const gs_camera *cam,
+                       const gs_raster_config *cfg, const float *t_final, const int32_t *n_last,
+                       const float *dl_dimage, const uint8_t *frozen, const float *resume, const int32_t *resume_pos,
+                       float *grad2d, const TileOrder &order, gs_stream_t stream) {
+    if (!camera_ok(cam) || !config_ok(cfg, cam->tile) || !ranges || !t_final || !n_last || !dl_dimage || !grad2d)
+        return GS_ERR_INVALID_ARG;
+    if ((resume == nullptr) != (resume_pos == nullptr)) return GS_ERR_INVALID_ARG;
+    if ((reinterpret_cast<uintptr_t>(splats) | reinterpret_cast<uintptr_t>(resume)) & 15) return GS_ERR_INVALID_ARG;
+    BwdArgs a{splats, vals, ranges, make_cam(cam), t_final, n_last, dl_dimage, frozen, grad2d,
+              reinterpret_cast<const float4 *>(resume), resume_pos, order};
+    int ppt, batch;
+    default_config(a.cam.tile, (int64_t)a.cam.tiles_x * a.cam.tiles_y, true, ppt, batch);
+    if (cfg) { ppt = cfg->pixels_per_thread; batch = cfg->batch; }
+    return dispatch(a.cam.tile, ppt, batch, a, as_stream(stream));
+}
+}  // namespace gs
+
+// The order in a sort's workspace, used if it is marked as this grid's.
+static TileOrder order_in(const gs_camera *cam, const void *sort_ws, size_t sort_ws_bytes) {
+    TileOrder o{};
+    if (!sort_ws || !camera_ok(cam)) return o;
+    const DevCam dc = make_cam(cam);
+    const int64_t tiles = (int64_t)dc.tiles_x * dc.tiles_y;
+    const SortFront f = sort_front(const_cast<void *>(sort_ws), tiles);
+    if (tiles < kOrderMinTiles || sort_ws_bytes < f.bytes || (reinterpret_cast<uintptr_t>(sort_ws) & 255)) return o;
+    return TileOrder{f.order, f.stamp, tile_order_key(dc.tiles_x, dc.tiles_y, dc.tile)};
+}
+
+extern "C" int gs_render_fwd_sorted(const float *splats, const uint32_t *vals, const uint32_t *ranges,
+                                    const gs_camera *cam, const gs_raster_config *cfg, const uint8_t *frozen,
+                                    float *image, float *t_final, int32_t *n_last, float *resume,
+                                    int32_t *resume_pos, const void *sort_ws, size_t sort_ws_bytes,
+                                    gs_stream_t stream) {
+    return render_fwd_ordered(splats, vals, ranges, cam, cfg, frozen, image, t_final, n_last, resume, resume_pos,
+                              order_in(cam, sort_ws, sort_ws_bytes), nullptr, stream);
+}
+
+extern "C" int gs_raster_bwd_sorted(const float *splats, const uint32_t *vals, const uint32_t *ranges,
+                                    const gs_camera *cam, const gs_raster_config *cfg, const float *t_final,
+                                    const int32_t *n_last, const float *dl_dimage, const uint8_t *frozen,
+                                    const float *resume, const int32_t *resume_pos, float *grad2d,
+                                    const void *sort_ws, size_t sort_ws_bytes, gs_stream_t stream) {
+    return raster_bwd_ordered(splats, vals, ranges, cam, cfg, t_final, n_last, dl_dimage, frozen, resume, resume_pos,
+                              grad2d, order_in(cam, sort_ws, sort_ws_bytes), stream);
+}
+
+extern "C" int gs_render_fwd_resume(const float *splats, const uint32_t *vals, const uint32_t *ranges,
+                                    const gs_camera *cam, const gs_raster_config *cfg, const uint8_t *frozen,
+                                    float *image, float *t_final, int32_t *n_last, float *resume,
+                                    int32_t *resume_pos, gs_stream_t stream) {
+    return render_fwd_ordered(splats, vals, ranges, cam, cfg, frozen, image, t_final, n_last, resume, resume_pos,
+                              TileOrder{}, nullptr, stream);
 }
 
 extern "C" int gs_render_fwd_cfg(const float *splats, const uint32_t *vals, const uint32_t *ranges,
@@ -1270,16 +1336,8 @@ extern "C" int gs_raster_bwd_resume(const float *splats, const uint32_t *vals, c
                                     const int32_t *n_last, const float *dl_dimage, const uint8_t *frozen,
                                     const float *resume, const int32_t *resume_pos, float *grad2d,
                                     gs_stream_t stream) {
-    if (!camera_ok(cam) || !config_ok(cfg, cam->tile) || !ranges || !t_final || !n_last || !dl_dimage || !grad2d)
-        return GS_ERR_INVALID_ARG;
-    if ((resume == nullptr) != (resume_pos == nullptr)) return GS_ERR_INVALID_ARG;
-    if ((reinterpret_cast<uintptr_t>(splats) | reinterpret_cast<uintptr_t>(resume)) & 15) return GS_ERR_INVALID_ARG;
-    BwdArgs a{splats, vals, ranges, make_cam(cam), t_final, n_last, dl_dimage, frozen, grad2d,
-              reinterpret_cast<const float4 *>(resume), resume_pos};
-    int ppt, batch;
-    default_config(a.cam.tile, (int64_t)a.cam.tiles_x * a.cam.tiles_y, true, ppt, batch);
-    if (cfg) { ppt = cfg->pixels_per_thread; batch = cfg->batch; }
-    return dispatch(a.cam.tile, ppt, batch, a, as_stream(stream));
+    return raster_bwd_ordered(splats, vals, ranges, cam, cfg, t_final, n_last, dl_dimage, frozen, resume, resume_pos,
+                              grad2d, TileOrder{}, stream);
 }
 
 extern "C" int gs_raster_bwd_cfg(const float *splats, const uint32_t *vals, const uint32_t *ranges,

@@ -1162,12 +1162,21 @@ __global__ void __launch_bounds__(kScanBlock) k_tile_starts(const uint32_t *__re
                                                            const unsigned long long *__restrict__ total_exact,
                                                            unsigned long long *__restrict__ tile_start,
                                                            uint32_t *__restrict__ ranges,
-                                                           int64_t *__restrict__ count_dev) {
-    wait_prior_grid();
+                                                           int64_t *__restrict__ count_dev,
+                                                           uint32_t *__restrict__ len_hist) {
     __shared__ unsigned long long ws[32];
     __shared__ unsigned long long ps[64];
+    __shared__ uint32_t bins[kLenBuckets];
+    if (threadIdx.x < kLenBuckets) bins[threadIdx.x] = 0u;
+    wait_prior_grid();
     const int64_t first = (int64_t)blockIdx.x * kScanBlock, j = first + threadIdx.x;
     const unsigned long long n = j < tiles ? tile_count[j] : 0ull;
+    if (len_hist) {  // tiles per length bucket, for the order that k_expand's first blocks make
+        __syncthreads();
+        take_place(bins, length_bucket((uint32_t)n), j < tiles);
+        __syncthreads();
+        if (threadIdx.x < kLenBuckets && bins[threadIdx.x]) atomicAdd(len_hist + threadIdx.x, bins[threadIdx.x]);
+    }
     unsigned long long before;
     if (part) {
         before = part_sum<unsigned long long>(part, (int)gridDim.x, (int)blockIdx.x, ps).before;
@@ -1194,6 +1203,33 @@ __global__ void __launch_bounds__(kScanBlock) k_tile_starts(const uint32_t *__re
     }
 }
 
+// What k_expand's first blocks turn into the tiles' order by list length: a
+// counting sort, the buckets from k_tile_starts, kOrderTiles tiles per block.
+constexpr int kOrderTiles = 4 * kChunk;
+struct OrderPlan {
+    int blocks;  // 0: no order is made
+    const uint32_t *count, *hist;
+    uint32_t *next;
+    SortFront front;
+    int tiles;
+    uint2 key;
+};
+
+__device__ __forceinline__ void order_tiles(const OrderPlan &o, uint32_t *s /* 3 * kLenBuckets + 32 */) {
+    static_assert(kChunk == kLenBuckets, "a bucket per thread");
+    place_buckets<kOrderTiles / kChunk>(
+        (int)blockIdx.x, o.tiles, [&](int t) { return o.count[t]; },
+        [&](int t, uint32_t at) {
+            o.front.order[at] = (uint32_t)t;
+            o.front.depth[t] = 0;
+        },
+        o.hist, o.next, s);
+    if (blockIdx.x == 0) {
+        o.front.hist[threadIdx.x] = o.front.next[threadIdx.x] = 0u;
+        if (threadIdx.x == 0) *o.front.stamp = o.key;
+    }
+}
+
 // Bound by instruction issue; a slot's place and its lanes are one 8-byte word
 // in shared memory and positions have 32 bits (40 -> 30 us at 931K entries,
 // 4.8M places).
@@ -1203,17 +1239,21 @@ __global__ void __launch_bounds__(kChunk) k_expand(const float *__restrict__ spl
                                                   DevCam cam, const uint32_t *__restrict__ counts,
                                                   const unsigned long long *__restrict__ tile_start, int64_t capacity,
                                                   const unsigned long long *__restrict__ masks,
-                                                  uint32_t *__restrict__ vals) {
+                                                  uint32_t *__restrict__ vals, OrderPlan plan) {
     wait_prior_grid();
     constexpr int kW = kChunk / 32;
     // per (warp, slot): where the warp's entries of the slot's tile start in the
     // final list (clipped to the capacity), and the lanes whose entry it lists
     __shared__ uint2 place[kW][64];
     __shared__ uint32_t before[kChunk / 64][64];         // partial sums of earlier chunks' counts
+    if ((int)blockIdx.x < plan.blocks) {
+        order_tiles(plan, reinterpret_cast<uint32_t *>(&place[0][0]));
+        return;
+    }
     const uint32_t nc = chunk_base[ns], cap = (uint32_t)capacity;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt = lanemask_lt();
-    for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
+    for (uint32_t c = blockIdx.x - plan.blocks; c < nc; c += gridDim.x - plan.blocks) {
         ChunkCtx cx;
         chunk_load(cx, c, splats, nullptr, svals, chunk_rec, supers_x, cam, TestScratch{}, masks, nullptr);
         const uint32_t lo = (uint32_t)cx.mask, hi = (uint32_t)(cx.mask >> 32);
@@ -1290,6 +1330,8 @@ struct SortWs {
     DepthSpan *span;
     uint32_t *seg_lo, *seg_hi, *chunk_base;    // [ns], [ns], [ns + 1]
     uint32_t *tile_count;                      // [tiles]
+    uint32_t *len_hist, *len_next;             // [kLenBuckets] tiles per length bucket, places given out
+    SortFront front;
     unsigned long long *tile_start;            // [tiles]
     uint32_t *chunk_counts;                    // [max chunks][64]
     uint4 *chunk_rec;                          // [max chunks]
@@ -1313,6 +1355,8 @@ inline SortWs sort_layout(char *base, int64_t n, int64_t cap, int64_t tiles, int
         off += align256(bytes);
         return p;
     };
+    w.front = sort_front(base, tiles);  // first: found by the rasteriser from the grid alone
+    take(w.front.bytes);
     for (int k = 0; k < 2; ++k) w.kv[k] = (uint2 *)take(8 * (size_t)n);
     w.order = (uint32_t *)w.kv[0];  // written by the pass that reads kv[1]
     w.entries[0] = (uint2 *)take(8 * (size_t)cap);
@@ -1331,10 +1375,12 @@ inline SortWs sort_layout(char *base, int64_t n, int64_t cap, int64_t tiles, int
     w.n_vis = (uint32_t *)take(4);
     w.span = (DepthSpan *)take(sizeof(DepthSpan));
     w.sclip = (uint32_t *)take(4);
-    // zeroed together before each sort: segment bounds, then tile counts
-    w.seg_lo = (uint32_t *)take(4 * (size_t)(2 * ns + tiles));
+    // zeroed together before each sort: segment bounds, tile counts, length buckets
+    w.seg_lo = (uint32_t *)take(4 * (size_t)(2 * ns + tiles + 2 * kLenBuckets));
     w.seg_hi = w.seg_lo ? w.seg_lo + ns : nullptr;
     w.tile_count = w.seg_lo ? w.seg_lo + 2 * ns : nullptr;
+    w.len_hist = w.seg_lo ? w.tile_count + tiles : nullptr;
+    w.len_next = w.seg_lo ? w.len_hist + kLenBuckets : nullptr;
     w.chunk_base = (uint32_t *)take(4 * (size_t)(ns + 1));
     w.chunk_rec = (uint4 *)take(16 * (size_t)max_chunks(cap, ns));
     w.tile_part = (unsigned long long *)take(8 * (size_t)((tiles + kScanBlock - 1) / kScanBlock));
@@ -1430,7 +1476,7 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
     // stage 1: visible Gaussians by depth (the first kernel also zeroes the
     // segment bounds, tile counts, digit counts and exact count)
     const ZeroSpans z{{w.seg_lo, w.hist_d, w.hist_s},
-                      {2 * sg.ns + tiles, kDepthPasses * kMaxRadix * chunk_rows(n),
+                      {2 * sg.ns + tiles + 2 * kLenBuckets, kDepthPasses * kMaxRadix * chunk_rows(n),
                        capacity ? npass * kMaxRadix * chunk_rows(capacity) : 0}};
     const unsigned vgrid = vis_blocks(n), egrid = entry_blocks(n);
     const size_t hstride = (size_t)chunk_rows(n) * kMaxRadix;
@@ -1477,6 +1523,10 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
     }
     launch_chained(k_chunk_counts, cgrid, kChunk, s, splats, w.cull, w.svals, w.chunk_base, w.chunk_rec, ns,
                    sg.supers_x, dc, w.chunk_counts, w.tile_count, w.masks);
+    OrderPlan plan{};
+    if (tiles >= kOrderMinTiles)
+        plan = OrderPlan{(int)((tiles + kOrderTiles - 1) / kOrderTiles), w.tile_count, w.len_hist, w.len_next, w.front,
+                         (int)tiles, tile_order_key(dc.tiles_x, dc.tiles_y, dc.tile)};
     const int tb = (int)((tiles + kScanBlock - 1) / kScanBlock);
     const bool direct = tb <= kDirectTiles;
     if (!direct) {
@@ -1484,9 +1534,9 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
         note_launches(1);
     }
     launch_chained(k_tile_starts, tb, kScanBlock, s, w.tile_count, tiles, direct ? nullptr : w.tile_part, capacity,
-                   w.total_s, w.total_exact, w.tile_start, ranges, count_dev);
-    launch_chained(k_expand, cgrid, kChunk, s, splats, w.svals, w.chunk_base, w.chunk_rec, ns, sg.supers_x, dc,
-                   w.chunk_counts, w.tile_start, capacity, w.masks, vals);
+                   w.total_s, w.total_exact, w.tile_start, ranges, count_dev, plan.blocks ? w.len_hist : nullptr);
+    launch_chained(k_expand, cgrid + plan.blocks, kChunk, s, splats, w.svals, w.chunk_base, w.chunk_rec, ns, sg.supers_x, dc,
+                   w.chunk_counts, w.tile_start, capacity, w.masks, vals, plan);
     note_launches(3);  // chunk counts, tile starts, lists
     return launch_status();
 }

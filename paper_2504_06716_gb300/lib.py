@@ -85,6 +85,10 @@ _SIGS = {
     "gs_render_fwd_resume": ([_P, _P, _P, _CAM, ctypes.POINTER(GsRasterConfig), _P, _P, _P, _P, _P, _P, _P], _I32),
     "gs_raster_bwd_resume": ([_P, _P, _P, _CAM, ctypes.POINTER(GsRasterConfig), _P, _P, _P, _P, _P, _P, _P, _P],
                              _I32),
+    "gs_render_fwd_sorted": ([_P, _P, _P, _CAM, ctypes.POINTER(GsRasterConfig), _P, _P, _P, _P, _P, _P, _P, _SZ, _P],
+                             _I32),
+    "gs_raster_bwd_sorted": ([_P, _P, _P, _CAM, ctypes.POINTER(GsRasterConfig), _P, _P, _P, _P, _P, _P, _P, _P, _SZ,
+                              _P], _I32),
     "gs_loss_workspace_bytes": ([_I32, _I32], _SZ),
     "gs_loss": ([_P, _P, _I32, _I32, _F32, _P, _SZ, _P, _P, _P], _I32),
     "gs_raster_bwd": ([_P, _P, _P, _CAM, _P, _P, _P, _P, _P, _P], _I32),
@@ -273,6 +277,36 @@ def gs_raster_bwd_resume(splats, vals, ranges, cam: GsCamera, cfg, t_final, n_la
         _ptr(n_last, torch.int32, "n_last"), _ptr(dl_dimage, torch.float32, "dl_dimage"),
         _ptr(frozen, torch.uint8, "frozen"), _ptr(resume, torch.float32, "resume"),
         _ptr(resume_pos, torch.int32, "resume_pos"), _ptr(grad2d, torch.float32, "grad2d"), _stream(stream)))
+
+
+def gs_render_fwd_sorted(splats, vals, ranges, cam: GsCamera, cfg, frozen, image, t_final, n_last, resume, resume_pos,
+                         sort_ws, stream=None):
+    """gs_render_fwd_resume, longest lists first; sort_ws: workspace of the gs_sort that made the lists."""
+    import torch
+
+    _resume_sizes(cam, resume, resume_pos)
+    _check("gs_render_fwd_sorted", load().gs_render_fwd_sorted(
+        _ptr(splats, torch.float32, "splats"), _ptr(vals, torch.int32, "vals"), _ptr(ranges, torch.int32, "ranges"),
+        ctypes.byref(cam), None if cfg is None else ctypes.byref(cfg), _ptr(frozen, torch.uint8, "frozen"),
+        _ptr(image, torch.float32, "image"), _ptr(t_final, torch.float32, "t_final"),
+        _ptr(n_last, torch.int32, "n_last"), _ptr(resume, torch.float32, "resume"),
+        _ptr(resume_pos, torch.int32, "resume_pos"), _ptr(sort_ws, torch.uint8, "sort_ws"), sort_ws.numel(),
+        _stream(stream)))
+
+
+def gs_raster_bwd_sorted(splats, vals, ranges, cam: GsCamera, cfg, t_final, n_last, dl_dimage, frozen, resume,
+                         resume_pos, grad2d, sort_ws, stream=None):
+    """gs_raster_bwd_resume, longest lists first; sort_ws: workspace of the gs_sort that made the lists."""
+    import torch
+
+    _resume_sizes(cam, resume, resume_pos)
+    _check("gs_raster_bwd_sorted", load().gs_raster_bwd_sorted(
+        _ptr(splats, torch.float32, "splats"), _ptr(vals, torch.int32, "vals"), _ptr(ranges, torch.int32, "ranges"),
+        ctypes.byref(cam), None if cfg is None else ctypes.byref(cfg), _ptr(t_final, torch.float32, "t_final"),
+        _ptr(n_last, torch.int32, "n_last"), _ptr(dl_dimage, torch.float32, "dl_dimage"),
+        _ptr(frozen, torch.uint8, "frozen"), _ptr(resume, torch.float32, "resume"),
+        _ptr(resume_pos, torch.int32, "resume_pos"), _ptr(grad2d, torch.float32, "grad2d"),
+        _ptr(sort_ws, torch.uint8, "sort_ws"), sort_ws.numel(), _stream(stream)))
 
 
 def gs_raster_bwd_cfg(splats, vals, ranges, cam: GsCamera, cfg, t_final, n_last, dl_dimage, frozen, grad2d,

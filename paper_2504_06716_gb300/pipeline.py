@@ -294,23 +294,16 @@ class Model:
         """The compositing forward; on a trainable view it also records where
         the backward resumes (gs_render_fwd_resume)."""
         cfg = self.fwd_cfg if cfg is None else cfg
-        if view.resume is not None:
-            lib.gs_render_fwd_resume(self.splats, view.vals, view.ranges, view.cam, cfg, self.frozen, view.image,
-                                     view.t_final, view.n_last, view.resume, view.resume_pos, stream)
-        else:
-            lib.gs_render_fwd_cfg(self.splats, view.vals, view.ranges, view.cam, cfg, view.image, view.t_final,
-                                  view.n_last, stream)
+        frozen = self.frozen if view.resume is not None else None
+        lib.gs_render_fwd_sorted(self.splats, view.vals, view.ranges, view.cam, cfg, frozen, view.image, view.t_final,
+                                 view.n_last, view.resume, view.resume_pos, view.sort_ws, stream)
 
     def raster_bwd(self, view: View, cfg=None, stream=None):
         """The rasteriser backward, from the forward's resume record when the
         view has one (the frozen splats behind a tile's last unfrozen one skipped)."""
         cfg = self.bwd_cfg if cfg is None else cfg
-        if view.resume is not None:
-            lib.gs_raster_bwd_resume(self.splats, view.vals, view.ranges, view.cam, cfg, view.t_final, view.n_last,
-                                     view.dl, self.frozen, view.resume, view.resume_pos, self.grad2d, stream)
-        else:
-            lib.gs_raster_bwd_cfg(self.splats, view.vals, view.ranges, view.cam, cfg, view.t_final, view.n_last,
-                                  view.dl, self.frozen, self.grad2d, stream)
+        lib.gs_raster_bwd_sorted(self.splats, view.vals, view.ranges, view.cam, cfg, view.t_final, view.n_last, view.dl,
+                                 self.frozen, view.resume, view.resume_pos, self.grad2d, view.sort_ws, stream)
 
     def loss(self, view: View, gt: torch.Tensor, lam: float = 0.2, stream=None):
         lib.gs_loss(view.image, gt, view.cam.height, view.cam.width, lam, view.loss_ws, view.loss, view.dl, stream)
