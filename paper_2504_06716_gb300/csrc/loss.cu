@@ -46,7 +46,8 @@ struct Win {
 // Bound by instruction issue (66-71%) and, at its four blocks per SM, by the
 // two barriers between the passes. 3 x 822 x 1237: 68.4 us with scalar passes, a
 // counted last block and a cleared counter; 61.8 us with packed passes; 50.0 us
-// with the reduction in the backward.
+// with the reduction in the backward; 48.5 us with the backward's pixels loaded ahead
+// of its last windows.
 constexpr int kV = 4;
 constexpr int kSeg = kT / kV;              // 8 segments per row / column
 constexpr int kHItems = kE * kSeg;         // 336 horizontal items
@@ -306,6 +307,15 @@ __global__ void __launch_bounds__(kLossThreads, 5) k_ssim_bwd(const float *__res
     __syncthreads();
     const float invN = 1.f / (3.f * (float)HW);
     const int cc = threadIdx.x % kT, r0 = (threadIdx.x / kT) * kV;
+    const int gx = blockIdx.x * kT + cc, gy0 = blockIdx.y * kT + r0;
+    float xv[kV], yv[kV];  // on their way while the windows are summed
+#pragma unroll
+    for (int v = 0; v < kV; ++v) {
+        const bool in = gx < W && gy0 + v < H;
+        const int64_t o = ch * HW + (int64_t)(gy0 + v) * W + gx;
+        xv[v] = in ? __ldg(img + o) : 0.f;
+        yv[v] = in ? __ldg(gt + o) : 0.f;
+    }
     f32x2 p[1][kV];
     float s0[kV], s1[kV], s2[kV];
     window<1>(win, [&](int q, f32x2 (&o)[1], float &z) { o[0] = h[r0 + q][cc]; z = hc[r0 + q][cc]; }, p, s2);
@@ -313,16 +323,13 @@ __global__ void __launch_bounds__(kLossThreads, 5) k_ssim_bwd(const float *__res
     for (int v = 0; v < kV; ++v) f2_unpack(p[0][v], s0[v], s1[v]);
 #pragma unroll
     for (int v = 0; v < kV; ++v) {
-        const int gy = blockIdx.y * kT + r0 + v, gx = blockIdx.x * kT + cc;
-        if (gy >= H || gx >= W) continue;
-        const int64_t p = ch * HW + (int64_t)gy * W + gx;
-        const float xv = __ldg(img + p), yv = __ldg(gt + p);
-        const float d = xv - yv;
+        if (gx >= W || gy0 + v >= H) continue;
+        const float d = xv[v] - yv[v];
         const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
-        const float dssim = s0[v] + 2.f * xv * s1[v] + yv * s2[v];
+        const float dssim = s0[v] + 2.f * xv[v] * s1[v] + yv[v] * s2[v];
         const float g = ((1.f - lambda) * sg - lambda * dssim) * invN;
         if (!isfinite(g)) atomicOr(&g_loss_flags, GS_FLAG_NONFINITE);
-        dl[p] = g;
+        dl[ch * HW + (int64_t)(gy0 + v) * W + gx] = g;
     }
 }
 
