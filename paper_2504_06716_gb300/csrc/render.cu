@@ -1137,9 +1137,11 @@ __global__ void __launch_bounds__(TS * TS / PPT) k_raster_bwd_batch(const gs_ras
 // workload). The backward of 16-pixel tiles takes one pixel per thread while
 // the tiles are few: below about 2048 the chip has fewer 8 x 8 blocks than
 // warps it can hold, and halving the blocks shortens every chain (100K
-// Gaussians at 512x512, 1024 tiles: 74 us against 88; 50K at 320x240 58
-// against 76); above, two per thread cost fewer instructions (800x800, 2500
-// tiles: 172 against 174; 200K at 1237x822 132 against 154).
+// Gaussians at 512x512, 1024 tiles: 67 us against 76; 50K at 320x240 47 against
+// 55); above, two per thread cost fewer instructions (surface scenes, 120K at
+// 800x800 74 us against 87, 400K 195 against 219, 200K at 1237x822 160 against
+// 196; where a few tiles are far longer than the rest one is better even there:
+// 400K, half frozen, 148 against 154).
 inline void default_config(int tile, int64_t tiles, bool bwd, int &ppt, int &batch) {
     if (tile == 8) { ppt = 1; batch = 64; return; }
     if (tile == 16) { ppt = bwd && tiles >= 2048 ? 2 : 1; batch = 256; return; }
