@@ -58,6 +58,13 @@ void note_launches(int k);
 
 inline int launch_status() { return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA; }
 
+// Whether a launch or another runtime call was accepted; a refusal is taken off
+// the runtime's record of the last error, since the caller returns it.
+inline bool accepted(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
+}
+
 // Two float32 values in one 64-bit register pair, and the packed FP32
 // instructions of sm_100 and later (add/sub/mul/fma .rn .f32x2): each half is
 // rounded exactly as the scalar __fadd_rn / __fsub_rn / __fmul_rn / __fmaf_rn
@@ -101,8 +108,8 @@ __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
 __device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
-inline void launch_chained_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                Args &&...args) {
+inline cudaError_t launch_chained_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                       Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -113,12 +120,12 @@ inline void launch_chained_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
 template <typename... KArgs, typename... Args>
-inline void launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args &&...args) {
-    launch_chained_smem(kernel, grid, block, 0, s, static_cast<Args &&>(args)...);
+inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args &&...args) {
+    return launch_chained_smem(kernel, grid, block, 0, s, static_cast<Args &&>(args)...);
 }
 
 inline unsigned grid_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }

@@ -1504,12 +1504,23 @@ inline Digit radix_digit(uint32_t *hist, int64_t bound, int total_bits, int p) {
     return Digit{hist_of(hist, bound, p), shift, per < total_bits - shift ? per : total_bits - shift};
 }
 
+// Lets the two kernels that need more than 48 KB of shared memory be launched
+// with the most they ever take. The limit belongs to the function on the
+// device, not to a launch: it is the same in every call and never lowered, so
+// that another thread's sort, or a captured launch replayed later, finds it.
+bool allow_shared() {
+    constexpr size_t radix_most = (sizeof(uint32_t) * (size_t)kRadixWarps) << kMaxRadixBits;  // 64 KB
+    const auto most = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    return accepted(cudaFuncSetAttribute(k_radix_pass, most, (int)radix_most)) &&
+           accepted(cudaFuncSetAttribute(k_depth_small, most, (int)kSmallShared));
+}
+
 // A radix pass over a count of at most `bound`, on a digit of at most `bits`.
 template <typename... Args>
-void launch_radix(int bits, int64_t bound, cudaStream_t s, Args &&...args) {
-    const size_t smem = (sizeof(uint32_t) * (size_t)kRadixWarps) << bits;  // 64 KB for a 9-bit digit
-    cudaFuncSetAttribute(k_radix_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);  // beyond 48 KB
-    launch_chained_smem(k_radix_pass, (unsigned)chunk_rows(bound), kRadixThreads, smem, s, static_cast<Args &&>(args)...);
+cudaError_t launch_radix(int bits, int64_t bound, cudaStream_t s, Args &&...args) {
+    const size_t smem = (sizeof(uint32_t) * (size_t)kRadixWarps) << bits;  // at most allow_shared's
+    return launch_chained_smem(k_radix_pass, (unsigned)chunk_rows(bound), kRadixThreads, smem, s,
+                               static_cast<Args &&>(args)...);
 }
 
 int ceil_log2(int64_t x) {
@@ -1559,6 +1570,9 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
         }
     }
     const int sbits = ceil_log2(sg.ns), npass = radix_passes(sbits);
+    // A launch that is refused ends the call: the kernels behind it would read as
+    // counts and indices whatever lies in the place of its output.
+    if (!allow_shared()) return GS_ERR_CUDA;
     // stage 1: visible Gaussians by depth (the first kernel also zeroes the
     // segment bounds, tile counts, digit counts and exact count)
     const ZeroSpans z{{w.seg_lo, w.hist_d, w.hist_s},
@@ -1566,32 +1580,39 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
                        capacity ? npass * kMaxRadix * chunk_rows(capacity) : 0}};
     const unsigned vgrid = vis_blocks(n), egrid = entry_blocks(n);
     const size_t hstride = (size_t)chunk_rows(n) * kMaxRadix;
-    launch_chained(k_count_visible, vgrid, kVisBlock, s, splats, n, w.part32, z, w.total_exact);
-    launch_chained(k_emit_visible, vgrid, kVisBlock, s, splats, n, w.part32, dc, w.kv[0], w.kv[1], w.cull,
-                   w.n_vis, w.span, w.hist_d, hstride);
+    if (!accepted(launch_chained(k_count_visible, vgrid, kVisBlock, s, splats, n, w.part32, z, w.total_exact)))
+        return GS_ERR_CUDA;
+    if (!accepted(launch_chained(k_emit_visible, vgrid, kVisBlock, s, splats, n, w.part32, dc, w.kv[0], w.kv[1],
+                                 w.cull, w.n_vis, w.span, w.hist_d, hstride)))
+        return GS_ERR_CUDA;
     if (n <= kSmallSort) {
-        cudaFuncSetAttribute(k_depth_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallShared);
-        launch_chained_smem(k_depth_small, 1, kRadixThreads, kSmallShared, s, w.kv[0], w.kv[1], w.order, w.n_vis,
-                            w.span);
+        if (!accepted(launch_chained_smem(k_depth_small, 1, kRadixThreads, kSmallShared, s, w.kv[0], w.kv[1], w.order,
+                                          w.n_vis, w.span)))
+            return GS_ERR_CUDA;
         note_launches(3);
     } else {
         for (int k = 0; k < kDepthPasses; ++k)
-            launch_radix(kMaxRadixBits, n, s, w.kv[k & 1], w.kv[1 - (k & 1)], static_cast<uint32_t *>(nullptr),
-                         k == 3 ? w.order : nullptr, w.n_vis, Digit{w.hist_d, 0, 0}, Digit{nullptr, 0, 0}, w.span, k,
-                         hstride, SegPlan{});
+            if (!accepted(launch_radix(kMaxRadixBits, n, s, w.kv[k & 1], w.kv[1 - (k & 1)],
+                                       static_cast<uint32_t *>(nullptr), k == 3 ? w.order : nullptr, w.n_vis,
+                                       Digit{w.hist_d, 0, 0}, Digit{nullptr, 0, 0}, w.span, k, hstride, SegPlan{})))
+                return GS_ERR_CUDA;
         note_launches(2 + kDepthPasses);
     }
     const uint32_t *order = w.order;
     // stage 2: super-tile entries in depth order, stable-sorted by super-tile
-    launch_chained(k_count_entries, egrid, kVisBlock, s, w.cull, order, w.n_vis, w.part_s);
+    if (!accepted(launch_chained(k_count_entries, egrid, kVisBlock, s, w.cull, order, w.n_vis, w.part_s)))
+        return GS_ERR_CUDA;
     note_launches(1);
-    launch_chained(k_emit_super, egrid, kVisBlock, s, splats, w.cull, order, w.n_vis, dc, sg.supers_x, w.part_s,
-                   w.total_s, w.sclip, capacity, w.entries[0], w.skeys, w.svals, w.total_exact,
-                   capacity ? radix_digit(w.hist_s, capacity, sbits, 0) : Digit{nullptr, 0, 0});
+    if (!accepted(launch_chained(k_emit_super, egrid, kVisBlock, s, splats, w.cull, order, w.n_vis, dc, sg.supers_x,
+                                 w.part_s, w.total_s, w.sclip, capacity, w.entries[0], w.skeys, w.svals, w.total_exact,
+                                 capacity ? radix_digit(w.hist_s, capacity, sbits, 0) : Digit{nullptr, 0, 0})))
+        return GS_ERR_CUDA;
     note_launches(1);
     if (capacity == 0) {
         cudaMemsetAsync(w.total_t, 0, sizeof(unsigned long long), s);
-        launch_chained(k_finish_count, 1, 1, s, w.total_t, w.total_s, w.total_exact, capacity, count_dev);
+        if (!accepted(launch_chained(k_finish_count, 1, 1, s, w.total_t, w.total_s, w.total_exact, capacity,
+                                     count_dev)))
+            return GS_ERR_CUDA;
         note_launches(1);
         return launch_status();
     }
@@ -1600,22 +1621,26 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
     for (int p = 0; p < npass; ++p) {
         const bool last = p == npass - 1;
         const Digit dg = radix_digit(w.hist_s, capacity, sbits, p);
-        launch_radix(dg.bits, capacity, s, w.entries[p], w.entries[1], last && npass == 2 ? w.skeys : nullptr,
-                     last ? w.svals : nullptr, w.sclip, dg, radix_digit(w.hist_s, capacity, sbits, p + 1),
-                     static_cast<DepthSpan *>(nullptr), 0, size_t(0),
-                     npass == 1 ? SegPlan{w.chunk_base, w.chunk_rec, ns, kChunk} : SegPlan{});
+        if (!accepted(launch_radix(dg.bits, capacity, s, w.entries[p], w.entries[1],
+                                   last && npass == 2 ? w.skeys : nullptr, last ? w.svals : nullptr, w.sclip, dg,
+                                   radix_digit(w.hist_s, capacity, sbits, p + 1), static_cast<DepthSpan *>(nullptr), 0,
+                                   size_t(0), npass == 1 ? SegPlan{w.chunk_base, w.chunk_rec, ns, kChunk} : SegPlan{})))
+            return GS_ERR_CUDA;
         note_launches(1);
     }
     // stage 3: per-tile lists
     const int64_t chunks = max_chunks(capacity, sg.ns), resident = resident_blocks();
     const unsigned cgrid = (unsigned)(chunks < resident ? chunks : resident);
     if (npass != 1) {
-        launch_chained(k_seg_mark, (unsigned)resident, 256, s, w.skeys, w.sclip, w.seg_lo, w.seg_hi);
-        launch_chained(k_super_plan, 1, 1024, s, w.seg_lo, w.seg_hi, ns, w.chunk_base, w.chunk_rec);
+        if (!accepted(launch_chained(k_seg_mark, (unsigned)resident, 256, s, w.skeys, w.sclip, w.seg_lo, w.seg_hi)))
+            return GS_ERR_CUDA;
+        if (!accepted(launch_chained(k_super_plan, 1, 1024, s, w.seg_lo, w.seg_hi, ns, w.chunk_base, w.chunk_rec)))
+            return GS_ERR_CUDA;
         note_launches(2);
     }
-    launch_chained(k_chunk_counts, cgrid, kChunk, s, splats, w.cull, w.svals, w.chunk_base, w.chunk_rec, ns,
-                   sg.supers_x, dc, w.chunk_counts, w.tile_count, w.masks);
+    if (!accepted(launch_chained(k_chunk_counts, cgrid, kChunk, s, splats, w.cull, w.svals, w.chunk_base, w.chunk_rec,
+                                 ns, sg.supers_x, dc, w.chunk_counts, w.tile_count, w.masks)))
+        return GS_ERR_CUDA;
     OrderPlan plan{};
     if (tiles >= kOrderMinTiles)
         plan = OrderPlan{(int)((tiles + kOrderTiles - 1) / kOrderTiles), w.tile_count, w.len_hist, w.len_next, w.front,
@@ -1623,13 +1648,17 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
     const int tb = (int)((tiles + kScanBlock - 1) / kScanBlock);
     const bool direct = tb <= kDirectTiles;
     if (!direct) {
-        launch_chained(k_tile_sums, tb, kScanBlock, s, w.tile_count, tiles, w.tile_part);
+        if (!accepted(launch_chained(k_tile_sums, tb, kScanBlock, s, w.tile_count, tiles, w.tile_part)))
+            return GS_ERR_CUDA;
         note_launches(1);
     }
-    launch_chained(k_tile_starts, tb, kScanBlock, s, w.tile_count, tiles, direct ? nullptr : w.tile_part, capacity,
-                   w.total_s, w.total_exact, w.tile_start, ranges, count_dev, plan.blocks ? w.len_hist : nullptr);
-    launch_chained(k_expand, cgrid + plan.blocks, kChunk, s, splats, w.svals, w.chunk_base, w.chunk_rec, ns, sg.supers_x, dc,
-                   w.chunk_counts, w.tile_start, capacity, w.masks, vals, plan);
+    if (!accepted(launch_chained(k_tile_starts, tb, kScanBlock, s, w.tile_count, tiles,
+                                 direct ? nullptr : w.tile_part, capacity, w.total_s, w.total_exact, w.tile_start,
+                                 ranges, count_dev, plan.blocks ? w.len_hist : nullptr)))
+        return GS_ERR_CUDA;
+    if (!accepted(launch_chained(k_expand, cgrid + plan.blocks, kChunk, s, splats, w.svals, w.chunk_base, w.chunk_rec,
+                                 ns, sg.supers_x, dc, w.chunk_counts, w.tile_start, capacity, w.masks, vals, plan)))
+        return GS_ERR_CUDA;
     note_launches(3);  // chunk counts, tile starts, lists
     return launch_status();
 }
