@@ -29,10 +29,17 @@ constexpr int kDB = 256;  // Gaussians per block
 constexpr uint8_t kKeep = 1, kClone = 2, kSplit = 4, kChild = 8;
 
 __device__ __forceinline__ uint8_t den_flags(const float *__restrict__ P, const gs_grad_stats st,
-                                             const gs_densify_params &p, int64_t i) {
-    // everything the decision reads, in flight together
-    const float4 *row = reinterpret_cast<const float4 *>(P + i * kRow);
-    const float4 r0 = __ldg(row), r1 = __ldg(row + 1), r2 = __ldg(row + 2);
+                                             const gs_densify_params &p, int64_t i, bool vec) {
+    // everything the decision reads, in flight together; 16 bytes at a time where
+    // P is so aligned (vec), which the plan does not ask of its caller
+    const float *r = P + i * kRow;
+    float4 r0, r1, r2;
+    if (vec) {
+        const float4 *row = reinterpret_cast<const float4 *>(r);
+        r0 = __ldg(row), r1 = __ldg(row + 1), r2 = __ldg(row + 2);
+    } else {
+        r0.w = r[3], r1.x = r[4], r1.y = r[5], r2.z = r[10];
+    }
     const int32_t c = st.cnt[i];
     const float acc_xyz = st.acc_xyz[i], acc_rgb = st.acc_rgb[i];
     bool cand = false;
@@ -45,7 +52,7 @@ __device__ __forceinline__ uint8_t den_flags(const float *__restrict__ P, const 
     const bool clone = cand && smax <= p.log_clone_max;
     const bool split = cand && !clone;
     // low opacity, or a volume mask that is off (its logit at most logit(0.01))
-    const bool low = r2.z < p.logit_min_opacity || (p.mask_prune && !(P[i * kRow + 59] > p.mask_logit_min)) ||
+    const bool low = r2.z < p.logit_min_opacity || (p.mask_prune && !(r[59] > p.mask_logit_min)) ||
                      (p.prune_mark && p.prune_mark[i]);
     bool big_world = false, big_child = false, big_screen = false;
     if (p.prune_big) {
@@ -102,11 +109,11 @@ __device__ __forceinline__ Quad block_scan4(Quad q, Quad *total) {
 
 __global__ void __launch_bounds__(kDB) k_den_plan(int64_t n, const float *__restrict__ P, gs_grad_stats st,
                                                   gs_densify_params p, uint8_t *__restrict__ flags,
-                                                  uint32_t *__restrict__ part, int nb) {
+                                                  uint32_t *__restrict__ part, int nb, bool vec) {
     const int64_t i = (int64_t)blockIdx.x * kDB + threadIdx.x;
     uint8_t f = 0;
     if (i < n) {
-        f = den_flags(P, st, p, i);
+        f = den_flags(P, st, p, i, vec);
         flags[i] = f;
     }
     Quad tot;
@@ -368,7 +375,7 @@ extern "C" int gs_densify_plan(int64_t n, const float *P, const gs_grad_stats *s
     }
     if (!P || !stats->acc_xyz || !stats->acc_rgb || !stats->cnt) return GS_ERR_INVALID_ARG;
     const int nb = (int)((n + kDB - 1) / kDB);
-    k_den_plan<<<nb, kDB, 0, s>>>(n, P, *stats, *prm, w.flags, w.part, nb);
+    k_den_plan<<<nb, kDB, 0, s>>>(n, P, *stats, *prm, w.flags, w.part, nb, (reinterpret_cast<uintptr_t>(P) & 15) == 0);
     k_den_scan<<<4, 1024, 0, s>>>(w.part, nb, w.totals, counts_dev);
     note_launches(2);
     return launch_status();
