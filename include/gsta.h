@@ -167,8 +167,8 @@ int gs_render_fwd(const float *splats, const uint32_t *vals, const uint32_t *ran
  * camera's tile size. */
 typedef struct {
     int32_t pixels_per_thread; /* pixels each thread composites: 1, 2, or 4 (tiles of 16 and 32) */
-    int32_t batch;             /* list entries per batch: 32, 64, 128 or 256 (the resume record of
-                                * gs_render_fwd_resume keeps one state per batch) */
+    int32_t batch;             /* 32, 64, 128 or 256; no kernel stages by it any more, so neither results
+                                * nor times depend on it */
 } gs_raster_config;
 
 /* Sec. 3.1, Eq. 2: gs_render_fwd with an explicit launch shape (cfg may be
@@ -213,10 +213,12 @@ int gs_raster_bwd_cfg(const float *splats, const uint32_t *vals, const uint32_t 
  * one only to rebuild the transmittance in front of it and the colour
  * blended behind it, so the forward records those: gs_render_fwd_resume is
  * gs_render_fwd_cfg that also writes, for each tile, resume_pos [tiles]
- * (int32) = 1 + the list position of the last splat with frozen[i] == 0 the
- * tile's walk passed (0 if none; frozen may be NULL: nothing frozen), and
- * for each pixel resume [H][W][4] (float, 16-byte aligned) = (T after that
- * splat, the colour blended behind it). gs_raster_bwd_resume is
+ * (int32) = 1 + the list position of a splat with frozen[i] == 0 behind
+ * which the tile's walk passed none (0 if there is none; frozen may be NULL:
+ * nothing frozen): of the 32 list entries among which the walk ends the last
+ * unfrozen one, or, if they have none, the last in front of them. For each
+ * pixel resume [H][W][4] (float, 16-byte aligned) = (T after that splat, the
+ * colour blended behind it). gs_raster_bwd_resume is
  * gs_raster_bwd_cfg that starts each tile's walk there from that state,
  * given the buffers of the forward of the same lists and freeze map; its
  * gradients equal gs_raster_bwd_cfg's up to float32 rounding (the state is

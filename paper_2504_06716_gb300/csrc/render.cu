@@ -168,13 +168,17 @@ __device__ __forceinline__ void alphas(V px, V py, const V4<V> &a, const V4<V> &
 // them -- and the stop T < 1e-4 is tested once per G, on the last T (T never
 // grows): only a group that crosses it is gone through splat by splat.
 //
-// With RES, the walk also records where the backward may start: in every
-// batch of `batch` list entries, the state after its last unfrozen splat is
-// kept if some pixel of the tile is still alive when the walk gets there;
-// resume_pos[tile] = 1 + that splat's list position (0 if none), and per
-// pixel resume = (T after that splat, the colour blended behind it), so that
-// the backward skips the frozen splats behind it: they carry no gradient,
-// and the state they would rebuild is this one.
+// With RES, the walk also records where the backward may start: of every 32
+// list entries that have an unfrozen one, the state after the last of them
+// (resume_pos[tile] = 1 + its list position, 0 if the tile has none; per pixel
+// resume = (T there, the colour blended behind it)), so that the backward
+// skips the frozen splats behind it: they carry no gradient, and the state
+// they would rebuild is this one. Rays that all stop in front of that entry,
+// but among its 32, have their final state there: no unfrozen splat that was
+// blended lies behind the recorded position, and at most 31 frozen ones in
+// front of it are visited for nothing. The position depends on the list, the
+// freeze map and the tile's deepest ray alone, not on how the tile is cut
+// into warps: the groups of 32 are the list's, and the deepest warp's decides.
 //
 // Measured against the kernel before it (a barrier-separated batch per CTA,
 // done flags and a stop test per splat, every warp through the whole tile's
@@ -186,7 +190,7 @@ template <int TS, int PPT, bool RES>
 __device__ __forceinline__ void render_tile(const float *__restrict__ splats, const uint32_t *__restrict__ vals,
                                             const uint32_t *__restrict__ ranges, const DevCam &cam,
                                             float *__restrict__ image, float *__restrict__ t_final,
-                                            int32_t *__restrict__ n_last, int tile, int batch = 0,
+                                            int32_t *__restrict__ n_last, int tile,
                                             const uint8_t *__restrict__ frozen = nullptr,
                                             float4 *__restrict__ resume = nullptr,
                                             int32_t *__restrict__ resume_pos = nullptr,
@@ -229,7 +233,7 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
         hit_last[k] = -1;
     }
     float4 u[PPT];  // RES: T and colour after the last unfrozen splat passed
-    int upos = 0, stop_at = -1, snap_at = -1;  // snap_at: the staged splat the snapshot is taken after
+    int upos = 0, snap_at = -1;  // snap_at: the staged splat the snapshot is yet to be taken after
     auto state = [&](float4 (&o)[PPT]) {
 #pragma unroll
         for (int h = 0; h < NP; ++h) {
@@ -240,6 +244,7 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
         }
     };
     auto snapshot = [&]() {
+        snap_at = -1;
         state(u);
         if (kSnapShared) {
 #pragma unroll
@@ -256,7 +261,7 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
     };
 
     // Staged splats j .. j + G - 1 for this thread's pixels; true once all
-    // pixels of the warp are done (stop_at: the staged splat that ended the last).
+    // pixels of the warp are done.
     auto blend = [&](auto Gc, int j) -> bool {
         constexpr int G = decltype(Gc)::value;
         float al[G][NP][L];
@@ -300,28 +305,21 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
         }
         const bool any_stop = __any_sync(kFull, stop);
         if (any_stop) {  // some ray ends in this group, before the splat that would take T below the floor
-            if (RES) stop_at = -1;
 #pragma unroll
             for (int h = 0; h < NP; ++h) {
-                int at[L];
-#pragma unroll
-                for (int l = 0; l < L; ++l) at[l] = -1;
-#pragma unroll
-                for (int i = G - 1; i >= 0; --i) {
-                    float e[L];
-                    v_get(t[i + 1][h], e);
-#pragma unroll
-                    for (int l = 0; l < L; ++l) {
-                        at[l] = e[l] < kTMin ? j + i : at[l];
-                        al[i][h][l] = e[l] < kTMin ? 0.f : al[i][h][l];
-                    }
-                }
+                float e[L];
+                v_get(t[G][h], e);
 #pragma unroll
                 for (int l = 0; l < L; ++l) {
                     const int k = L * h + l;
-                    if (RES) stop_at = max(stop_at, at[l]);
-                    fy[k] = at[l] >= 0 ? nan : fy[k];
+                    fy[k] = e[l] < kTMin ? nan : fy[k];  // T never grows: the last one is below if any is
                     hit_last[k] = before[k];
+                }
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+                    v_get(t[i + 1][h], e);
+#pragma unroll
+                    for (int l = 0; l < L; ++l) al[i][h][l] = e[l] < kTMin ? 0.f : al[i][h][l];
                 }
 #pragma unroll
                 for (int i = 0; i < G; ++i) {
@@ -384,24 +382,7 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
         }
         if (lane + kStage < n) g1 = list[lane + kStage];
     }
-    // RES: a snapshot is taken at the last unfrozen entry of every 32; when its
-    // batch has been walked to the end it is kept (written to the record), and
-    // when the walk ends inside a batch it counts only if it is the batch's
-    // last unfrozen entry, else the state kept before is the one.
-    int kept = 0, batch_end = batch;
-    auto keep = [&]() {
-        kept = upos;
-#pragma unroll
-        for (int k = 0; k < PPT; ++k) {
-            const int y = py0 + 4 * k;
-            if (px < cam.W && y < cam.H) resume[(int64_t)y * cam.W + px] = snapped(k);
-        }
-    };
     for (int base = 0; base < n && !dead; base += kStage) {
-        if (RES && base == batch_end) {
-            if (upos != kept) keep();
-            batch_end += batch;
-        }
         const bool valid = base + lane < n;
         bool hit = valid;
         if (!kWholeTile && valid)
@@ -427,33 +408,14 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
         }
         int j = 0;
         dead = walk(j, cnt);
-        bool cut = false;  // the walk ended in front of an unfrozen entry of its batch
         if (RES && wake) {
-            snap_at = -1;
+            if (snap_at >= 0) snapshot();  // every ray stopped in front of that entry: final
             upos = base + lu + 1;
-            if (dead) {
-                const int e = __reduce_max_sync(kFull, stop_at);
-                cut = (kWholeTile ? e : (int)S.pos[e]) < lu;
-            }
         }
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
             if (hit_last[k] >= 0) last[k] = base + 1 + (kWholeTile ? hit_last[k] : (int)S.pos[hit_last[k]]);
             hit_last[k] = -1;
-        }
-        if (RES && dead && upos != kept) {
-            for (int q = base + kStage; q < min(n, batch_end) && !cut; q += kStage)
-                cut = __any_sync(kFull, q + lane < min(n, batch_end) && !(frozen && frozen[list[q + lane]]));
-            if (cut) {  // back to the state kept before
-                upos = kept;
-#pragma unroll
-                for (int k = 0; k < PPT; ++k) {
-                    const int y = py0 + 4 * k;
-                    const bool in = kept > 0 && px < cam.W && y < cam.H;
-                    u[k] = in ? resume[(int64_t)y * cam.W + px] : make_float4(1.f, 0.f, 0.f, 0.f);
-                    if (kSnapShared) s_snap[k * (TS * TS / PPT) + threadIdx.x] = u[k];
-                }
-            }
         }
         __syncwarp();  // the staged splats are no longer read
     }
@@ -515,11 +477,11 @@ template <int TS, int PPT, bool RES>
 __global__ void __launch_bounds__(TS * TS / PPT, fwd_blocks<TS, PPT, RES>())
     k_render_fwd(const float *__restrict__ splats, const uint32_t *__restrict__ vals, const uint32_t *__restrict__ ranges,
                  DevCam cam, float *__restrict__ image, float *__restrict__ t_final, int32_t *__restrict__ n_last,
-                 int batch, const uint8_t *__restrict__ frozen, float4 *__restrict__ resume,
+                 const uint8_t *__restrict__ frozen, float4 *__restrict__ resume,
                  int32_t *__restrict__ resume_pos, TileOrder order, int32_t *__restrict__ depth) {
     wait_prior_grid();
-    render_tile<TS, PPT, RES>(splats, vals, ranges, cam, image, t_final, n_last, ordered_tile(order), batch, frozen,
-                              resume, resume_pos, depth);
+    render_tile<TS, PPT, RES>(splats, vals, ranges, cam, image, t_final, n_last, ordered_tile(order), frozen, resume,
+                              resume_pos, depth);
 }
 
 // Sums over a warp by recursive halving: at each xor level a lane keeps half
@@ -1132,21 +1094,19 @@ __global__ void __launch_bounds__(TS * TS / PPT) k_raster_bwd_batch(const gs_ras
     }
 }
 
-// Launch shape used when the caller gives none: pixels per thread and batch
-// size by tile size (timed on GB300; the autotuner may pick another per
-// workload). The backward of 16-pixel tiles takes one pixel per thread while
-// the tiles are few: below about 2048 the chip has fewer 8 x 8 blocks than
-// warps it can hold, and halving the blocks shortens every chain (100K
-// Gaussians at 512x512, 1024 tiles: 67 us against 76; 50K at 320x240 47 against
-// 55); above, two per thread cost fewer instructions (surface scenes, 120K at
-// 800x800 74 us against 87, 400K 195 against 219, 200K at 1237x822 160 against
-// 196; where a few tiles are far longer than the rest one is better even there:
-// 400K, half frozen, 148 against 154).
-inline void default_config(int tile, int64_t tiles, bool bwd, int &ppt, int &batch) {
-    if (tile == 8) { ppt = 1; batch = 64; return; }
-    if (tile == 16) { ppt = bwd && tiles >= 2048 ? 2 : 1; batch = 256; return; }
-    ppt = 2;
-    batch = 256;
+// Launch shape used when the caller gives none: pixels per thread by tile size
+// (timed on GB300; the autotuner may pick another per workload). The backward
+// of 16-pixel tiles takes one pixel per thread while the tiles are few: below
+// about 2048 the chip has fewer 8 x 8 blocks than warps it can hold, and halving
+// the blocks shortens every chain (100K Gaussians at 512x512, 1024 tiles: 67 us
+// against 76; 50K at 320x240 47 against 55); above, two per thread cost fewer
+// instructions (surface scenes, 120K at 800x800 74 us against 87, 400K 195
+// against 219, 200K at 1237x822 160 against 196; where a few tiles are far longer
+// than the rest one is better even there: 400K, half frozen, 148 against 154).
+inline int default_ppt(int tile, int64_t tiles, bool bwd) {
+    if (tile == 8) return 1;
+    if (tile == 16) return bwd && tiles >= 2048 ? 2 : 1;
+    return 2;
 }
 
 struct FwdArgs {
@@ -1177,18 +1137,18 @@ struct BwdArgs {
 };
 
 template <int TS, int PPT>
-void launch(int batch, const FwdArgs &a, cudaStream_t s) {
+void launch(const FwdArgs &a, cudaStream_t s) {
     const int tiles = a.cam.tiles_x * a.cam.tiles_y;
     if (a.resume)
         launch_chained(k_render_fwd<TS, PPT, true>, tiles, TS * TS / PPT, s, a.splats, a.vals, a.ranges, a.cam, a.image,
-                       a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos, a.order, a.depth);
+                       a.t_final, a.n_last, a.frozen, a.resume, a.resume_pos, a.order, a.depth);
     else
         launch_chained(k_render_fwd<TS, PPT, false>, tiles, TS * TS / PPT, s, a.splats, a.vals, a.ranges, a.cam,
-                       a.image, a.t_final, a.n_last, batch, a.frozen, a.resume, a.resume_pos, a.order, a.depth);
+                       a.image, a.t_final, a.n_last, a.frozen, a.resume, a.resume_pos, a.order, a.depth);
 }
 
 template <int TS, int PPT>
-void launch(int, const BwdArgs &a, cudaStream_t s) {
+void launch(const BwdArgs &a, cudaStream_t s) {
     launch_chained(k_raster_bwd<TS, PPT>, a.cam.tiles_x * a.cam.tiles_y, TS * TS / PPT, s, a.splats, a.vals, a.ranges,
                    a.cam, a.t_final, a.n_last, a.dl, a.frozen, a.grad2d, a.resume, a.resume_pos, a.order);
 }
@@ -1211,7 +1171,7 @@ int resident_ctas(K kernel, int threads) {
 }
 
 template <int TS, int PPT>
-void launch(int, const BatchArgs &a, cudaStream_t s) {
+void launch(const BatchArgs &a, cudaStream_t s) {
     constexpr int NT = TS * TS / PPT;
     if (a.bwd) {
         const int grid = resident_ctas(k_raster_bwd_batch<TS, PPT>, NT);
@@ -1223,16 +1183,16 @@ void launch(int, const BatchArgs &a, cudaStream_t s) {
 }
 
 template <class A>
-int dispatch(int tile, int ppt, int batch, const A &a, cudaStream_t s) {
+int dispatch(int tile, int ppt, const A &a, cudaStream_t s) {
     switch (tile * 10 + ppt) {
-        case 81: launch<8, 1>(batch, a, s); break;
-        case 82: launch<8, 2>(batch, a, s); break;
-        case 161: launch<16, 1>(batch, a, s); break;
-        case 162: launch<16, 2>(batch, a, s); break;
-        case 164: launch<16, 4>(batch, a, s); break;
-        case 321: launch<32, 1>(batch, a, s); break;
-        case 324: launch<32, 4>(batch, a, s); break;
-        default: launch<32, 2>(batch, a, s); break;
+        case 81: launch<8, 1>(a, s); break;
+        case 82: launch<8, 2>(a, s); break;
+        case 161: launch<16, 1>(a, s); break;
+        case 162: launch<16, 2>(a, s); break;
+        case 164: launch<16, 4>(a, s); break;
+        case 321: launch<32, 1>(a, s); break;
+        case 324: launch<32, 4>(a, s); break;
+        default: launch<32, 2>(a, s); break;
     }
     note_launches(1);
     return launch_status();
@@ -1261,10 +1221,9 @@ int render_fwd_ordered(const float *splats, const uint32_t *vals, const uint32_t
     if ((reinterpret_cast<uintptr_t>(splats) | reinterpret_cast<uintptr_t>(resume)) & 15) return GS_ERR_INVALID_ARG;
     FwdArgs a{splats, vals, ranges, make_cam(cam), image, t_final, n_last, frozen, reinterpret_cast<float4 *>(resume),
               resume_pos, order, depth};
-    int ppt, batch;
-    default_config(a.cam.tile, (int64_t)a.cam.tiles_x * a.cam.tiles_y, false, ppt, batch);
-    if (cfg) { ppt = cfg->pixels_per_thread; batch = cfg->batch; }
-    return dispatch(a.cam.tile, ppt, batch, a, as_stream(stream));
+    const int ppt = cfg ? cfg->pixels_per_thread
+                        : default_ppt(a.cam.tile, (int64_t)a.cam.tiles_x * a.cam.tiles_y, false);
+    return dispatch(a.cam.tile, ppt, a, as_stream(stream));
 }
 
 int raster_bwd_ordered(const float *splats, const uint32_t *vals, const uint32_t *ranges, const gs_camera *cam,
@@ -1277,10 +1236,9 @@ int raster_bwd_ordered(const float *splats, const uint32_t *vals, const uint32_t
     if ((reinterpret_cast<uintptr_t>(splats) | reinterpret_cast<uintptr_t>(resume)) & 15) return GS_ERR_INVALID_ARG;
     BwdArgs a{splats, vals, ranges, make_cam(cam), t_final, n_last, dl_dimage, frozen, grad2d,
               reinterpret_cast<const float4 *>(resume), resume_pos, order};
-    int ppt, batch;
-    default_config(a.cam.tile, (int64_t)a.cam.tiles_x * a.cam.tiles_y, true, ppt, batch);
-    if (cfg) { ppt = cfg->pixels_per_thread; batch = cfg->batch; }
-    return dispatch(a.cam.tile, ppt, batch, a, as_stream(stream));
+    const int ppt = cfg ? cfg->pixels_per_thread
+                        : default_ppt(a.cam.tile, (int64_t)a.cam.tiles_x * a.cam.tiles_y, true);
+    return dispatch(a.cam.tile, ppt, a, as_stream(stream));
 }
 }  // namespace gs
 
@@ -1367,10 +1325,7 @@ static int batch_common(const gs_raster_job *jobs_dev, int32_t n_jobs, int32_t w
     cudaStream_t s = as_stream(stream);
     if (cudaMemsetAsync(queue_dev, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
     BatchArgs a{jobs_dev, width, height, (int)tiles, (int)(tiles * n_jobs), queue_dev, bwd};
-    int ppt, batch;
-    default_config(tile, tiles * n_jobs, bwd, ppt, batch);
-    if (cfg) { ppt = cfg->pixels_per_thread; batch = cfg->batch; }
-    return dispatch(tile, ppt, batch, a, s);
+    return dispatch(tile, cfg ? cfg->pixels_per_thread : default_ppt(tile, tiles * n_jobs, bwd), a, s);
 }
 
 extern "C" int gs_render_fwd_batch(const gs_raster_job *jobs_dev, int32_t n_jobs, int32_t width, int32_t height,
