@@ -771,6 +771,9 @@ __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats
         const int cnt = __popc(hits);
         if (hit) {
             const int q = kWholeTile ? lane : __popc(hits & ((1u << lane) - 1u));
+            // the opacity's gradient is a sum / opacity: for a splat too faint to be
+            // blended anywhere the sum is 0, and so may its opacity be
+            if (fabsf(rec.co.y) < 1e-3f) rec.co.y = 1e-3f;
             stage_splat(S, q, rec);
             gid[q] = g0 | (asleep ? 0x80000000u : 0u);
         }
