@@ -98,6 +98,14 @@ __device__ __forceinline__ SplatIn splat_in(const float *__restrict__ splats, ui
     return s;
 }
 
+// Whether every value of the record is finite (0 x is NaN where x is not).
+__device__ __forceinline__ bool all_finite(const SplatIn &s) {
+    const float p = fmaf(0.f, s.xa.z, fmaf(0.f, s.xa.y, 0.f * s.xa.x));
+    const float q = fmaf(0.f, s.co.y, fmaf(0.f, s.co.x, 0.f * s.xa.w));
+    const float r = fmaf(0.f, s.blue, fmaf(0.f, s.co.w, 0.f * s.co.z));
+    return p + q + r == 0.f;
+}
+
 template <class V>
 __device__ __forceinline__ void stage_splat(Stage<V> &S, int q, const SplatIn &s) {
     S.a[q] = V4<V>{v_dup<V>(s.xa.x), v_dup<V>(s.xa.y), v_dup<V>(__fmul_rn(-0.5f, s.xa.z)), v_dup<V>(-s.xa.w)};
@@ -677,9 +685,10 @@ __device__ __noinline__ void scalar_steps(PixBwd *p, const Stage<V> &S, const ui
 // A frozen splat only moves T and G, a uniform branch.
 //
 // In the packed steps a pixel that does not use a splat contributes terms
-// multiplied by alpha = 0, which is nothing only while they are finite: a
-// block whose pixel state is not finite, or 32 splats with a colour or
-// opacity that is not, go through the scalar steps (pix_bwd), which skip.
+// multiplied by alpha = 0, which is nothing only while they are finite, and a
+// splat that no pixel uses is summed with one that is used: a block whose pixel
+// state is not finite, or 32 splats with a record that is not, go through the
+// scalar steps (pix_bwd), which skip.
 //
 // Measured against the kernel before it (a barrier-separated batch per CTA,
 // scalar steps with divisions, one splat's sums at a time into a shared
@@ -766,8 +775,7 @@ __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats
         if (!kWholeTile && valid)
             hit = block_hit(rec, (float)bx, (float)(bx + 7), (float)by, (float)(by + kH - 1));
         const unsigned hits = __ballot_sync(kFull, hit);
-        const bool odd = hit && !(isfinite(rec.co.y) && isfinite(rec.co.z) && isfinite(rec.co.w) && isfinite(rec.blue));
-        const bool packed = finite && !__any_sync(kFull, odd);
+        const bool packed = finite && !__any_sync(kFull, hit && !all_finite(rec));
         const int cnt = __popc(hits);
         if (hit) {
             const int q = kWholeTile ? lane : __popc(hits & ((1u << lane) - 1u));
