@@ -314,7 +314,8 @@ typedef struct {
 /* gs_project_bwd (accumulate = 0) or gs_project_bwd_accum (accumulate != 0)
  * that updates n_sets (0..2) statistics windows at once -- the freeze window
  * of Sec. 3.2.1 and the densification window of Sec. 4.1 have different
- * lengths. sets: host array of n_sets. Errors: INVALID_ARG, CUDA. */
+ * lengths. sets: host array of n_sets; an array may stand in more than one
+ * place, every addition to it counts. Errors: INVALID_ARG, CUDA. */
 int gs_project_bwd_stats(const float *P, int64_t n, int32_t sh_degree, const gs_camera *cam, const float *splats,
                          const int32_t *act, const int32_t *n_active_dev, float *grad2d, float *G, int32_t accumulate,
                          const gs_grad_stats *sets, int32_t n_sets, gs_stream_t stream);

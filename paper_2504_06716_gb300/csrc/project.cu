@@ -247,6 +247,7 @@ struct StatSets {
     float *ax[2], *ar[2];
     int32_t *cnt[2], *maxr[2];
     int n;
+    bool shared;  // some array stands in two places: each addition sees the one before it
 };
 
 // Backward of the projection for act[0 .. *n_active). See gs_project_bwd;
@@ -499,6 +500,13 @@ __global__ void __launch_bounds__(32 * kBwdWarps, 4)
 #pragma unroll
             for (int w = 0; w < 2; ++w) {
                 if (w >= st.n) break;
+                if (st.shared) {
+                    st.ax[w][i] += nrm.x;
+                    st.ar[w][i] += nrm.y;
+                    st.cnt[w][i] += 1;
+                    if (st.maxr[w] && radius > st.maxr[w][i]) st.maxr[w][i] = radius;
+                    continue;
+                }
                 st.ax[w][i] = ax[w] + nrm.x;
                 st.ar[w][i] = ar[w] + nrm.y;
                 st.cnt[w][i] = cnt[w] + 1;
@@ -573,6 +581,14 @@ static int project_bwd(bool acc, const float *P, int64_t n, int32_t sh_degree, i
         st.cnt[k] = sets[k].cnt;
         st.maxr[k] = sets[k].max_radius;
     }
+    const void *arrays[8];
+    int n_arrays = 0;
+    for (int k = 0; k < n_sets; ++k)
+        for (const void *a : {(const void *)st.ax[k], (const void *)st.ar[k], (const void *)st.cnt[k],
+                              (const void *)st.maxr[k]}) {
+            for (int j = 0; a && j < n_arrays; ++j) st.shared = st.shared || arrays[j] == a;
+            if (a) arrays[n_arrays++] = a;
+        }
     const DevCam dc = make_cam(cam);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
