@@ -235,9 +235,10 @@ int gs_raster_bwd_resume(const float *splats, const uint32_t *vals, const uint32
 
 /* Sec. 3.1 and Sec. 3.2.4: gs_render_fwd_resume and gs_raster_bwd_resume (same results) with the tiles taken
  * longest list first, in the order that gs_sort left in its workspace for
- * these lists: sort_ws of sort_ws_bytes, unchanged since that call. A NULL, too
- * small or unaligned workspace, or one whose last sort was for another grid, means
- * ascending tiles. */
+ * these lists: sort_ws of sort_ws_bytes, written by nothing else since that call.
+ * A NULL, too small or unaligned workspace, or one whose last sort was for another
+ * grid or made no order (under 456 tiles, n or capacity 0), means ascending
+ * tiles. */
 int gs_render_fwd_sorted(const float *splats, const uint32_t *vals, const uint32_t *ranges, const gs_camera *cam,
                          const gs_raster_config *cfg, const uint8_t *frozen, float *image, float *t_final,
                          int32_t *n_last, float *resume, int32_t *resume_pos, const void *sort_ws,

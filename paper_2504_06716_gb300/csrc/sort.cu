@@ -166,7 +166,8 @@ struct ZeroSpans {
 // among them (part [3][kVisGrid]).
 __global__ void __launch_bounds__(kVisBlock) k_count_visible(const float *__restrict__ splats, int64_t n,
                                                             uint32_t *__restrict__ part, ZeroSpans z,
-                                                            unsigned long long *__restrict__ total_exact) {
+                                                            unsigned long long *__restrict__ total_exact,
+                                                            uint2 *__restrict__ stamp) {
     __shared__ uint32_t s_c[kVisBlock / 32], s_lo[kVisBlock / 32], s_hi[kVisBlock / 32];
     wait_prior_grid();
     const int64_t range = vis_range(n), lo = (int64_t)blockIdx.x * range, hi = lo + range < n ? lo + range : n;
@@ -174,7 +175,10 @@ __global__ void __launch_bounds__(kVisBlock) k_count_visible(const float *__rest
 #pragma unroll
     for (int k = 0; k < 3; ++k)
         for (int64_t i = t; i < z.n[k]; i += all) z.p[k][i] = 0u;
-    if (t == 0) *total_exact = 0ull;
+    if (t == 0) {
+        *total_exact = 0ull;
+        *stamp = make_uint2(0u, 0u);  // an earlier sort's tile order is good no more; order_tiles marks this one's
+    }
     uint32_t c = 0u, kl = 0xffffffffu, kh = 0u;
 #pragma unroll 4
     for (int64_t i = lo + threadIdx.x; i < hi; i += kVisBlock) {
@@ -1565,7 +1569,9 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
         k_zero_u32<<<grid_for(2 * tiles, 256), 256, 0, s>>>(ranges, 2 * tiles);
         note_launches(1);
         if (n == 0) {
-            cudaMemsetAsync(count_dev, 0, sizeof(int64_t), s);
+            if (!accepted(cudaMemsetAsync(count_dev, 0, sizeof(int64_t), s)) ||
+                !accepted(cudaMemsetAsync(w.front.stamp, 0, sizeof(uint2), s)))  // no order either
+                return GS_ERR_CUDA;
             return launch_status();
         }
     }
@@ -1580,7 +1586,8 @@ extern "C" int gs_sort(const float *splats, int64_t n, const gs_camera *cam, voi
                        capacity ? npass * kMaxRadix * chunk_rows(capacity) : 0}};
     const unsigned vgrid = vis_blocks(n), egrid = entry_blocks(n);
     const size_t hstride = (size_t)chunk_rows(n) * kMaxRadix;
-    if (!accepted(launch_chained(k_count_visible, vgrid, kVisBlock, s, splats, n, w.part32, z, w.total_exact)))
+    if (!accepted(launch_chained(k_count_visible, vgrid, kVisBlock, s, splats, n, w.part32, z, w.total_exact,
+                                 w.front.stamp)))
         return GS_ERR_CUDA;
     if (!accepted(launch_chained(k_emit_visible, vgrid, kVisBlock, s, splats, n, w.part32, dc, w.kv[0], w.kv[1],
                                  w.cull, w.n_vis, w.span, w.hist_d, hstride)))
