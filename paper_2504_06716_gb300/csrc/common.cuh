@@ -203,6 +203,10 @@ __device__ __forceinline__ float rcp_ftz(float x) {
 
 constexpr float kLog2e = 1.44269504088896341f;  // exp(x) = 2^(x log2 e)
 
+// exp(power), the one formula of every kernel that decides whether a splat is
+// blended (the rasteriser's packed steps take the product for two pixels at once).
+__device__ __forceinline__ float splat_falloff(float power) { return ex2_ftz(__fmul_rn(power, kLog2e)); }
+
 template <int N>
 struct IntC {  // a compile-time integer passed as an argument
     static constexpr int value = N;

@@ -580,7 +580,7 @@ struct PixBwd {
 __device__ __forceinline__ bool pix_bwd(PixBwd &p, bool frz, const SplatRow &row, float dy, const float4 &co,
                                         float blue, float (&g)[9]) {
     const float power = splat_power(row, dy);
-    const float G = ex2_ftz(__fmul_rn(power, kLog2e));
+    const float G = splat_falloff(power);
     const float oG = __fmul_rn(co.y, G);
     const float alpha = fminf(kAlphaMax, oG);
     if (!(power <= 0.f && alpha >= kAlphaMin)) return false;
@@ -963,6 +963,15 @@ __global__ void __launch_bounds__(TS * TS / PPT, bwd_blocks<TS, PPT>())
 }
 
 // ---- measurement support: the (pixel, splat) pairs the backward visits ----
+// Whether splat g is blended at a pixel that is still alive: the rasteriser's decision.
+__device__ __forceinline__ bool pair_blended(const float *__restrict__ splats, uint32_t g, float fpx, float fpy) {
+    const float4 *r = reinterpret_cast<const float4 *>(splats + (int64_t)g * kSplat);
+    const float4 xa = __ldg(r), co = __ldg(r + 1);
+    const float power = splat_power(splat_row(__fsub_rn(xa.x, fpx), xa.z, xa.w, co.x), __fsub_rn(xa.y, fpy));
+    const float alpha = fminf(kAlphaMax, __fmul_rn(co.y, splat_falloff(power)));
+    return power <= 0.f && alpha >= kAlphaMin;
+}
+
 // Per Gaussian, the pixels of this view it is blended into (the "hits" of
 // significance pruning, Sec. 3.3): one CTA per tile, one thread per pixel,
 // all threads at the same list position at once, one atomic per warp and
@@ -986,15 +995,7 @@ __global__ void k_hit_counts(const float *__restrict__ splats, const uint32_t *_
     const int lane = threadIdx.x & 31;
     for (int j = 0; j < jmax; ++j) {
         const uint32_t g = vals[start + j];
-        bool hit = false;
-        if (j < nl) {
-            const float4 *r = reinterpret_cast<const float4 *>(splats + (int64_t)g * kSplat);
-            const float4 xa = __ldg(r), co = __ldg(r + 1);
-            const float power = splat_power(splat_row(__fsub_rn(xa.x, fpx), xa.z, xa.w, co.x), __fsub_rn(xa.y, fpy));
-            const float alpha = fminf(kAlphaMax, __fmul_rn(co.y, __expf(power)));
-            hit = power <= 0.f && alpha >= kAlphaMin;
-        }
-        const unsigned b = __ballot_sync(kFull, hit);
+        const unsigned b = __ballot_sync(kFull, j < nl && pair_blended(splats, g, fpx, fpy));
         if (lane == 0 && b) atomicAdd(hits + g, (uint32_t)__popc(b));
     }
 }
@@ -1003,16 +1004,8 @@ __global__ void k_hit_counts(const float *__restrict__ splats, const uint32_t *_
 // forward's own decisions up to where the resuming backward walks it: the
 // pixel's last contributor, or with a freeze map 1 + the tile's last unfrozen
 // entry among those the tile's deepest contributor reaches, if that is less
-// (a lower bound of the backward's walk, which may go on to the deepest
-// contributor when an unfrozen entry lies further on in the list).
-__device__ __forceinline__ bool pair_blended(const float *__restrict__ splats, uint32_t g, float fpx, float fpy) {
-    const float4 *r = reinterpret_cast<const float4 *>(splats + (int64_t)g * kSplat);
-    const float4 xa = __ldg(r), co = __ldg(r + 1);
-    const float power = splat_power(splat_row(__fsub_rn(xa.x, fpx), xa.z, xa.w, co.x), __fsub_rn(xa.y, fpy));
-    const float alpha = fminf(kAlphaMax, __fmul_rn(co.y, __expf(power)));
-    return power <= 0.f && alpha >= kAlphaMin;
-}
-
+// (a lower bound of the backward's walk, which goes on to the deepest
+// contributor when an unfrozen entry lies behind it among the same 32 entries).
 __global__ void k_pair_counts(const float *__restrict__ splats, const uint32_t *__restrict__ vals,
                               const uint32_t *__restrict__ ranges, DevCam cam, const int32_t *__restrict__ n_last,
                               const uint8_t *__restrict__ frozen, unsigned long long *__restrict__ counts) {
