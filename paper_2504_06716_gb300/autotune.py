@@ -1,10 +1,10 @@
 """Autotuner for the rasteriser launch shape.
 
 Times, on the caller's own model and views, every tile size (8, 16, 32) with
-every pixels-per-thread (1, 2, 4 where a tile fills whole warps) and batch size (32, 64, 128, 256) of the two
+every pixels-per-thread (1, 2, 4 where a tile fills whole warps) of the two
 rasteriser kernels, and picks the tile size whose projection + sort + best
-forward + best backward is fastest. Every shape computes the same image; the
-forward's batch is the grain of the resume record (see pick).
+forward + best backward is fastest. Every shape computes the same image and
+resume record; a shape's batch changes nothing and is not timed.
 """
 from __future__ import annotations
 
@@ -47,14 +47,22 @@ def retile(cam: lib.GsCamera, tile: int) -> lib.GsCamera:
     return c
 
 
+def time_shapes(run, ppts, batches, reps: int) -> dict:
+    """Milliseconds of run(cfg) by (pixels per thread, batch). No kernel depends
+    on the batch, so that each pixels-per-thread is timed once for all of them."""
+    times = {}
+    for ppt in ppts:
+        cfg = lib.raster_config(ppt, batches[0])
+        t = _time(lambda: run(cfg), reps)
+        times.update({(ppt, b): t for b in batches})
+    return times
+
+
 def pick(times: dict) -> tuple[int, int]:
     """The (pixels per thread, batch) to take: of the shapes within 5% of the
-    fastest the smallest batch, then the fastest. The batch is not a staging
-    size any more, so shapes that differ in it alone take the same time but for
-    noise; in the forward it is the grain of the resume record, which may leave
-    out gradients of up to a batch of entries in front of where a tile's walk
-    stops (a schedule of 1000 iterations on the 1M-Gaussian scene: 39.96 dB held
-    out with batches of 32, 39.6 and 33.1 dB with larger ones taken by noise)."""
+    fastest the smallest batch, then the fastest. Of time_shapes' times, where
+    the batches of a pixels-per-thread are equal, that is the fastest
+    pixels-per-thread with the smallest batch."""
     best = min(times.values())
     return min((k for k, t in times.items() if t <= 1.05 * best), key=lambda k: (k[1], times[k]))
 
@@ -77,17 +85,11 @@ def tune(model, cams, targets, tiles=(8, 16, 32), ppts=(1, 2, 4), batches=(32, 6
             t_ps += _time(lambda: (lib.gs_project(model.P, model.n, model.sh_degree, v.cam, model.splats),
                                    lib.gs_sort(model.splats, model.n, v.cam, v.sort_ws, v.capacity, v.vals, v.ranges,
                                                v.count)), reps)
-            for ppt in ppts:
-                for b in batches:
-                    cfg = lib.raster_config(ppt, b)
-                    fwd_times[(ppt, b)] = fwd_times.get((ppt, b), 0.0) + _time(
-                        lambda: model.render_fwd(v, cfg), reps)
+            for k, t in time_shapes(lambda cfg: model.render_fwd(v, cfg), ppts, batches, reps).items():
+                fwd_times[k] = fwd_times.get(k, 0.0) + t
             model.loss(v, gt)
-            for ppt in ppts:
-                for b in batches:
-                    cfg = lib.raster_config(ppt, b)
-                    bwd_times[(ppt, b)] = bwd_times.get((ppt, b), 0.0) + _time(
-                        lambda: model.raster_bwd(v, cfg), reps)
+            for k, t in time_shapes(lambda cfg: model.raster_bwd(v, cfg), ppts, batches, reps).items():
+                bwd_times[k] = bwd_times.get(k, 0.0) + t
         model.grad2d.zero_()
         bf, bb = pick(fwd_times), pick(bwd_times)
         total = t_ps + fwd_times[bf] + bwd_times[bb]

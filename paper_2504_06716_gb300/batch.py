@@ -44,7 +44,7 @@ import numpy as np
 import torch
 
 from . import lib, pipeline, synth
-from .autotune import retile
+from .autotune import _time, pick, retile, time_shapes
 from .schedule import FREEZE_RESET, FREEZE_UPDATE, GStaConfig, GStaController, calibrate_eps0
 
 SIZES = (50_000, 120_000, 250_000, 400_000, 600_000, 900_000, 1_400_000, 2_000_000)
@@ -383,22 +383,10 @@ class BatchTrainer:
 
 
 # ---- autotuner for the batched launches ----
-def _time(fn, reps: int) -> float:
-    fn()
-    torch.cuda.synchronize()
-    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    e0.record()
-    for _ in range(reps):
-        fn()
-    e1.record()
-    torch.cuda.synchronize()
-    return e0.elapsed_time(e1) / reps
-
-
 def tune(bt: BatchTrainer, tiles=(8, 16, 32), ppts=(1, 2, 4), batches=(32, 64, 128, 256), reps: int = 3) -> dict:
-    """Pick the tile size (8/16/32) and the (pixels per thread, splats per
-    shared-memory batch) of the two persistent launches by timing them on the
-    trainer's own scenes, for view group 0. Tile size moves work between the
+    """Pick the tile size (8/16/32) and the pixels per thread of the two persistent
+    launches by timing them on the trainer's own scenes, for view group 0 (their
+    batch changes nothing: the smallest is taken). Tile size moves work between the
     sort and the rasteriser, so the choice minimises projection + sort + best
     forward + best backward. Runs real training steps (one per tile)."""
     table, best = {}, None
@@ -410,19 +398,12 @@ def tune(bt: BatchTrainer, tiles=(8, 16, 32), ppts=(1, 2, 4), batches=(32, 64, 1
         tbl, n_jobs = bt.job_tables[0]
         H, W = bt.active[0].cams[0].height, bt.active[0].cams[0].width
         t_front = _time(lambda: bt.per_view(lambda s, i: s.enqueue_front(0, i)), reps)
-        fwd_t, bwd_t = {}, {}
-        for ppt in ppts:
-            for b in batches:
-                c = lib.raster_config(ppt, b)
-                fwd_t[(ppt, b)] = _time(lambda: lib.gs_render_fwd_batch(tbl, n_jobs, W, H, tile, c, bt.queue), reps)
-        for ppt in ppts:
-            for b in batches:
-                c = lib.raster_config(ppt, b)
-                bwd_t[(ppt, b)] = _time(lambda: lib.gs_raster_bwd_batch(tbl, n_jobs, W, H, tile, c, bt.queue), reps)
+        fwd_t = time_shapes(lambda c: lib.gs_render_fwd_batch(tbl, n_jobs, W, H, tile, c, bt.queue), ppts, batches, reps)
+        bwd_t = time_shapes(lambda c: lib.gs_raster_bwd_batch(tbl, n_jobs, W, H, tile, c, bt.queue), ppts, batches, reps)
         for s in bt.active:
             for slot in s.slots:
                 slot.grad2d.zero_()
-        bf, bb = min(fwd_t, key=fwd_t.get), min(bwd_t, key=bwd_t.get)
+        bf, bb = pick(fwd_t), pick(bwd_t)
         total = t_front + fwd_t[bf] + bwd_t[bb]
         table[tile] = dict(project_sort_ms=t_front, fwd_ms={f"{p}x{b}": t for (p, b), t in fwd_t.items()},
                            bwd_ms={f"{p}x{b}": t for (p, b), t in bwd_t.items()}, best_fwd=bf, best_bwd=bb,
