@@ -188,7 +188,10 @@ def _stream(stream=None):
     if stream is not None:
         return stream.cuda_stream
     if torch.cuda.is_initialized():
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:  # private names: a PyTorch without them builds the object
+            pass
     return torch.cuda.current_stream().cuda_stream
 
 
