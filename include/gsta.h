@@ -167,8 +167,8 @@ int gs_render_fwd(const float *splats, const uint32_t *vals, const uint32_t *ran
  * camera's tile size. */
 typedef struct {
     int32_t pixels_per_thread; /* pixels each thread composites: 1, 2, or 4 (tiles of 16 and 32) */
-    int32_t batch;             /* 32, 64, 128 or 256; no kernel stages by it any more, so neither results
-                                * nor times depend on it */
+    int32_t batch;             /* 32, 64, 128 or 256: no kernel reads it, neither results nor times
+                                * depend on it */
 } gs_raster_config;
 
 /* Sec. 3.1, Eq. 2: gs_render_fwd with an explicit launch shape (cfg may be

@@ -251,9 +251,9 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_sums, int *
 // the rasteriser's time). The sort leaves the order by list length at the front of
 // its workspace, marked with the grid it is for; a training step's backward
 // takes them by the depth that the forward's walk reached. 1M Gaussians, 1237 x
-// 822, 8-pixel tiles: forward 140 -> 128 us, backward 323 -> 262 (nothing frozen)
-// and 156 -> 123 us (95% frozen); by list length 290 and 132. 120K at 800 x 800,
-// 16-pixel tiles: 46 -> 39 and 83 -> 75 us.
+// 822, 8-pixel tiles: forward 136 -> 123 us, backward 355 -> 296 (nothing frozen)
+// and 167 -> 137 us (95% frozen); by list length 320 and 144. 120K at 800 x 800,
+// 16-pixel tiles, half frozen: 44 -> 37 and 82 -> 75 us.
 struct TileOrder {
     const uint32_t *order;  // [tiles]; NULL: ascending tiles
     const uint2 *stamp;     // read and compared with key where the caller vouches for nothing; NULL: order is good

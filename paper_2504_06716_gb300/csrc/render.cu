@@ -169,7 +169,8 @@ __device__ __forceinline__ void alphas(V px, V py, const V4<V> &a, const V4<V> &
 //
 // What a step does per pixel: two compares decide whether the splat blends,
 // a select zeroes alpha if not, and from there on nothing is conditional (an
-// alpha of 0 leaves T and the colour as they are, bit for bit). A pixel that
+// alpha of 0 leaves T and, the splat's colour being finite, the colour as they
+// are, bit for bit). A pixel that
 // has stopped gets a NaN row coordinate, so that every later exponent is NaN
 // and fails its compare: no done flag is tested. G splats are evaluated
 // together -- their alphas do not depend on one another, only T runs through
@@ -190,10 +191,12 @@ __device__ __forceinline__ void alphas(V px, V py, const V4<V> &a, const V4<V> &
 //
 // Measured against the kernel before it (a barrier-separated batch per CTA,
 // done flags and a stop test per splat, every warp through the whole tile's
-// list): 1M Gaussians, 1237x822, 8-pixel tiles, two pixels per thread with the
-// record 202 -> 140 us; 3M at 1920x1080, 16-pixel tiles 633 -> 327 us; 400K
-// at 800x800, 16-pixel tiles with the record 240 -> 103 us; 2K at 128x128
-// 31 -> 15 us; the same bits in every output.
+// list), tiles ascending: 1M Gaussians, 1237x822, 8-pixel tiles, two pixels per
+// thread with the record 199 -> 136 us; 3M at 1920x1080, 16-pixel tiles, one
+// pixel per thread 671 -> 325 us; 400K at 800x800, 16-pixel tiles, one pixel, with
+// the record 262 -> 98 us; 2K at 128x128 33 -> 12.5 us; the same bits in image, T
+// and last contributor. (With a record kept per batch of the list 140, 103 and
+// 14 us.)
 template <int TS, int PPT, bool RES>
 __device__ __forceinline__ void render_tile(const float *__restrict__ splats, const uint32_t *__restrict__ vals,
                                             const uint32_t *__restrict__ ranges, const DevCam &cam,
@@ -469,12 +472,12 @@ __device__ __forceinline__ void render_tile(const float *__restrict__ splats, co
     }
 }
 
-// Blocks to keep resident per SM: with one pixel per thread 32 warps (24 when
-// the resume record is kept, whose state would spill), which cost registers
-// the step can spare (3M Gaussians at 1920x1080, 16-pixel tiles: 327 us
-// against 355 without; 400K at 800x800 with the record 103 against 119); with
-// two or four the G splats in flight need them (140 us against 144 at 1M,
-// 1237x822).
+// Blocks to keep resident per SM: with one pixel per thread 32 warps, which cost
+// registers the step can spare (3M Gaussians at 1920x1080, 16-pixel tiles: 325 us
+// against 358 without); 24 when the resume record is kept, whose state would
+// spill (400K at 800x800: 97.5 us against 96.7 without, so it holds the kernel at
+// what it takes anyway); with two or four the G splats in flight need them (136 us
+// at 1M, 1237x822, at 103 registers).
 template <int TS, int PPT, bool RES>
 constexpr int fwd_blocks() {
     constexpr int warps = PPT == 1 ? (RES ? 24 : 32) : 1, per = TS * TS / PPT / 32;
@@ -692,10 +695,11 @@ __device__ __noinline__ void scalar_steps(PixBwd *p, const Stage<V> &S, const ui
 //
 // Measured against the kernel before it (a barrier-separated batch per CTA,
 // scalar steps with divisions, one splat's sums at a time into a shared
-// accumulator by atomics): 1M Gaussians, 1237x822, 8-pixel tiles, two pixels
-// per thread, nothing frozen 492 -> 324 us (348 with nine sums over all lanes),
-// 95% frozen 220 -> 156 us (one pixel per thread 208 -> 138 us); 400K at 800x800,
-// 16-pixel tiles, half frozen 445 -> 168 us; 2K at 128x128 114 -> 28 us.
+// accumulator by atomics), the whole list walked and the tiles ascending: 1M
+// Gaussians, 1237x822, 8-pixel tiles, two pixels per thread, nothing frozen 521 ->
+// 350 us (7% more with nine sums over all lanes), 95% frozen 227 -> 168 us (one
+// pixel per thread 220 -> 150 us); 400K at 800x800, 16-pixel tiles, half frozen
+// 469 -> 174 us (one pixel 431 -> 176); 2K at 128x128, one pixel 77 -> 28 us.
 template <int TS, int PPT>
 __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats, const uint32_t *__restrict__ vals,
                                                 const uint32_t *__restrict__ ranges, const DevCam &cam,
@@ -941,10 +945,11 @@ __device__ __forceinline__ void raster_bwd_tile(const float *__restrict__ splats
     if (waiting) give(sum_one(pend, pend_s, fpx, lane), pend_g, pend_o, slot >= 0 && lane < 16);
 }
 
-// Warps to keep resident per SM: 24 with one pixel per thread (78 registers), 16
-// with two (1M Gaussians, 1237x822, nothing frozen, with nine sums over all lanes:
-// 349 us against 362 without the bound, at 132 registers and 12 warps, and 361 at
-// 20 warps; 324 us now at 111 registers and 18 warps).
+// Warps to keep resident per SM: 24 with one pixel per thread (78 registers: 147
+// us against 174 without the bound at 1M, 95% frozen, 177 against 199 at 400K, 79
+// against 87 at 120K; few tiles would rather have the registers, 100K at 512x512 95
+// against 89), 16 with two, which the kernel takes anyway (355 us against 353 at
+// 1M, nothing frozen, at 111 registers and 18 warps).
 template <int TS, int PPT>
 constexpr int bwd_blocks() {
     constexpr int warps = PPT == 1 ? 24 : PPT == 2 ? 16 : 1, per = TS * TS / PPT / 32;
@@ -1102,11 +1107,13 @@ __global__ void __launch_bounds__(TS * TS / PPT) k_raster_bwd_batch(const gs_ras
 // (timed on GB300; the autotuner may pick another per workload). The backward
 // of 16-pixel tiles takes one pixel per thread while the tiles are few: below
 // about 2048 the chip has fewer 8 x 8 blocks than warps it can hold, and halving
-// the blocks shortens every chain (100K Gaussians at 512x512, 1024 tiles: 67 us
-// against 76; 50K at 320x240 47 against 55); above, two per thread cost fewer
-// instructions (surface scenes, 120K at 800x800 74 us against 87, 400K 195
-// against 219, 200K at 1237x822 160 against 196; where a few tiles are far longer
-// than the rest one is better even there: 400K, half frozen, 148 against 154).
+// the blocks shortens every chain (100K Gaussians at 512x512, 1024 tiles: 95 us
+// against 112; 50K at 320x240 75 against 93); above, two per thread cost fewer
+// instructions (tiles ascending, nothing frozen: 120K at 800x800, 2500 tiles 102 us
+// against 104, 400K 223 against 236, 200K at 1237x822, 4056 tiles 167 against 200).
+// Longest first, as a training step takes them, the line lies higher: one pixel
+// is the better one at 2500 tiles (120K 85 against 97, 400K 205 against 211, half
+// frozen 154 against 168), two at 4056 (155 against 189).
 inline int default_ppt(int tile, int64_t tiles, bool bwd) {
     if (tile == 8) return 1;
     if (tile == 16) return bwd && tiles >= 2048 ? 2 : 1;
